@@ -1,0 +1,683 @@
+// FP32 implicit-GEMM convolution with the carry-through filter on the CUDA
+// cores (packed FFMA, no TF32), operands staged by TMA.
+//
+// GEMM view as in conv_simt.cu: m = output pixel, n = output channel,
+// k = (tap, channel).  A K block is 32 channels of one tap: a TMA im2col load
+// brings BM pixels x 32 channels (128-byte swizzled rows, zeros outside the
+// image and past the last channel), a tiled load BN filters x 32 channels.
+// Both tiles keep k innermost, as the tensors have it, so nothing is
+// transposed: a thread reads 4 consecutive k of one row per 16-byte access,
+// and the swizzle puts the rows a warp reads together into different banks.
+//
+// Every multiply-add is the packed fma.rn.f32x2 on (k, k + 1): one
+// accumulator pair per output holds the sums over even and odd k, added in
+// the epilogue.  Each half is an FP32 FMA like the scalar one.
+//
+// Persistent CTAs: four compute warps with 8 x 8 outputs per thread, and a
+// producer warp whose elected lane issues the copies ahead, across tile
+// boundaries, through a ring of stages.  The compute warps' fragments are
+// double-buffered in registers (two warps per scheduler hide little of the
+// shared-memory latency), which takes over 200 registers: the producer's
+// warpgroup gives its share up (setmaxnreg).
+//
+// What bounds it: the FMA pipe, busy 64% of the cycles (a probe of the same
+// inner step without barriers or copies reaches 72%, of register operands
+// alone 89%).  128 images of 32 x 32 x 64 channels through a 3 x 3 layer
+// (4.8 G multiply-adds): 268 us with conv_simt.cu's scalar kernel, 201 us
+// here; 16 x 16 x 128: 272 -> 201 us; 4 x 4 x 512: 327 -> 197 us (that one
+// with its split-K sum).  Of these, fragments in plain C++ loads and the
+// __ffma2_rn intrinsic instead of inline PTX took 233 -> 202 us (the operands
+// of asm blocks cost a register move for every second multiply-add).
+//
+// Work split: the K blocks of all tiles form one list, of which every CTA
+// takes an equal contiguous share, so a layer whose tiles do not fill the
+// last round still keeps every SM busy to the end.  A CTA runs its pieces
+// from the last to the first: a piece that stops short of its tile's end is
+// a partial sum, left in the workspace with a flag; the piece that reaches
+// the end adds the partials of the CTAs before it, in K order, and applies
+// the epilogue.  So a CTA waits only for CTAs of lower index, which started
+// earlier and wrote their partial before anything else.
+//
+// Carry-through filter (Sec. II-A): its output is the channel sum of the
+// centre-tap K blocks, which are in shared memory anyway; the warps of the
+// first channel tile add them there, the lanes that share a row each taking
+// other channels.  The incoming checksum plane enters only the checksum
+// output.  Epilogue on data and checksum alike: + bias (0 for the checksum),
+// + residual, ReLU, store.
+#include <cuda.h>
+#include <cudaTypedefs.h>
+#include <string.h>
+
+#include <algorithm>
+#include <utility>
+
+#include "ct_internal.h"
+#include "tc_common.cuh"
+
+namespace ct {
+namespace {
+
+using namespace tc;
+
+constexpr int F_BK = 32;               // channels per K block (128 bytes)
+constexpr int F_TM = 8, F_TN = 8;      // outputs per thread
+constexpr int F_WARPS = 4;             // compute warps
+constexpr int F_THREADS = 32 * F_WARPS;        // compute threads
+constexpr int F_CTA = 2 * F_THREADS;           // and the producer's warpgroup
+// registers per thread of the two warpgroups; together what the CTA is
+// launched with (256 threads at two CTAs per SM: 128 each)
+constexpr int F_REGS_COMPUTE = 232, F_REGS_PRODUCER = 24;
+static_assert(F_REGS_COMPUTE + F_REGS_PRODUCER == 2 * 128, "the split must not exceed the launch's registers");
+
+struct FGeom {
+    int M, PQ, Q, stride, pad, C, K, S, RS;
+    int cpb, n_kb, ctr_tap;            // K blocks per tap, in all; the centre tap
+    int n_tiles;                       // channel tiles
+    // CTA c runs K blocks [unit * (c * units / gridDim.x), unit * ((c + 1) * units / gridDim.x))
+    // of the list of all tiles' K blocks; unit = n_kb: whole tiles
+    int unit;
+    int units;
+    float *part;                       // [CTA][BM * BN + BM] partial sums
+    uint32_t *flags;                   // [CTA] 1: the CTA's partial is ready; 0 between launches
+};
+
+struct Quad {
+    float2 lo, hi;                     // k, k + 1 and k + 2, k + 3
+};
+// four floats of shared memory
+__device__ __forceinline__ Quad lds4(const uint8_t *p) {
+    const float4 v = *reinterpret_cast<const float4 *>(p);
+    return Quad{make_float2(v.x, v.y), make_float2(v.z, v.w)};
+}
+__device__ __forceinline__ void fma2(float2 &d, float2 a, float2 b) { d = __ffma2_rn(a, b, d); }
+// compile-time loop: f(std::integral_constant<int, 0>) .. <N - 1>
+template <typename F, int... I>
+__device__ __forceinline__ void static_for_(F &&f, std::integer_sequence<int, I...>) {
+    (f(std::integral_constant<int, I>()), ...);
+}
+template <int N, typename F>
+__device__ __forceinline__ void static_for(F &&f) {
+    static_for_(f, std::make_integer_sequence<int, N>());
+}
+__device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap *map, uint32_t bar, int x, int y, int z,
+                                            int w) {
+    asm volatile(
+        "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+        " [%0], [%1, {%2, %3, %4, %5}], [%6];" ::"r"(dst),
+        "l"((uint64_t)map), "r"(x), "r"(y), "r"(z), "r"(w), "r"(bar)
+        : "memory");
+}
+
+__device__ __forceinline__ void flag_set(uint32_t *p, uint32_t v) {
+    asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+// bounded wait for a flag of a CTA of lower index
+__device__ __forceinline__ bool flag_wait(const uint32_t *p, uint32_t *err, uint32_t code) {
+    const long long t0 = clock64();
+    for (;;) {
+        uint32_t v;
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+        if (v) return true;
+        if (clock64() - t0 > WAIT_CYCLES) {
+            atomicOr(err, code);
+            return false;
+        }
+    }
+}
+
+// mbar_wait of the producer, which is far ahead of the compute warps: it
+// sleeps between polls (polling took a fifth of the issue slots)
+__device__ __forceinline__ bool mbar_wait_idle(uint32_t bar, uint32_t parity, uint32_t *err, uint32_t code) {
+    if (mbar_try_wait(bar, parity)) return true;
+    const long long t0 = clock64();
+    for (;;) {
+        __nanosleep(256);
+        if (mbar_try_wait(bar, parity)) return true;
+        if (clock64() - t0 > WAIT_CYCLES) {
+            atomicOr(err, code);
+            return false;
+        }
+    }
+}
+
+// input value behind a fault delta at output pixel (n, p, q)
+__device__ __forceinline__ float f_fault_source(const ConvArgs &a, int n, int p, int q) {
+    const int h = p * a.stride + a.fd.r - a.pad, w = q * a.stride + a.fd.s - a.pad;
+    if (h < 0 || h >= a.H || w < 0 || w >= a.W) return 0.f;
+    const size_t pix = ((size_t)n * a.H + h) * a.W + w;
+    if (a.fd.cin < a.C) return static_cast<const float *>(a.x)[pix * a.C + a.fd.cin];
+    return a.cs_in ? static_cast<const float *>(a.cs_in)[pix] : 0.f;
+}
+
+// floats of one CTA's partial: its threads' outputs and checksum sums
+template <int KW>
+__host__ __device__ constexpr int f_partial() { return F_TM / KW * F_THREADS * (F_TN + 1); }
+
+// first K block of CTA c
+__device__ __forceinline__ int f_first(int c, const FGeom &g) {
+    return (int)((long long)c * g.units / gridDim.x) * g.unit;
+}
+
+// A warp's lanes are LM (rows) x LN = 32 / LM (columns).  Lane (lm, ln) owns
+// rows lm + LM * i of its warp's tile and the columns of rows ln + LN * j of
+// the staged B tile; the rows read together are consecutive, so the swizzle
+// spreads them over the banks.  The copies put filter 4 * LN * jh + 4 * ln +
+// jl of the warp's tile in B row ln + LN * (4 * jh + jl), so a lane's outputs
+// are groups of four consecutive channels (16-byte stores).
+// WM x WN warps share the tile's rows and columns; KW warps share the K
+// blocks' channels and add their sums through shared memory at the end
+// (small layers: less to add across CTAs per tile).
+template <int LM, int WM, int WN, int KW, int STAGES>
+__global__ void __launch_bounds__(F_CTA, 2)
+conv_ffma2_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ CUtensorMap bmap,
+                  const ConvArgs a, const FGeom g) {
+    constexpr int LN = 32 / LM;
+    constexpr int BM = LM * F_TM * WM, BN = LN * F_TN * WN;
+    constexpr int A_BYTES = BM * 128, B_BYTES = BN * 128, ST_BYTES = A_BYTES + B_BYTES;
+    constexpr int KC = F_BK / 4 / KW;              // 4-channel steps of a K block per warp
+    constexpr int NI = F_TM / KW;                  // rows per lane whose outputs a warp writes
+    static_assert(WM * WN * KW == F_WARPS, "four warps");
+    static_assert(KW == 1 || WM * WN == 1, "warps split K or the tile");
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    uint8_t *smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+    float *red = (float *)(smem + STAGES * ST_BYTES);            // [KW][F_TM * F_TN][32] (KW > 1)
+    // running centre-tap sums of each thread's rows: [F_TM][F_THREADS] (they
+    // are touched in centre-tap blocks only, and registers are short)
+    float *csum = red + (KW > 1 ? KW * F_TM * F_TN * 32 : 0);
+    uint64_t *full = (uint64_t *)(csum + F_TM * F_THREADS);
+    uint64_t *empty = full + STAGES;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < STAGES; ++s) {
+            mbar_init(smem_u32(&full[s]), 1);
+            mbar_init(smem_u32(&empty[s]), F_WARPS);
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __shared__ int abort_s;
+    if (threadIdx.x == 0) abort_s = 0;
+    __syncthreads();
+    pdl_wait();
+    pdl_trigger();
+    const uint32_t sbase = smem_u32(smem);
+    const int lo = f_first(blockIdx.x, g);
+    int end = f_first(blockIdx.x + 1, g);
+
+    if (warp >= F_WARPS) {
+        // ---------------- producer ----------------
+        // Copies in the order the blocks are consumed.  Block i goes to slot
+        // i % STAGES once every compute warp has arrived on its empty barrier.
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(F_REGS_PRODUCER));
+        if (warp > F_WARPS || lane != 0) return;
+        asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&amap) : "memory");
+        asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&bmap) : "memory");
+        int st = 0, issued = 0;
+        uint32_t ph = 1;                           // the first pass finds the slots free
+        bool ok = true;
+        while (end > lo && ok) {
+            const int t = (end - 1) / g.n_kb, t0 = t * g.n_kb;
+            const int m0 = t / g.n_tiles * BM, n0 = t % g.n_tiles * BN;
+            const int nimg = m0 / g.PQ, rem = m0 % g.PQ;
+            const int w0 = (rem % g.Q) * g.stride - g.pad, h0 = (rem / g.Q) * g.stride - g.pad;
+            const int kb = max(lo, t0) - t0;
+            int left = end - t0 - kb;
+            end = max(lo, t0);
+            int tap = kb / g.cpb, cb = kb - tap * g.cpb;
+            int r = tap / g.S, s = tap - r * g.S;
+            for (; left > 0; --left) {
+                if (!mbar_wait_idle(smem_u32(&empty[st]), ph, a.err, 1u)) { ok = false; break; }
+                const uint32_t fb = smem_u32(&full[st]), dst = sbase + st * ST_BYTES;
+                mbar_arrive_expect_tx(fb, ST_BYTES);
+                tma_load_im2col(dst, &amap, fb, cb * F_BK, w0, h0, nimg, (uint16_t)s, (uint16_t)r);
+#pragma unroll
+                for (int b = 0; b < 2 * WN; ++b)   // filters n0 + 4 * LN * b .. + 4 * LN - 1
+                    tma_load_4d(dst + A_BYTES + b * (4 * LN * 128), &bmap, fb, cb * F_BK, n0 / 4 + b * LN, 0, tap);
+                ++issued;
+                if (++st == STAGES) { st = 0; ph ^= 1u; }
+                if (++cb == g.cpb) {
+                    cb = 0;
+                    ++tap;
+                    if (++s == g.S) { s = 0; ++r; }
+                }
+            }
+        }
+        // a wait gave up: copies in flight land before the CTA exits
+        if (!ok)
+            for (int i = max(0, issued - STAGES); i < issued; ++i)
+                mbar_wait(smem_u32(&full[i % STAGES]), (uint32_t)(i / STAGES) & 1u, a.err, 2u);
+        return;
+    }
+
+    // ---------------- compute warps ----------------
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(F_REGS_COMPUTE));
+    auto csync = [] { asm volatile("bar.sync 1, %0;" ::"n"(F_THREADS) : "memory"); };
+    const int lm = lane / LN, ln = lane % LN;
+    const int wrow = KW > 1 ? 0 : (warp / WN) * LM * F_TM, wcol = KW > 1 ? 0 : (warp % WN) * LN * F_TN;
+    const int kc0 = KW > 1 ? warp * KC : 0;
+    // byte offsets of this lane's first row in the A and B tiles, and the
+    // swizzle phase of the row (row & 7, in 16-byte chunks); rows LM (LN)
+    // apart keep the phase when that is 8 and alternate by 4 when it is 4
+    const uint32_t arow = (uint32_t)(wrow + lm) * 128u, brow = (uint32_t)A_BYTES + (uint32_t)(wcol + ln) * 128u;
+    const uint32_t aph = (uint32_t)(lm & 7) * 16u, bph = (uint32_t)(ln & 7) * 16u;
+    const int ctr_lo = g.ctr_tap * g.cpb, ctr_hi = ctr_lo + g.cpb;
+    int st = 0;
+    uint32_t ph = 0;
+    while (end > lo) {
+        const int t = (end - 1) / g.n_kb, t0 = t * g.n_kb;
+        const int m0 = t / g.n_tiles * BM, n0 = t % g.n_tiles * BN;
+        const int kb_lo = max(lo, t0) - t0, kb_hi = end - t0;
+        end = max(lo, t0);
+        const bool do_cs = a.cs_out != nullptr && n0 == 0 && wcol == 0;
+        const bool sum_cs = do_cs && a.role == CT_ROLE_CT;
+        float2 acc[F_TM][F_TN];
+#pragma unroll
+        for (int i = 0; i < F_TM; ++i) {
+            if (sum_cs) csum[i * F_THREADS + threadIdx.x] = 0.f;
+#pragma unroll
+            for (int j = 0; j < F_TN; ++j) acc[i][j] = make_float2(0.f, 0.f);
+        }
+        // fragments of step kc are loaded while step kc - 1 is multiplied:
+        // the rows of A one by one, the columns of B a pair ahead
+        Quad av[2][F_TM], bv[2][2];
+        // multiply the fragments of buffer `cur`, whose B columns sit at bc,
+        // loading those of the next step (A rows at an, B columns at bn) into
+        // the other buffer
+        auto step = [&](auto cur_c, uint32_t bc, uint32_t an, uint32_t bn) {
+            constexpr int cur = decltype(cur_c)::value;
+            const uint32_t an2 = LM == 4 ? an ^ 64u : an, bc2 = LN == 4 ? bc ^ 64u : bc, bn2 = LN == 4 ? bn ^ 64u : bn;
+            static_for<F_TN / 2>([&](auto jc) {
+                constexpr int j = 2 * decltype(jc)::value, pb = (j / 2) & 1;
+                av[cur ^ 1][j] = lds4(smem + an + j * LM * 128);
+                av[cur ^ 1][j + 1] = lds4(smem + an2 + (j + 1) * LM * 128);
+                if constexpr (j + 2 < F_TN) {
+                    bv[pb ^ 1][0] = lds4(smem + bc + (j + 2) * LN * 128);
+                    bv[pb ^ 1][1] = lds4(smem + bc2 + (j + 3) * LN * 128);
+                } else {
+                    bv[pb ^ 1][0] = lds4(smem + bn);
+                    bv[pb ^ 1][1] = lds4(smem + bn2 + LN * 128);
+                }
+                // 2 x 2 blocks, each operand used twice in a row
+#pragma unroll
+                for (int i = 0; i < F_TM; i += 2) {
+                    fma2(acc[i][j], av[cur][i].lo, bv[pb][0].lo);
+                    fma2(acc[i][j + 1], av[cur][i].lo, bv[pb][1].lo);
+                    fma2(acc[i + 1][j + 1], av[cur][i + 1].lo, bv[pb][1].lo);
+                    fma2(acc[i + 1][j], av[cur][i + 1].lo, bv[pb][0].lo);
+                }
+#pragma unroll
+                for (int i = 0; i < F_TM; i += 2) {
+                    fma2(acc[i][j], av[cur][i].hi, bv[pb][0].hi);
+                    fma2(acc[i][j + 1], av[cur][i].hi, bv[pb][1].hi);
+                    fma2(acc[i + 1][j + 1], av[cur][i + 1].hi, bv[pb][1].hi);
+                    fma2(acc[i + 1][j], av[cur][i + 1].hi, bv[pb][0].hi);
+                }
+            });
+        };
+        const std::integral_constant<int, 0> c0_{};
+        const std::integral_constant<int, 1> c1_{};
+        const uint32_t kx0 = (uint32_t)kc0 * 16u;
+        bool ok = warp_wait(smem_u32(&full[st]), ph, a.err, 2u);
+        if (ok) {
+            const uint32_t sa = st * ST_BYTES;
+            const uint32_t an = sa + arow + (aph ^ kx0), bn = sa + brow + (bph ^ kx0);
+            static_for<F_TM>([&](auto ic) {
+                constexpr int i = decltype(ic)::value;
+                av[0][i] = lds4(smem + (LM == 4 && (i & 1) ? an ^ 64u : an) + i * LM * 128);
+            });
+            bv[0][0] = lds4(smem + bn);
+            bv[0][1] = lds4(smem + (LN == 4 ? bn ^ 64u : bn) + LN * 128);
+        }
+        for (int kb = kb_lo; kb < kb_hi && ok; ++kb) {
+            const uint32_t sa = st * ST_BYTES;
+            const int cur_st = st;
+            if (++st == STAGES) { st = 0; ph ^= 1u; }
+            uint32_t sn = sa;
+            const uint32_t sar = sa + arow, sbr = sa + brow;
+            uint32_t bc = sbr + (bph ^ kx0);
+#pragma unroll 1
+            for (int kk = 0; kk < KC; kk += 2) {
+                const uint32_t k1 = kx0 + (uint32_t)kk * 16u + 16u;
+                const uint32_t b1 = sbr + (bph ^ k1);
+                step(c0_, bc, sar + (aph ^ k1), b1);
+                uint32_t kn = k1 + 16u;
+                if (kk + 2 == KC) {
+                    kn = kx0;
+                    if (kb + 1 < kb_hi) {           // the next block's first step
+                        ok = warp_wait(smem_u32(&full[st]), ph, a.err, 2u);
+                        sn = st * ST_BYTES;
+                    }
+                }
+                bc = sn + brow + (bph ^ kn);
+                step(c1_, b1, sn + arow + (aph ^ kn), bc);
+            }
+            if (sum_cs && kb >= ctr_lo && kb < ctr_hi) {
+                // 4-channel steps c = ln, ln + LN, ... of this warp's K share
+#pragma unroll
+                for (int i = 0; i < F_TM; ++i)
+#pragma unroll
+                    for (int c = 0; c < (KC + LN - 1) / LN; ++c) {
+                        if (ln + c * LN >= KC) continue;
+                        const Quad v = lds4(smem + sa + arow + (uint32_t)(i * LM) * 128u +
+                                            (uint32_t)(((kc0 + ln + c * LN) ^ ((lm + i * LM) & 7)) * 16));
+                        const float2 p = v.lo, q = v.hi;
+                        csum[i * F_THREADS + threadIdx.x] += (p.x + p.y) + (q.x + q.y);
+                    }
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&empty[cur_st]));
+        }
+        if (!ok && lane == 0) abort_s = 1;
+        // outputs of this lane: rows i0 .. i0 + NI - 1
+        const int i0 = KW > 1 ? warp * NI : 0;
+        float v[NI][F_TN], cs[NI];
+        if (KW > 1) {
+#pragma unroll
+            for (int i = 0; i < F_TM; ++i)
+#pragma unroll
+                for (int j = 0; j < F_TN; ++j) {
+                    const float2 f = acc[i][j];
+                    red[((warp * F_TM + i) * F_TN + j) * 32 + lane] = f.x + f.y;
+                }
+            csync();
+#pragma unroll
+            for (int i = 0; i < NI; ++i) {
+#pragma unroll
+                for (int j = 0; j < F_TN; ++j) {
+                    float s = 0.f;
+#pragma unroll
+                    for (int w = 0; w < KW; ++w) s += red[((w * F_TM + i0 + i) * F_TN + j) * 32 + lane];
+                    v[i][j] = s;
+                }
+                cs[i] = 0.f;
+                if (sum_cs)
+#pragma unroll
+                    for (int w = 0; w < KW; ++w) cs[i] += csum[(i0 + i) * F_THREADS + 32 * w + lane];
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < NI; ++i) {
+#pragma unroll
+                for (int j = 0; j < F_TN; ++j) {
+                    const float2 f = acc[i][j];
+                    v[i][j] = f.x + f.y;
+                }
+                cs[i] = sum_cs ? csum[i * F_THREADS + threadIdx.x] : 0.f;
+            }
+            // pieces that exchange partials meet here, as the KW > 1 warps did above
+            if (kb_lo > 0 || kb_hi < g.n_kb) csync();
+        }
+        if (sum_cs) {                               // the lanes that share a row
+#pragma unroll
+            for (int i = 0; i < NI; ++i)
+#pragma unroll
+                for (int o = LN / 2; o > 0; o >>= 1) cs[i] += __shfl_xor_sync(0xffffffffu, cs[i], o);
+        }
+        constexpr int PV = NI * F_TN * F_THREADS, PSZ = f_partial<KW>();   // floats of a CTA's partial
+        if (kb_hi < g.n_kb) {
+            // partial sums of this tile, in this thread's order
+            float *pt = g.part + (size_t)blockIdx.x * PSZ;
+#pragma unroll
+            for (int i = 0; i < NI; ++i) {
+#pragma unroll
+                for (int j = 0; j < F_TN; j += 4)
+                    __stcg(reinterpret_cast<float4 *>(pt) + ((i * F_TN + j) / 4) * F_THREADS + threadIdx.x,
+                           make_float4(v[i][j], v[i][j + 1], v[i][j + 2], v[i][j + 3]));
+                if (sum_cs) __stcg(pt + PV + i * F_THREADS + threadIdx.x, cs[i]);
+            }
+            __threadfence();
+            csync();
+            if (threadIdx.x == 0 && !abort_s) flag_set(g.flags + blockIdx.x, 1u);
+            if (abort_s) return;
+            continue;
+        }
+        if (kb_lo > 0) {
+            // the tile's earlier K blocks: partials of the CTAs before this one
+            int c0 = (int)blockIdx.x - 1;
+            while (f_first(c0, g) > t0) --c0;
+            for (int c = c0 + (int)threadIdx.x; c < (int)blockIdx.x; c += F_THREADS)
+                if (!flag_wait(g.flags + c, a.err, 2u)) abort_s = 1;
+            csync();
+            if (abort_s) return;
+            float u[NI][F_TN], uc[NI];
+#pragma unroll
+            for (int i = 0; i < NI; ++i) {
+                uc[i] = 0.f;
+#pragma unroll
+                for (int j = 0; j < F_TN; ++j) u[i][j] = 0.f;
+            }
+#pragma unroll (KW > 1 ? 4 : 1)
+            for (int c = c0; c < (int)blockIdx.x; ++c) {
+                const float *pt = g.part + (size_t)c * PSZ;
+#pragma unroll
+                for (int i = 0; i < NI; ++i) {
+#pragma unroll
+                    for (int j = 0; j < F_TN; j += 4) {
+                        const float4 f = __ldcg(reinterpret_cast<const float4 *>(pt) +
+                                                ((i * F_TN + j) / 4) * F_THREADS + threadIdx.x);
+                        u[i][j] += f.x; u[i][j + 1] += f.y; u[i][j + 2] += f.z; u[i][j + 3] += f.w;
+                    }
+                    if (sum_cs) uc[i] += __ldcg(pt + PV + i * F_THREADS + threadIdx.x);
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < NI; ++i) {
+                cs[i] = uc[i] + cs[i];
+#pragma unroll
+                for (int j = 0; j < F_TN; ++j) v[i][j] = u[i][j] + v[i][j];
+            }
+            csync();
+            for (int c = c0 + (int)threadIdx.x; c < (int)blockIdx.x; c += F_THREADS)
+                flag_set(g.flags + c, 0u);         // for the next launch
+        }
+        if (abort_s) return;
+        // ---- epilogue ----
+        const float *res = static_cast<const float *>(a.res);
+        float *y = static_cast<float *>(a.y);
+        const FaultDelta fd = a.fd;
+        const int nb = n0 + wcol + 4 * ln;          // channels nb .. nb + 3 and nb + 4 LN .. + 3
+        float4 bias[F_TN / 4];
+#pragma unroll
+        for (int h = 0; h < F_TN / 4; ++h)
+            bias[h] = nb + 4 * LN * h < g.K ? __ldg(reinterpret_cast<const float4 *>(a.bias + nb + 4 * LN * h))
+                                            : make_float4(0.f, 0.f, 0.f, 0.f);
+        constexpr int RB = NI < 4 ? NI : 4;         // rows whose residual loads are in flight together
+#pragma unroll
+        for (int ib = 0; ib < NI; ib += RB) {
+            float4 rv[RB][F_TN / 4];
+#pragma unroll
+            for (int i = 0; i < RB; ++i) {
+                const int m = m0 + wrow + lm + (i0 + ib + i) * LM;
+#pragma unroll
+                for (int h = 0; h < F_TN / 4; ++h)
+                    rv[i][h] = (res && m < g.M && nb + 4 * LN * h < g.K)
+                                   ? __ldg(reinterpret_cast<const float4 *>(res + (size_t)m * g.K + nb + 4 * LN * h))
+                                   : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+#pragma unroll
+            for (int i = 0; i < RB; ++i) {
+                const int m = m0 + wrow + lm + (i0 + ib + i) * LM;
+                if (m >= g.M) continue;
+                float fsrc = 0.f;
+                if (fd.active) {
+                    const int nimg = m / g.PQ, rem = m % g.PQ;
+                    fsrc = f_fault_source(a, nimg, rem / g.Q, rem % g.Q);
+                }
+#pragma unroll
+                for (int h = 0; h < F_TN / 4; ++h) {
+                    const int k = nb + 4 * LN * h;
+                    const float *bp = reinterpret_cast<const float *>(&bias[h]);
+                    const float *rp = reinterpret_cast<const float *>(&rv[i][h]);
+                    float o[4];
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        o[e] = v[ib + i][4 * h + e] + bp[e];
+                        if (fd.active && fd.kout == k + e) o[e] += fd.dv * fsrc;
+                        if (res) o[e] += rp[e];
+                        if (a.relu) o[e] = relu_keep_nan(o[e]);
+                    }
+                    if (k < g.K)
+                        *reinterpret_cast<float4 *>(y + (size_t)m * g.K + k) = make_float4(o[0], o[1], o[2], o[3]);
+                }
+                if (do_cs && ln == 0) {
+                    const float *csi = static_cast<const float *>(a.cs_in);
+                    const int nimg = m / g.PQ, rem = m % g.PQ, p = rem / g.Q, q = rem % g.Q;
+                    const int hc = p * a.stride + (a.R - 1) / 2 - a.pad, wc = q * a.stride + (a.S - 1) / 2 - a.pad;
+                    const bool inb = hc >= 0 && hc < a.H && wc >= 0 && wc < a.W;
+                    const float cin = (csi && inb) ? csi[((size_t)nimg * a.H + hc) * a.W + wc] : 0.f;
+                    float o = 0.f;
+                    if (a.role == CT_ROLE_CT) o = a.coef * (cs[ib + i] + cin);
+                    else if (a.role == CT_ROLE_PASS) o = cin;
+                    if (fd.active && fd.kout == g.K) o += fd.dv * fsrc;
+                    if (a.res_cs) o += static_cast<const float *>(a.res_cs)[m];
+                    if (a.relu) o = relu_keep_nan(o);
+                    static_cast<float *>(a.cs_out)[m] = o;
+                }
+            }
+        }
+        if (KW > 1) csync();               // the reduction buffer is reused by the next piece
+    }
+}
+
+PFN_cuTensorMapEncodeTiled_v12000 f_encode_tiled = nullptr;
+PFN_cuTensorMapEncodeIm2col_v12000 f_encode_im2col = nullptr;
+
+bool f_load_encoders() {
+    static const bool ok = [] {
+        cudaDriverEntryPointQueryResult q;
+        void *p = nullptr;
+        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
+                cudaSuccess && q == cudaDriverEntryPointSuccess)
+            f_encode_tiled = (PFN_cuTensorMapEncodeTiled_v12000)p;
+        p = nullptr;
+        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeIm2col", &p, 12000, cudaEnableDefault, &q) ==
+                cudaSuccess && q == cudaDriverEntryPointSuccess)
+            f_encode_im2col = (PFN_cuTensorMapEncodeIm2col_v12000)p;
+        return f_encode_tiled && f_encode_im2col;
+    }();
+    return ok;
+}
+
+// tile variants: lanes' rows LM, warps WM x WN over the tile, KW over K; ring
+// stages in about 110 KB (two CTAs per SM)
+template <int LM_, int WM_, int WN_, int KW_>
+struct FTile {
+    static constexpr int LM = LM_, WM = WM_, WN = WN_, KW = KW_;
+    static constexpr int BM = LM * F_TM * WM, LN = 32 / LM, BN = LN * F_TN * WN;
+    static constexpr int RED = (KW > 1 ? KW * F_TM * F_TN * 32 * 4 : 0) + F_TM * F_THREADS * 4;
+    static constexpr int FIT = (110 * 1024 - RED) / ((BM + BN) * 128);
+    static constexpr int STAGES = FIT > 6 ? 6 : FIT;
+    static constexpr size_t SMEM = 1024 + (size_t)STAGES * (BM + BN) * 128 + RED + 16 * STAGES;
+    static bool maps(CUtensorMap *am, CUtensorMap *bm, const ConvArgs &a, int max_batch, const void *x, const void *w) {
+        cuuint64_t gdim[4] = {(cuuint64_t)a.C, (cuuint64_t)a.W, (cuuint64_t)a.H, (cuuint64_t)max_batch};
+        cuuint64_t gstr[3] = {(cuuint64_t)a.C * 4, (cuuint64_t)a.W * a.C * 4, (cuuint64_t)a.H * a.W * a.C * 4};
+        int lower[2] = {-a.pad, -a.pad};
+        int upper[2] = {a.pad - (a.S - 1), a.pad - (a.R - 1)};
+        cuuint32_t estr[4] = {1, (cuuint32_t)a.stride, (cuuint32_t)a.stride, 1};
+        if (f_encode_im2col(am, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, const_cast<void *>(x), gdim, gstr, lower, upper,
+                            F_BK, (cuuint32_t)BM, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                            CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+            return false;
+        // weights [K][taps][C] as (channel, filter / 4, filter % 4, tap), which
+        // permutes the filters on their way to shared memory; a block never
+        // reads past its tap's channels (zeros on both sides there, so a
+        // non-finite faulted weight of the next tap cannot meet them)
+        const cuuint64_t tap = (cuuint64_t)a.C * 4, row = tap * a.R * a.S;
+        cuuint64_t wdim[4] = {(cuuint64_t)a.C, (cuuint64_t)a.K / 4, 4, (cuuint64_t)a.R * a.S};
+        cuuint64_t wstr[3] = {4 * row, row, tap};
+        cuuint32_t wes[4] = {1, 1, 1, 1};
+        cuuint32_t box[4] = {F_BK, (cuuint32_t)LN, 4, 1};
+        return f_encode_tiled(bm, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, const_cast<void *>(w), wdim, wstr, box, wes,
+                              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                              CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS &&
+               cudaFuncSetAttribute(conv_ffma2_kernel<LM, WM, WN, KW, STAGES>,
+                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM) == cudaSuccess;
+    }
+    static void launch(const CUtensorMap &am, const CUtensorMap &bm, const ConvArgs &a, FGeom g, int grid,
+                       cudaStream_t st) {
+        pdl_launch(conv_ffma2_kernel<LM, WM, WN, KW, STAGES>, grid, F_CTA, SMEM, st, am, bm, a, g);
+    }
+};
+using FWide = FTile<4, 4, 1, 1>;        // 128 pixels x 64 channels
+using FNarrow = FTile<8, 4, 1, 1>;      // 256 x 32
+using FSmall = FTile<4, 1, 1, 4>;       // 32 x 64, K over the warps
+using FSmallNarrow = FTile<8, 1, 1, 4>; // 64 x 32, K over the warps
+
+}  // namespace
+
+struct FfmaPlan {
+    FGeom g;
+    CUtensorMap amap[4], bmap[4];       // FWide, FNarrow, FSmall, FSmallNarrow
+    int sms;
+};
+
+bool ffma_supported(int C, int K, int R, int S, int stride, int pad) {
+    return C % 4 == 0 && K % 4 == 0 && R == S && R <= 7 && stride >= 1 && stride <= 2 && pad <= 3 && pad <= R / 2 + 1;
+}
+
+void ffma_plan_destroy(FfmaPlan *p) { delete p; }
+
+FfmaPlan *ffma_plan_create(const ConvArgs &a, int max_batch, const void *w_dev, const void *x_dev) {
+    if (!f_load_encoders()) return nullptr;
+    FfmaPlan *pl = new FfmaPlan();
+    memset(pl, 0, sizeof(*pl));
+    FGeom &g = pl->g;
+    pl->sms = device_sm_count();
+    g.PQ = a.P * a.Q; g.Q = a.Q; g.stride = a.stride; g.pad = a.pad; g.C = a.C; g.K = a.K; g.S = a.S;
+    g.RS = a.R * a.S;
+    g.cpb = (a.C + F_BK - 1) / F_BK;
+    g.n_kb = g.RS * g.cpb;
+    g.ctr_tap = ((a.R - 1) / 2) * a.S + (a.S - 1) / 2;
+    if (!FWide::maps(&pl->amap[0], &pl->bmap[0], a, max_batch, x_dev, w_dev) ||
+        !FNarrow::maps(&pl->amap[1], &pl->bmap[1], a, max_batch, x_dev, w_dev) ||
+        !FSmall::maps(&pl->amap[2], &pl->bmap[2], a, max_batch, x_dev, w_dev) ||
+        !FSmallNarrow::maps(&pl->amap[3], &pl->bmap[3], a, max_batch, x_dev, w_dev)) {
+        cudaGetLastError();
+        delete pl;
+        return nullptr;
+    }
+    return pl;
+}
+
+cudaError_t launch_conv_ffma(const ConvArgs &a, const FfmaPlan *pl, cudaStream_t st) {
+    FGeom g = pl->g;
+    g.M = a.N * g.PQ;
+    // channels in 64-wide tiles unless that pads 32 or more of them
+    const bool narrow = (g.K + 63) / 64 * 64 - g.K >= 32;
+    auto tiles_of = [&](int BM, int BN) { return (long long)((g.M + BM - 1) / BM) * ((g.K + BN - 1) / BN); };
+    // small tiles when the large ones are fewer than half the SMs: a tile's
+    // partial sums then take a quarter of the traffic (one CIFAR ResNet-18
+    // image: 295 us with large tiles and a reduction kernel per layer, 239 us
+    // so; shares of six blocks instead of four: its 512-channel layers 43 ->
+    // 18 us together with polling the flags in parallel)
+    const long long large = narrow ? tiles_of(FNarrow::BM, FNarrow::BN) : tiles_of(FWide::BM, FWide::BN);
+    const bool small = large * 2 < pl->sms;
+    const int v = (small ? 2 : 0) + (narrow ? 1 : 0);
+    const long long tiles = v == 0 ? large : v == 1 ? large : v == 2 ? tiles_of(FSmall::BM, FSmall::BN)
+                                                                   : tiles_of(FSmallNarrow::BM, FSmallNarrow::BN);
+    if (tiles * g.n_kb > 0x7fffffffll) return launch_conv_simt(a, false, st, nullptr);   // K-block list beyond 31 bits
+    g.n_tiles = (g.K + (narrow ? 32 : 64) - 1) / (narrow ? 32 : 64);
+    const size_t part = sizeof(float) * (small ? f_partial<4>() : f_partial<1>());
+    // CTAs: two per SM; shares of at least four K blocks (six small ones);
+    // partials that fit the workspace
+    const long long slots = 2 * pl->sms;
+    long long grid = std::min(slots, std::max(tiles, tiles * g.n_kb / (small ? 6 : 4)));
+    if (a.ws && a.sk_flags) grid = std::min<long long>(grid, std::min<long long>(SK_FLAGS, a.ws_bytes / part));
+    else grid = std::min(grid, tiles);
+    // whole tiles per CTA when their last round is nearly full (or nothing
+    // can be split): the partial of a cut tile costs about as much as the
+    // sixteenth of a round that cutting would save
+    const long long rounds = (tiles + grid - 1) / grid;
+    const bool whole = !a.ws || !a.sk_flags || g.n_kb < 2 || (rounds * grid - tiles) * 16 <= tiles;
+    g.unit = whole ? g.n_kb : 1;
+    g.units = (int)(whole ? tiles : tiles * g.n_kb);
+    if (whole) grid = std::min(grid, tiles);
+    g.part = a.ws;
+    g.flags = a.sk_flags;
+    if (v == 0) FWide::launch(pl->amap[0], pl->bmap[0], a, g, (int)grid, st);
+    else if (v == 1) FNarrow::launch(pl->amap[1], pl->bmap[1], a, g, (int)grid, st);
+    else if (v == 2) FSmall::launch(pl->amap[2], pl->bmap[2], a, g, (int)grid, st);
+    else FSmallNarrow::launch(pl->amap[3], pl->bmap[3], a, g, (int)grid, st);
+    return cudaGetLastError();
+}
+
+}  // namespace ct

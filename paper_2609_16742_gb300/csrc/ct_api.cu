@@ -93,6 +93,7 @@ struct LayerRT {
     float *bias = nullptr;
     bool tc = false;
     TcPlan *plan = nullptr;
+    FfmaPlan *fplan = nullptr;   // FP32, input channels a multiple of 4: packed FFMA
     HaloPlan *hplan = nullptr;   // stride-1 3x3 layers: halo tiles when the batch fills the GPU
     bool tc_small = false;       // first layer with <= 4 input channels on the tensor cores
     TcSmallPlan *splan = nullptr;
@@ -150,6 +151,7 @@ struct ct_model {
     uint8_t *rh_flag = nullptr;
     uint32_t *d_err = nullptr;
     float *ws = nullptr;         // split-K partial sums
+    uint32_t *sk_flags = nullptr;   // SK_FLAGS words: partial sums ready (0 between launches)
     // re-execution: one captured inference graph per power-of-two batch
     cudaStream_t cap_stream = nullptr;
     std::vector<cudaGraphExec_t> re_graph;
@@ -215,6 +217,7 @@ void free_all(ct_model *m) {
         if (l.splan) tc_small_plan_destroy(l.splan);
         if (l.stplan) stem_plan_destroy(l.stplan);
         if (l.hplan) halo_plan_destroy(l.hplan);
+        if (l.fplan) ffma_plan_destroy(l.fplan);
     }
     for (void *p : m->dev_allocs) cudaFree(p);
     m->dev_allocs.clear();
@@ -685,6 +688,14 @@ ct_status build_impl(ct_model *m, const ct_model_desc *desc, const float *const 
             if (!l.plan) return CT_ECUDA;
             continue;
         }
+        if (l.d.op == CT_OP_CONV && prec == CT_FP32 && !l.dw && ffma_supported(l.C, l.K, l.R, l.S, l.d.stride, l.d.pad) &&
+            m->slots[l.d.src].cp == l.C) {
+            ConvArgs a{};
+            a.N = B; a.H = l.H; a.W = l.W; a.C = l.C; a.K = l.K; a.R = l.R; a.S = l.S;
+            a.stride = l.d.stride; a.pad = l.d.pad; a.P = l.P; a.Q = l.Q; a.role = l.role; a.coef = l.coef;
+            l.fplan = ffma_plan_create(a, B, l.w, m->slots[l.d.src].data);   // null: conv_simt runs the layer
+            continue;
+        }
         if (!l.tc) continue;
         ConvArgs a{};
         a.N = B; a.H = l.H; a.W = l.W; a.C = l.C; a.K = l.K; a.R = l.R; a.S = l.S;
@@ -745,7 +756,9 @@ ct_status build_impl(ct_model *m, const ct_model_desc *desc, const float *const 
     if ((st = dalloc(m, (void **)&m->rh_flag, B)) != CT_OK) return st;
     if ((st = dalloc(m, (void **)&m->d_err, sizeof(uint32_t))) != CT_OK) return st;
     if ((st = dalloc(m, (void **)&m->ws, SPLITK_WS_BYTES)) != CT_OK) return st;
+    if ((st = dalloc(m, (void **)&m->sk_flags, sizeof(uint32_t) * SK_FLAGS)) != CT_OK) return st;
     CUDA_TRY(cudaMemset(m->d_err, 0, sizeof(uint32_t)));
+    CUDA_TRY(cudaMemset(m->sk_flags, 0, sizeof(uint32_t) * SK_FLAGS));
     if (cudaMallocHost((void **)&m->h_flags, B) != cudaSuccess) return CT_ENOMEM;
     if (cudaHostAlloc((void **)&m->h_idx, sizeof(int32_t) * B, cudaHostAllocMapped) != cudaSuccess ||
         cudaHostGetDevicePointer((void **)&m->h_idx_d, m->h_idx, 0) != cudaSuccess)
@@ -956,7 +969,7 @@ ct_status infer_impl(ct_model *m, const float *input, int batch, float *logits, 
         a.N = batch; a.H = l.H; a.W = l.W; a.C = l.C; a.K = l.K; a.R = l.R; a.S = l.S;
         a.stride = d.stride; a.pad = d.pad; a.P = l.P; a.Q = l.Q;
         a.role = l.role; a.relu = d.relu; a.coef = l.coef; a.err = m->d_err;
-        a.ws = m->ws; a.ws_bytes = SPLITK_WS_BYTES;
+        a.ws = m->ws; a.ws_bytes = SPLITK_WS_BYTES; a.sk_flags = m->sk_flags;
         const bool wfault = armed && m->f_kind == CT_BUF_WEIGHT && m->f_layer == (int)li;
         if (wfault) {
             wf = resolve_weight_fault(m, l, m->f_elem, m->f_bit);
@@ -1022,6 +1035,8 @@ ct_status infer_impl(ct_model *m, const float *input, int batch, float *logits, 
                     sc_done = i + 1;
                 } else if (l.tc) {
                     CUDA_TRY(launch(m, FAM_TC, flops, st, [&] { return launch_conv_tc(a, l.plan, st, &nk); }, &nk));
+                } else if (l.fplan) {
+                    CUDA_TRY(launch(m, FAM_SIMT, flops, st, [&] { return launch_conv_ffma(a, l.fplan, st); }));
                 } else {
                     CUDA_TRY(launch(m, FAM_SIMT, flops, st, [&] { return launch_conv_simt(a, half, st, &nk); }, &nk));
                 }
@@ -1916,6 +1931,8 @@ ct_status ct_device_error(ct_model *m, uint32_t *code) {
     CUDA_TRY(cudaDeviceSynchronize());
     CUDA_TRY(cudaMemcpy(code, m->d_err, sizeof(uint32_t), cudaMemcpyDeviceToHost));
     CUDA_TRY(cudaMemset(m->d_err, 0, sizeof(uint32_t)));
+    // a wait that gave up may leave flags of partial sums set
+    if (*code) CUDA_TRY(cudaMemset(m->sk_flags, 0, sizeof(uint32_t) * SK_FLAGS));
     return CT_OK;
 }
 

@@ -22,6 +22,8 @@ struct FaultDelta {
     float dv;
 };
 
+constexpr int SK_FLAGS = 1024;
+
 // Arguments of every convolution kernel.  Activations are NHWC, the checksum
 // plane is [N, H, W]; weights are KRSC (C innermost).
 struct ConvArgs {
@@ -43,6 +45,7 @@ struct ConvArgs {
                           // is the sum of cs_in[m * cs_rowsum .. m * cs_rowsum + cs_rowsum)
     float *ws;            // split-K workspace (null: never split)
     size_t ws_bytes;
+    uint32_t *sk_flags;   // SK_FLAGS words, 0 between launches (partial sums exchanged between CTAs)
     const void *x2;       // first layer only: images n >= n_split are image n - n_split of x2
     int n_split;          // (null x2: every image comes from x)
     const int32_t *x2_idx;  // non-null: image n >= n_split is image x2_idx[n - n_split] of x2
@@ -231,6 +234,15 @@ ct_status noalloc_scratch_setup(int device);
 
 // number of SMs of the current device (148 if the query fails)
 int device_sm_count();
+
+// FP32 convolution on packed FFMA with TMA-staged operands (conv_ffma2.cu):
+// input and output channels a multiple of 4 (16-byte rows).  The plan holds the tensor
+// maps of the layer's input and weights.
+struct FfmaPlan;
+bool ffma_supported(int C, int K, int R, int S, int stride, int pad);
+FfmaPlan *ffma_plan_create(const ConvArgs &shape_args, int max_batch, const void *w_dev, const void *x_dev);
+void ffma_plan_destroy(FfmaPlan *p);
+cudaError_t launch_conv_ffma(const ConvArgs &a, const FfmaPlan *p, cudaStream_t st);
 
 // tensor-core conv plan (opaque outside conv_tc.cu)
 struct TcPlan;
