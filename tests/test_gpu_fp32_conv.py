@@ -1,0 +1,120 @@
+"""FP32 convolution kernels at the edges of their tiles and K blocks: a
+network of two or three convolutions per shape, every stored tensor against
+the oracle.  Covers the image kernel (3x3 on 1 to 4 channels), the packed-FFMA
+kernel's four tile variants, input channels that do not fill a 32-channel K
+block, output channels that do not fill a tile, strides, shares of a tile's K
+blocks split over CTAs, depthwise strips, and faults in stored and implicit
+weights."""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+from _gpu import TOL, ct, run, same_class
+
+pytestmark = pytest.mark.gpu
+
+
+def net_of(C, K, k, stride, H, cin=3, depthwise=False, residual=False):
+    Ly = synth.Layer
+    L = [Ly("conv", 0, 1, cin=cin, cout=C, k=3, pad=1, relu=True)]
+    s = 1
+    if depthwise:
+        L.append(Ly("conv", 1, 2, cin=C, cout=C, k=3, stride=stride, pad=1, relu=True, ct="pass", groups=C))
+        s, stride = 2, 1
+    if residual:          # block: none, then ct with the block input added
+        L.append(Ly("conv", s, s + 1, cin=C, cout=C, k=3, pad=1, relu=True, ct="none"))
+        L.append(Ly("conv", s + 1, s + 2, cin=C, cout=C, k=3, pad=1, relu=True, res=s))
+        s += 2
+    L.append(Ly("conv", s, s + 1, cin=C, cout=K, k=k, stride=stride, pad=k // 2, relu=True))
+    L.append(Ly("gap", s + 1, s + 2))
+    L.append(Ly("fc", s + 2, s + 3, cin=K, cout=10, final=True))
+    wl = synth.Workload("edge", L, (cin, H, H), 10, 1, "fp32", 7, "normal")
+    return wl, synth.make_params(L, 7), s
+
+
+def check(wl, params, batch, sel, fault=None):
+    m = ct().ct_build_workload(wl, params, max_batch=batch)
+    net = oracle.build_workload(wl, params=params)
+    x = synth.make_input(wl, batch=batch)
+    if fault is not None:
+        ct().ct_inject(m, *fault)
+    lg, S, _ = run(m, x)
+    assert ct().ct_device_error(m) == 0
+    f = None if fault is None else oracle.Fault(*fault)
+    o = oracle.forward(net, x[sel], f, keep=fault is None)
+    tol = TOL["fp32"]
+    for j, i in enumerate(sel):
+        ref = np.append(o["logits"][j], o["S"][j])
+        got = np.append(lg[i], S[i])
+        for a, b in zip(got, ref):
+            assert same_class(a, b), (fault, i, got, ref)
+        fin = np.isfinite(ref)
+        if fin.any():
+            assert (np.abs(got[fin] - ref[fin]) <= tol * np.abs(ref[fin]).max()).all(), (fault, i, got, ref)
+    if fault is None:
+        for L in wl.layers:
+            if L.op != "conv":
+                continue
+            gd, gc = ct().ct_copy_activation(m, L.dst, batch)
+            for j, i in enumerate(sel):
+                a = o["acts"][j][L.dst]
+                assert np.abs(gd[i] - a[:L.cout]).max() <= tol * np.abs(a[:L.cout]).max(), (L.dst, i)
+                if gc is not None:
+                    assert np.abs(gc[i] - a[L.cout]).max() <= tol * max(np.abs(a[L.cout]).max(), 1e-6), (L.dst, i)
+    # the same inference again: no state is left behind
+    again = run(m, x)
+    if fault is None:
+        assert np.array_equal(again[0], lg) and np.array_equal(again[1], S)
+    m.close()
+
+
+@pytest.mark.parametrize("C,K,k,stride,H,batch", [
+    (24, 40, 3, 1, 9, 3),        # K block of 24 channels, 40 of 64 filters, few pixels
+    (36, 132, 3, 2, 13, 5),      # second K block of 4 channels, a tile of 4 filters
+    (16, 16, 1, 1, 16, 2),       # one K block per tile, narrow tiles
+    (16, 24, 1, 1, 32, 200),     # narrow tiles, many whole rounds
+    (144, 24, 1, 1, 16, 40),     # five K blocks, the last of 16 channels
+    (64, 64, 3, 1, 32, 20),      # large tiles, shares that cut tiles
+    (64, 128, 3, 1, 8, 61),      # ragged rows
+    (320, 100, 1, 1, 4, 1),      # 16 pixels
+    (32, 4, 5, 2, 11, 3),        # four filters
+])
+def test_ffma_conv_matches_oracle(C, K, k, stride, H, batch):
+    wl, p, _ = net_of(C, K, k, stride, H)
+    check(wl, p, batch, sorted({0, batch // 2, batch - 1}))
+
+
+@pytest.mark.parametrize("cin,C,H,batch", [(1, 4, 5, 1), (2, 36, 7, 3), (3, 64, 32, 9), (4, 128, 6, 33)])
+def test_image_conv_matches_oracle(cin, C, H, batch):
+    wl, p, _ = net_of(C, 8, 1, 1, H, cin=cin)
+    check(wl, p, batch, sorted({0, batch // 2, batch - 1}))
+
+
+@pytest.mark.parametrize("C,H,stride,batch", [(4, 5, 1, 1), (20, 6, 2, 3), (96, 32, 1, 17), (192, 7, 2, 9)])
+def test_depthwise_matches_oracle(C, H, stride, batch):
+    wl, p, _ = net_of(C, 16, 1, stride, H, depthwise=True)
+    check(wl, p, batch, sorted({0, batch - 1}))
+
+
+@pytest.mark.parametrize("C,H,batch", [(40, 8, 2), (64, 16, 30)])
+def test_residual_block_matches_oracle(C, H, batch):
+    wl, p, _ = net_of(C, 32, 1, 1, H, residual=True)
+    check(wl, p, batch, sorted({0, batch - 1}))
+
+
+@pytest.mark.parametrize("batch", [2, 40])
+def test_faults_match_oracle(batch):
+    """Flips of stored weights (one to infinity next to a tap boundary of a
+    K block that is not full), of the carry-through row and of the zero
+    checksum slice, in the image kernel's and the packed-FFMA kernel's layers."""
+    C, K = 24, 40
+    wl, p, li = net_of(C, K, 3, 1, 10)
+    p[1]["w"][5, 0, 1, 1] = 1.5                      # bit 30 flips 1.5 to NaN / infinity range
+    Ct = C + 1
+    cases = [(0, 0, 3 * 27 + 4, 29), (0, 0, C * 27 + 13, 28),
+             (0, 1, (5 * Ct + 0) * 9 + 4, 30), (0, 1, (7 * Ct + 3) * 9 + 2, 29),
+             (0, 1, (9 * Ct + C) * 9 + 4, 29), (0, 1, (K * Ct + 2) * 9 + 4, 29), (0, 1, (K * Ct + C) * 9 + 0, 28),
+             (1, 1, 3 * 100 + 5, 29), (1, 1, C * 100 + 7, 29)]
+    for f in cases:
+        check(wl, p, batch, [0, batch - 1], f)
