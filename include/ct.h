@@ -446,9 +446,10 @@ ct_status ct_profile_read(ct_model *m, int32_t family, int64_t *launches, double
                           double *flops);
 
 /* Number of library kernels the most recent inference of this model
- * launched (fault-injection bit flips not counted); a layer whose K
- * dimension is split across CTAs (small batches) launches two.  Before the
- * first inference: the count without split K. */
+ * launched (fault-injection bit flips not counted); an FC layer, or a
+ * convolution on the general CUDA-core kernel, whose K dimension is split
+ * across CTAs (small batches) launches two.  Before the first inference: the
+ * count without split K. */
 ct_status ct_launches_per_infer(const ct_model *m, int32_t *n);
 
 /* ct_kernel_count -- number of library kernels launched for this model since

@@ -13,10 +13,8 @@
 //     non-zero part is a constant 16-row tile (row 0 = coef) kept after the
 //     weight rows in shared memory, and the centre-tap K blocks, which the
 //     K loop visits first, are issued with N = BN + 16: the tensor core
-//     computes the checksum column.  For BN = 256 two spare warps compute it
-//     from the same A tiles with warp-level MMAs against a ones vector
-//     (conv_tc_kernel), or the epilogue adds up the centre-tap pixel's
-//     channels (conv_tc_pair_kernel).
+//     computes the checksum column.  For BN = 256 the epilogue adds up the
+//     centre-tap pixel's channels (conv_tc_pair_kernel).
 //   The incoming checksum plane (weight coef at the centre), the residual
 //   checksum and the epilogue (bias, residual, ReLU) are applied by the
 //   epilogue warps.
@@ -32,15 +30,16 @@
 // (a ResNet downsample) can run in the launch of its block's first
 // convolution, whose centre-tap K blocks are its A operand (UnitSeq).
 //
-// With N = 256 and no split K, conv_tc_pair_kernel runs the tiles on pairs of
+// With N = 256, conv_tc_pair_kernel runs the tiles on pairs of
 // CTAs (a cluster of two, tcgen05 cta_group::2): one M = 256 MMA reads the
 // 128 A rows and 128 weight rows each CTA holds, which halves the weight
 // bytes every SM copies and reads per step.  Its epilogue sums the
 // carry-through column from the centre-tap input pixel.
 //
-// Warp roles.  conv_tc_kernel: a producer group (producer warps, each owning
-// whole ring slots, plus for N = 256 the two carry-through warps), one MMA
-// warp (one elected lane issues tcgen05.mma), eight epilogue warps;
+// Layers with few tiles split K over a cluster (conv_tc_cluster_kernel).
+//
+// Warp roles.  conv_tc_kernel: producer warps (each owning whole ring slots),
+// one MMA warp (one elected lane issues tcgen05.mma), eight epilogue warps;
 // conv_tc_pair_kernel: three producer warps, each owning two ring slots (with
 // two, the copy issue held the 7 x 7 layers back by 8%, measured), the MMA
 // warp (issuing in the even CTA only), eight epilogue warps.
@@ -71,18 +70,15 @@ constexpr int BK = 64;             // channels per K block (128 bytes of fp16)
 constexpr int A_BYTES = BM * BK * 2;
 constexpr int NTHREADS = 320;      // 1 TMA warp, 1 MMA warp, 8 epilogue warps
 constexpr int N_EPI_WARPS = 8;
-// conv_tc_kernel: a producer group (TMA producer warps, each owning whole ring
-// slots, plus for N = 256 two carry-through warps), one MMA warp, 8 epilogue
-// warps.  The group is as large as the variant needs: a warp fewer raises the
-// register budget of a 1-CTA-per-SM kernel (384 threads: 168 registers, 416:
-// 128).
-constexpr int tc_nprod(int BN, int STAGES) {
-    return BN > 128 ? 2 : STAGES % 4 == 0 ? 4 : STAGES % 3 == 0 ? 3 : STAGES % 2 == 0 ? 2 : 1;
-}
-constexpr int tc_npg(int BN, int STAGES) { return BN > 128 ? 4 : tc_nprod(BN, STAGES); }
-constexpr int tc_threads(int BN, int STAGES) { return 32 * (tc_npg(BN, STAGES) + 1 + N_EPI_WARPS); }
+// conv_tc_kernel: TMA producer warps (each owning whole ring slots), one MMA
+// warp, 8 epilogue warps.  There are as few producers as the ring allows: a
+// warp fewer raises the register budget of a 1-CTA-per-SM kernel (384
+// threads: 168 registers, 416: 128).
+constexpr int tc_nprod(int STAGES) { return STAGES % 4 == 0 ? 4 : STAGES % 3 == 0 ? 3 : STAGES % 2 == 0 ? 2 : 1; }
+constexpr int tc_threads(int STAGES) { return 32 * (tc_nprod(STAGES) + 1 + N_EPI_WARPS); }
 
-enum CtMode { CT_NONE_ = 0, CT_MERGED = 1, CT_SEPARATE = 2 };
+// carry-through column: none, or (on the first channel tile) computed
+enum CtMode { CT_NONE_ = 0, CT_COLUMN = 1 };
 
 struct TcGeom {
     int M, PQ, Q, stride, pad, C, K, RSC;
@@ -90,7 +86,7 @@ struct TcGeom {
     int ct_mode;
     int tmem_cols;
     int m_tiles, n_tiles;
-    int splits, kps, ws_ld;      // split-K: K blocks per split, workspace row length
+    int splits, kps;             // conv_tc_cluster_kernel: cluster size, K blocks per CTA
     // conv_tc_pair_kernel<true>: tiles t_first .. end are each run as two
     // 128-channel halves, units 0 .. units - t_first - 1 (unit 2 * (tile -
     // t_first) + half); whole tiles 0 .. t_first - 1 follow them
@@ -103,22 +99,16 @@ struct TcGeom {
     uint16_t coef_h;
 };
 
-// K-block range [lo, hi) and output tile of persistent work item `item`.
+// Output tile of persistent work item `item`.
 struct TileRef {
-    int m0, n_tile, sp, kb_lo, kb_hi;
+    int m0, n_tile;
 };
 __device__ __forceinline__ TileRef tile_ref(int item, const TcGeom &g) {
     TileRef t;
-    const int per = g.m_tiles * g.n_tiles;
-    t.sp = item / per;
-    const int rt = item - t.sp * per;
-    t.m0 = (rt / g.n_tiles) * BM;
-    t.n_tile = rt % g.n_tiles;
-    t.kb_lo = t.sp * g.kps;
-    t.kb_hi = min(g.n_kb, t.kb_lo + g.kps);
+    t.m0 = (item / g.n_tiles) * BM;
+    t.n_tile = item % g.n_tiles;
     return t;
 }
-
 
 // Work units of one CTA (or CTA pair) cid of ncl: first this layer's n1
 // units, round-robin (cid, cid + ncl, ...), then a contiguous share of the
@@ -462,7 +452,7 @@ __device__ __forceinline__ void store_checksum_pre(float ctv, const CsIn &c, con
 // SC: the launch also runs a 1x1 shortcut convolution (bmap2, a2, g2; see
 // UnitSeq); otherwise those arguments are unused.
 template <int BN, int STAGES, int SUB, int NCH, bool SC>
-__global__ void __launch_bounds__(tc_threads(BN, STAGES), 1)
+__global__ void __launch_bounds__(tc_threads(STAGES), 1)
 conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ CUtensorMap bmap,
                const __grid_constant__ ConvArgs a, const __grid_constant__ TcGeom g,
                const __grid_constant__ CUtensorMap bmap2, const __grid_constant__ ConvArgs a2,
@@ -471,58 +461,40 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
     constexpr int B_SUB_BYTES = B_ROWS * BK * 2;
     constexpr int B_TMA_BYTES = BN * BK * 2;
     constexpr int CH = BN + 16;                           // TMEM columns per chain
-    constexpr bool EARLY = BN <= 128;                     // release TMEM before the stores
-    // N = 256: two 256-column accumulators fill TMEM, so the carry-through
-    // column is summed (warp-level MMAs against a ones vector) from the
-    // centre-tap A tiles in shared memory by the warps of the producer group
-    // that do not issue copies (they consume every stage, like the MMA warp),
-    // and the epilogue of one tile overlaps the MMAs of the next
-    constexpr bool DBUF = !EARLY;
-    // accumulator buffers, 256 TMEM columns apart: two when both fit (N =
-    // 256; N <= 128 with one chain), so that a tile's MMAs never wait for
-    // the previous tile's epilogue to read TMEM
-    constexpr int NACC = (DBUF || 2 * NCH * CH <= 512) ? 2 : 1;
-    static_assert(NACC == 1 || DBUF || NCH * CH <= 256, "an accumulator buffer spans at most 256 columns");
-    // producer warps (each owns whole ring slots) and carry-through warps
-    constexpr int NPROD = tc_nprod(BN, STAGES);
-    constexpr int NPG = tc_npg(BN, STAGES);               // producer group: producers + carry-through warps
-    constexpr int NCT = DBUF ? NPG - NPROD : 0;
-    constexpr int TC_MMA_WARP = NPG;
-    constexpr int TC_EPI_WARP0 = NPG + 1;
+    // accumulator buffers, 256 TMEM columns apart: two when both fit, so that
+    // a tile's MMAs never wait for the previous tile's epilogue to read TMEM
+    constexpr int NACC = 2 * NCH * CH <= 512 ? 2 : 1;
+    static_assert(BN <= 128 && (NACC == 1 || NCH * CH <= 256), "an accumulator buffer spans at most 256 columns");
+    constexpr int NPROD = tc_nprod(STAGES);               // producer warps (each owns whole ring slots)
+    constexpr int TC_MMA_WARP = NPROD;
+    constexpr int TC_EPI_WARP0 = NPROD + 1;
     static_assert(STAGES % NPROD == 0, "producer warps must own whole ring slots");
-    static_assert(DBUF ? NCT > 0 : NCT == 0, "carry-through warps only beside double-buffered accumulators");
-    static_assert(!DBUF || (NCT > 0 && BM % (16 * (NCT > 0 ? NCT : 1)) == 0), "carry-through warps split the tile rows");
-    static_assert(!SC || !DBUF, "a shortcut only beside single-buffered accumulators");
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     uint8_t *As = smem;                                   // [STAGES][SUB][A_BYTES]
     uint8_t *Bs = As + STAGES * SUB * A_BYTES;            // [STAGES][SUB][B_SUB_BYTES]
-    uint8_t *CTt = Bs + STAGES * SUB * B_SUB_BYTES;       // separate 16-row carry-through tile
-    float *ct_sum = (float *)(CTt + 16 * BK * 2);          // [2][BM] carry-through sums (DBUF)
-    uint64_t *full = (uint64_t *)(ct_sum + 2 * BM);
+    uint64_t *full = (uint64_t *)(Bs + STAGES * SUB * B_SUB_BYTES);
     uint64_t *empty = full + STAGES;
     uint64_t *acc_full = empty + STAGES;                  // [2]
     uint64_t *acc_empty = acc_full + 2;                   // [2]
-    uint64_t *ct_ready = acc_empty + 2;                   // [2]
-    uint32_t *tmem_holder = (uint32_t *)(ct_ready + 2);
+    uint32_t *tmem_holder = (uint32_t *)(acc_empty + 2);
     volatile uint32_t *abort_flag = tmem_holder + 1;
     float *bias_s = (float *)(((uintptr_t)(tmem_holder + 2) + 15) & ~(uintptr_t)15);   // [BIAS_SMEM]
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int cid = blockIdx.x, ncl = gridDim.x;
-    const int n1 = g.m_tiles * g.n_tiles * g.splits;     // this layer's items
+    const int n1 = g.m_tiles * g.n_tiles;                // this layer's items
     const UnitSeq us = unit_seq<SC>(cid, ncl, n1, g);
     const int n_units = us.k1 + us.cnt;                 // this CTA's units
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) {
             mbar_init(smem_u32(&full[s]), 1);
-            mbar_init(smem_u32(&empty[s]), 1 + NCT);   // MMA commit + carry-through warps
+            mbar_init(smem_u32(&empty[s]), 1);
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(smem_u32(&acc_full[b]), 1);
             mbar_init(smem_u32(&acc_empty[b]), N_EPI_WARPS);
-            mbar_init(smem_u32(&ct_ready[b]), NCT > 0 ? NCT : 1);
         }
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -540,8 +512,6 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
             uint32_t *rows = (uint32_t *)(Bs + sb * B_SUB_BYTES + BN * BK * 2);
             for (int i = t; i < 16 * BK / 2; i += 32 * N_EPI_WARPS) rows[i] = (i < BK / 2) ? coef2 : 0u;
         }
-        uint32_t *ctt = (uint32_t *)CTt;
-        for (int i = t; i < 16 * BK / 2; i += 32 * N_EPI_WARPS) ctt[i] = (i < BK / 2) ? coef2 : 0u;
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -578,12 +548,13 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
             const int p = rem / g.Q, q = rem % g.Q;
             const int w0 = q * g.stride - g.pad, h0 = p * g.stride - g.pad;
             bool ok = true;
-            for (int kb0 = tr.kb_lo; kb0 < tr.kb_hi; kb0 += SUB, ++it) {
+            const int n_kb = sc ? g2.n_kb : g.n_kb;
+            for (int kb0 = 0; kb0 < n_kb; kb0 += SUB, ++it) {
                 const int s = it % STAGES;
                 if (s % NPROD != warp) continue;
                 const uint32_t ph = (uint32_t)(it / STAGES) & 1u;
                 if (!warp_wait(smem_u32(&empty[s]), ph ^ 1u, a.err, 1u)) { ok = false; break; }
-                const int nsub = min(SUB, tr.kb_hi - kb0);
+                const int nsub = min(SUB, n_kb - kb0);
                 const uint32_t fb = smem_u32(&full[s]);
                 if (elect_one()) {
                     mbar_arrive_expect_tx(fb, nsub * (A_BYTES + B_TMA_BYTES));
@@ -606,8 +577,6 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
         // ---------------- MMA issuer (whole warp, one lane issues) ----------------
         const uint32_t id_main = idesc_f16(BM, BN);
         const uint32_t id_merged = idesc_f16(BM, BN + 16);
-        const uint32_t id_ct = idesc_f16(BM, 16);
-        const uint32_t ct_base = smem_u32(CTt);
         int it = 0;
         for (int lt = 0; lt < n_units; ++lt) {
             if (__any_sync(0xffffffffu, *abort_flag)) break;
@@ -625,36 +594,26 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
             }
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             bool ok = true;
-            for (int kb0 = tr.kb_lo; kb0 < tr.kb_hi; kb0 += SUB, ++it) {
+            for (int kb0 = 0; kb0 < G.n_kb; kb0 += SUB, ++it) {
                 const int s = it % STAGES;
                 const uint32_t ph = (uint32_t)(it / STAGES) & 1u;
                 if (!warp_wait(smem_u32(&full[s]), ph, a.err, 2u)) { ok = false; break; }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const int nsub = min(SUB, tr.kb_hi - kb0);
+                const int nsub = min(SUB, G.n_kb - kb0);
                 if (elect_one()) {
                     // descriptors advance 32 bytes (2 in the 16-byte address field)
                     // per 16-element K step; the instruction choice is per K block
                     for (int j = 0; j < nsub; ++j) {
                         const int kb = kb0 + j;
-                        const int kr = kb - tr.kb_lo;               // position within this split
-                        const uint32_t d = tmem + (uint32_t)(ab * 256 + (kr % NCH) * CH);
+                        const uint32_t d = tmem + (uint32_t)(ab * 256 + (kb % NCH) * CH);
                         const bool centre = kb < G.cpb;
                         const uint64_t ad0 = smem_desc_sw128(smem_u32(As + (s * SUB + j) * A_BYTES));
                         const uint64_t bd0 = smem_desc_sw128(smem_u32(Bs + (s * SUB + j) * B_SUB_BYTES));
-                        const uint32_t acc0 = kr >= NCH ? 1u : 0u;  // first use of the chain
-                        if (!DBUF && ct_here && centre && G.ct_mode == CT_SEPARATE) {
-                            const uint64_t cd0 = smem_desc_sw128(ct_base);
+                        const uint32_t acc0 = kb >= NCH ? 1u : 0u;  // first use of the chain
+                        const uint32_t idm = ct_here && centre ? id_merged : id_main;
 #pragma unroll
-                            for (int k16 = 0; k16 < BK / 16; ++k16) {
-                                umma_f16(d, ad0 + 2 * k16, bd0 + 2 * k16, id_main, k16 ? 1u : acc0);
-                                umma_f16(d + BN, ad0 + 2 * k16, cd0 + 2 * k16, id_ct, k16 ? 1u : acc0);
-                            }
-                        } else {
-                            const uint32_t idm = (!DBUF && ct_here && centre && G.ct_mode == CT_MERGED) ? id_merged : id_main;
-#pragma unroll
-                            for (int k16 = 0; k16 < BK / 16; ++k16)
-                                umma_f16(d, ad0 + 2 * k16, bd0 + 2 * k16, idm, k16 ? 1u : acc0);
-                        }
+                        for (int k16 = 0; k16 < BK / 16; ++k16)
+                            umma_f16(d, ad0 + 2 * k16, bd0 + 2 * k16, idm, k16 ? 1u : acc0);
                     }
                 }
                 __syncwarp();
@@ -665,78 +624,8 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
             if (elect_one()) umma_commit(smem_u32(&acc_full[ab]));   // fires when the tile's MMAs have completed
             __syncwarp();
         }
-    } else if (warp < NPG) {
-        if (NCT > 0) {
-            // ---------------- carry-through sums (N = 256) ----------------
-            // Consumes every stage in order (arrives on its empty barrier);
-            // on the centre-tap K blocks of the first N tile it adds each A
-            // row's 64 channels.  The row sums run on the warp-level MMA
-            // against a B of ones (FP32 accumulation, like the tcgen05
-            // column of the other kernels): per K block and 64-row share,
-            // 16 ldmatrix + 16 MMAs.  Rows are read through the 128-byte
-            // swizzle (chunk c of row r sits at chunk c ^ (r & 7)), so the
-            // eight rows of one 8x8 matrix hit eight different bank groups.
-            constexpr int ROWS_W = BM / (NCT > 0 ? NCT : 1);       // rows per carry-through warp
-            constexpr int MT = ROWS_W / 16;                          // 16-row MMA tiles per warp
-            const float coef = __half2float(__ushort_as_half(g.coef_h));
-            const int w = warp - NPROD;
-            // ldmatrix row address of this lane: matrix lane / 8 = (rows +8, chunk +1) bits
-            const int lm_row = (lane & 7) + ((lane >> 3) & 1) * 8, lm_chk = lane >> 4;
-            int it = 0;
-            bool ok = true;
-            for (int lt = 0; lt < n_units && ok; ++lt) {
-                if (__any_sync(0xffffffffu, *abort_flag)) break;
-                const TileRef tr = tile_ref(unit_at(us, lt, cid, ncl), g);
-                const bool ct_here = g.ct_mode != CT_NONE_ && tr.n_tile == 0;
-                const int ab = lt & 1;
-                float acc[MT][4];
-#pragma unroll
-                for (int m = 0; m < MT; ++m)
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) acc[m][e] = 0.f;
-                for (int kb0 = tr.kb_lo; kb0 < tr.kb_hi; kb0 += SUB, ++it) {
-                    const int s = it % STAGES;
-                    if (!warp_wait(smem_u32(&full[s]), (uint32_t)(it / STAGES) & 1u, a.err, 2u)) { ok = false; break; }
-                    const int nsub = min(SUB, tr.kb_hi - kb0);
-                    for (int j = 0; j < nsub; ++j) {
-                        if (!(ct_here && kb0 + j < g.cpb)) continue;
-                        const uint32_t tbase = smem_u32(As + (s * SUB + j) * A_BYTES);
-#pragma unroll
-                        for (int m = 0; m < MT; ++m) {
-                            const int row = w * ROWS_W + m * 16 + lm_row;
-                            const uint32_t rbase = tbase + (uint32_t)row * 128u;
-#pragma unroll
-                            for (int t = 0; t < 4; ++t) {
-                                const uint32_t chk = (uint32_t)((2 * t + lm_chk) ^ (row & 7));
-                                uint32_t a0, a1, a2, a3;
-                                ldsm_x4(rbase + chk * 16u, a0, a1, a2, a3);
-                                mma_rowsum_16x16(acc[m], a0, a1, a2, a3);
-                            }
-                        }
-                    }
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(smem_u32(&empty[s]));
-                }
-                if (!ok) break;
-                // ct_sum[ab] is free once the epilogue released accumulator ab
-                if (!warp_wait(smem_u32(&acc_empty[ab]), ((uint32_t)(lt >> 1) & 1u) ^ 1u, a.err, 8u)) { ok = false; break; }
-                // D fragment: lane l holds rows l / 4 (acc[m][0]) and l / 4 + 8 (acc[m][2]) of tile m
-                if ((lane & 3) == 0) {
-#pragma unroll
-                    for (int m = 0; m < MT; ++m) {
-                        const int r0 = w * ROWS_W + m * 16 + (lane >> 2);
-                        ct_sum[ab * BM + r0] = coef * acc[m][0];
-                        ct_sum[ab * BM + r0 + 8] = coef * acc[m][2];
-                    }
-                }
-                __syncwarp();
-                if (lane == 0) mbar_arrive(smem_u32(&ct_ready[ab]));
-            }
-            if (!ok && lane == 0) *abort_flag = 1;
-        }
     } else if (warp >= TC_EPI_WARP0) {
         // ---------------- epilogue: 8 warps ----------------
-        // (producer warps beyond NPROD have no role)
         const int ep = warp - TC_EPI_WARP0;
         const int quad = warp & 3;                 // TMEM lanes this warp may read
         const int half = ep >> 2;                  // which half of the tile's channels
@@ -752,7 +641,6 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
             const float *bias_l = bias_s + (sc ? G.K : 0);
             const __half *x = static_cast<const __half *>(A.x);
             const FaultDelta fd = A.fd;
-            const bool split = G.splits > 1;
             const bool has_res = A.res != nullptr, relu = A.relu != 0;
             const TileRef tr = tile_ref(sc ? unit - n1 : unit, G);
             const int m0 = tr.m0, n_tile = tr.n_tile;
@@ -762,25 +650,24 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
                 const int mp = m0 + row;
 #pragma unroll
                 for (int c = 0; c < BN / 32; ++c)
-                    rs[c] = (mp < G.M && G.splits == 1)
+                    rs[c] = mp < G.M
                                 ? load_res16(A, G.K, (size_t)mp, n_tile * BN + half * (BN / 2) + 16 * c)
                                 : Res16{make_uint4(0u, 0u, 0u, 0u), make_uint4(0u, 0u, 0u, 0u)};
             }
             CsIn csv{0.f, 0, 0};
             {
                 const int mp = m0 + row;
-                if (half == 0 && A.cs_out != nullptr && n_tile == 0 && mp < G.M && G.splits == 1) {
+                if (half == 0 && A.cs_out != nullptr && n_tile == 0 && mp < G.M) {
                     const int ni = mp / G.PQ, rm = mp % G.PQ;
                     csv = load_cs_inputs(A, G, mp, ni, rm / G.Q, rm % G.Q);
                 }
             }
-            const int chains = min(NCH, tr.kb_hi - tr.kb_lo);                    // chains that received MMAs
+            const int chains = min(NCH, G.n_kb);                                 // chains that received MMAs
             // chains whose first K block is a centre block hold a carry-through column
-            const int ct_chains = max(0, min(NCH, min(G.cpb, tr.kb_hi) - tr.kb_lo));
+            const int ct_chains = min(NCH, G.cpb);
             const int ab = NACC == 2 ? (lt & 1) : 0;
             const uint32_t aph = NACC == 2 ? ((uint32_t)(lt >> 1) & 1u) : ((uint32_t)lt & 1u);
             bool ok = mbar_wait(smem_u32(&acc_full[ab]), aph, A.err, 4u) && !*abort_flag;
-            if (DBUF) ok = ok && mbar_wait(smem_u32(&ct_ready[ab]), aph, A.err, 4u);
             ok = __all_sync(0xffffffffu, ok);      // tcgen05.ld below is warp-collective
             if (!ok) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -790,7 +677,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
             const int mm = valid ? m : 0;
             const int nimg = mm / G.PQ, rem = mm % G.PQ, p = rem / G.Q, q = rem % G.Q;
             float fsrc = 0.f;
-            if (fd.active && !split) {
+            if (fd.active) {
                 const int h = p * G.stride + fd.r - G.pad, w = q * G.stride + fd.s - G.pad;
                 if (h >= 0 && h < A.H && w >= 0 && w < A.W) {
                     if (fd.cin < G.C) fsrc = ldh(x, (((size_t)nimg * A.H + h) * A.W + w) * G.C + fd.cin);
@@ -800,113 +687,76 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
             const int n0 = n_tile * BN;
             const bool do_cs = half == 0 && A.cs_out != nullptr && n_tile == 0;
             float ctv = 0.f;
-            if (EARLY) {
-                // TMEM reads in few round trips: chain 0 (all of this warp's
-                // columns) with the carry-through columns, then the other
-                // chains two chunks at a time; the sums keep the order
-                // ((chain 0 + chain 1) + chain 2) + ...
-                float vals[BN / 2];
-                const bool ld_ct = do_cs && G.ct_mode != CT_NONE_;
-                uint32_t ctr[NCH];
-                {
-                    uint32_t tv[BN / 32][16];
+            // TMEM reads in few round trips: chain 0 (all of this warp's
+            // columns) with the carry-through columns, then the other
+            // chains two chunks at a time; the sums keep the order
+            // ((chain 0 + chain 1) + chain 2) + ...
+            float vals[BN / 2];
+            const bool ld_ct = do_cs && G.ct_mode != CT_NONE_;
+            uint32_t ctr[NCH];
+            {
+                uint32_t tv[BN / 32][16];
 #pragma unroll
-                    for (int c = 0; c < BN / 2; c += 16) tmem_ld16_nw(trow + half * (BN / 2) + c, tv[c / 16]);
-#pragma unroll
-                    for (int ch = 0; ch < NCH; ++ch)
-                        if (ld_ct && ch < ct_chains) tmem_ld1_nw(trow + ch * CH + BN, ctr[ch]);
-                    tmem_wait_ld();
-#pragma unroll
-                    for (int c = 0; c < BN / 2; c += 16) tmem_done16(tv[c / 16], vals + c);
-                }
-                for (int ch = 1; ch < chains; ++ch) {
-#pragma unroll
-                    for (int c = 0; c < BN / 2; c += 32) {
-                        uint32_t t2[2][16];
-                        tmem_ld16_nw(trow + ch * CH + half * (BN / 2) + c, t2[0]);
-                        tmem_ld16_nw(trow + ch * CH + half * (BN / 2) + c + 16, t2[1]);
-                        tmem_wait_ld();
-                        float t[16];
-                        tmem_done16(t2[0], t);
-#pragma unroll
-                        for (int i = 0; i < 16; ++i) vals[c + i] += t[i];
-                        tmem_done16(t2[1], t);
-#pragma unroll
-                        for (int i = 0; i < 16; ++i) vals[c + 16 + i] += t[i];
-                    }
-                }
+                for (int c = 0; c < BN / 2; c += 16) tmem_ld16_nw(trow + half * (BN / 2) + c, tv[c / 16]);
 #pragma unroll
                 for (int ch = 0; ch < NCH; ++ch)
-                    if (ld_ct && ch < ct_chains) ctv += tmem_done(ctr[ch]);
-                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-                __syncwarp();
-                if (lane == 0) mbar_arrive(smem_u32(&acc_empty[ab]));   // accumulators free for a later tile
-                if (valid && split) {
-                    float *wrow = A.ws + ((size_t)tr.sp * G.M + m) * G.ws_ld;
+                    if (ld_ct && ch < ct_chains) tmem_ld1_nw(trow + ch * CH + BN, ctr[ch]);
+                tmem_wait_ld();
 #pragma unroll
-                    for (int c = 0; c < BN / 2; c += 4)
-                        *reinterpret_cast<float4 *>(wrow + n0 + half * (BN / 2) + c) =
-                            make_float4(vals[c], vals[c + 1], vals[c + 2], vals[c + 3]);
-                    if (do_cs) wrow[G.K] = ctv;
-                } else if (valid && fd.active) {
+                for (int c = 0; c < BN / 2; c += 16) tmem_done16(tv[c / 16], vals + c);
+            }
+            for (int ch = 1; ch < chains; ++ch) {
 #pragma unroll
-                    for (int c = 0; c < BN / 2; c += 16)
-                        store_chunk_pre(vals + c, rs[c / 16], A, G.K, (size_t)m, n0 + half * (BN / 2) + c, fsrc);
-                    if (do_cs) store_checksum_pre(ctv, csv, A, G, m, fsrc);
-                } else if (BN == 128 && !split && !fd.active && !has_res) {
-                    // whole lines: the lanes of each group of four swap their
-                    // 16-channel pieces (all lanes take part; stores of pixels
-                    // past M are skipped)
-                    uint32_t pk[4][8];
+                for (int c = 0; c < BN / 2; c += 32) {
+                    uint32_t t2[2][16];
+                    tmem_ld16_nw(trow + ch * CH + half * (BN / 2) + c, t2[0]);
+                    tmem_ld16_nw(trow + ch * CH + half * (BN / 2) + c + 16, t2[1]);
+                    tmem_wait_ld();
+                    float t[16];
+                    tmem_done16(t2[0], t);
 #pragma unroll
-                    for (int c = 0; c < 4; ++c)
-                        pack16(vals + 16 * c, bias16_at(bias_l, A.bias, bias_sm, n0 + half * (BN / 2) + 16 * c), relu,
-                               pk[c]);
-                    transpose4_pieces(pk, lane & 3);
+                    for (int i = 0; i < 16; ++i) vals[c + i] += t[i];
+                    tmem_done16(t2[1], t);
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        const int mk = m0 + quad * 32 + (lane & ~3) + k;
-                        if (mk < G.M)
-                            st_global_v8(static_cast<__half *>(A.y) + (size_t)mk * G.K + n0 + half * (BN / 2) +
-                                             16 * (lane & 3), pk[k]);
-                    }
-                    if (do_cs && valid) store_checksum_pre(ctv, csv, A, G, m, 0.f);
-                } else if (valid) {
-                    __half *yrow = static_cast<__half *>(A.y) + (size_t)m * G.K + n0 + half * (BN / 2);
-#pragma unroll
-                    for (int c = 0; c < BN / 2; c += 16)
-                        store16_fast(vals + c, bias16_at(bias_l, A.bias, bias_sm, n0 + half * (BN / 2) + c), rs[c / 16], has_res,
-                                     relu, yrow + c);
-                    if (do_cs) store_checksum_pre(ctv, csv, A, G, m, 0.f);
+                    for (int i = 0; i < 16; ++i) vals[c + 16 + i] += t[i];
                 }
-            } else {
+            }
 #pragma unroll
-                for (int c = half * (BN / 2); c < (half + 1) * (BN / 2); c += 16) {
-                    float v[16];
-                    tmem_ld16(trow + c, v);
-                    for (int ch = 1; ch < chains; ++ch) {
-                        float t[16];
-                        tmem_ld16(trow + ch * CH + c, t);
+            for (int ch = 0; ch < NCH; ++ch)
+                if (ld_ct && ch < ct_chains) ctv += tmem_done(ctr[ch]);
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&acc_empty[ab]));   // accumulators free for a later tile
+            if (valid && fd.active) {
 #pragma unroll
-                        for (int i = 0; i < 16; ++i) v[i] += t[i];
-                    }
-                    if (valid && split) {
-                        float4 *wp = reinterpret_cast<float4 *>(A.ws + ((size_t)tr.sp * G.M + m) * G.ws_ld + n0 + c);
+                for (int c = 0; c < BN / 2; c += 16)
+                    store_chunk_pre(vals + c, rs[c / 16], A, G.K, (size_t)m, n0 + half * (BN / 2) + c, fsrc);
+                if (do_cs) store_checksum_pre(ctv, csv, A, G, m, fsrc);
+            } else if (BN == 128 && !fd.active && !has_res) {
+                // whole lines: the lanes of each group of four swap their
+                // 16-channel pieces (all lanes take part; stores of pixels
+                // past M are skipped)
+                uint32_t pk[4][8];
 #pragma unroll
-                        for (int i = 0; i < 4; ++i) wp[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
-                    } else if (valid && fd.active) {
-                        store_chunk_pre(v, rs[(c - half * (BN / 2)) / 16], A, G.K, (size_t)m, n0 + c, fsrc);
-                    } else if (valid) {
-                        store16_fast(v, bias16_at(bias_l, A.bias, bias_sm, n0 + c), rs[(c - half * (BN / 2)) / 16], has_res,
-                                     relu, static_cast<__half *>(A.y) + (size_t)m * G.K + n0 + c);
-                    }
+                for (int c = 0; c < 4; ++c)
+                    pack16(vals + 16 * c, bias16_at(bias_l, A.bias, bias_sm, n0 + half * (BN / 2) + 16 * c), relu,
+                           pk[c]);
+                transpose4_pieces(pk, lane & 3);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const int mk = m0 + quad * 32 + (lane & ~3) + k;
+                    if (mk < G.M)
+                        st_global_v8(static_cast<__half *>(A.y) + (size_t)mk * G.K + n0 + half * (BN / 2) +
+                                         16 * (lane & 3), pk[k]);
                 }
-                if (do_cs && G.ct_mode != CT_NONE_) ctv = ct_sum[ab * BM + row];
-                if (do_cs && valid && split) A.ws[((size_t)tr.sp * G.M + m) * G.ws_ld + G.K] = ctv;
-                else if (do_cs && valid) store_checksum_pre(ctv, csv, A, G, m, fsrc);
-                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-                __syncwarp();
-                if (lane == 0) mbar_arrive(smem_u32(&acc_empty[ab]));
+                if (do_cs && valid) store_checksum_pre(ctv, csv, A, G, m, 0.f);
+            } else if (valid) {
+                __half *yrow = static_cast<__half *>(A.y) + (size_t)m * G.K + n0 + half * (BN / 2);
+#pragma unroll
+                for (int c = 0; c < BN / 2; c += 16)
+                    store16_fast(vals + c, bias16_at(bias_l, A.bias, bias_sm, n0 + half * (BN / 2) + c), rs[c / 16], has_res,
+                                 relu, yrow + c);
+                if (do_cs) store_checksum_pre(ctv, csv, A, G, m, 0.f);
             }
         }
     }
@@ -915,6 +765,292 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
     if (warp == TC_MMA_WARP) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)g.tmem_cols));
+    }
+}
+
+// ---------------------------------------------------------------------------
+// K split over a cluster, for layers with few output tiles (small batches,
+// re-execution, deep layers, hidden FC layers).  The Z CTAs of a cluster
+// compute the same 128-pixel x BN-channel tile, each over its own K blocks,
+// and add their partial sums through distributed shared memory: CTA r owns
+// rows r * 128 / Z .. of the tile; every CTA writes its FP32 partial rows into
+// their owners' shared memory (the pipeline stages: a cluster barrier first
+// makes sure that every CTA's MMAs have completed), and after a second
+// barrier each owner adds the Z partials in K order from its own shared memory
+// and applies the epilogue.  One launch per layer, no workspace.  (Owners
+// that read their peers' memory instead paid a remote round trip per eight
+// channels: the 128-channel tiles ran 20-30 us.)
+//
+// These layers are bound by latency: a launch, two or three copy round trips,
+// the exchange.  Splitting over a workspace with a reduction kernel per layer
+// took 12-20 us a layer on one ResNet-18/224 image (conv 7-11, reduction
+// 4-9).  Two CTAs fit an SM.  A 1x1 shortcut of the same input can share the
+// launch: clusters n1 .. run its tiles, on the centre-tap K blocks.
+//
+// The copy latency (about 1.5 us) bounds the K loop of these short tiles: with
+// three stages a K block took 0.46 us, so the ring takes up to six stages of
+// 128 channels or eight of 64 (a CTA then fills its SM), and no more than the
+// CTA has K blocks (a short CTA leaves room for the next launch's prologue).
+// Where the partials fit beside the stages they get their own room: then only
+// the peers' start has to be known before the exchange, a barrier that is
+// passed while the MMAs run, and one exposed barrier is left.
+// When no fault is armed nothing before this launch writes weights, and the
+// first stages' filters are fetched while the previous kernel still runs.
+//
+// 224 threads: two TMA producer warps (alternate stages), the MMA warp, four
+// epilogue warps (one per TMEM lane quadrant).  Every thread reaches both cluster barriers, also after a
+// wait that gave up (all waits are bounded); nothing remote is touched after
+// the second, so a CTA may then leave.
+constexpr int CL_NPROD = 2, CL_MMA_WARP = CL_NPROD, CL_EPI_WARP0 = CL_NPROD + 1;
+constexpr int CL_THREADS = 32 * (CL_EPI_WARP0 + 4);
+constexpr int CL_MAX_Z = 8;                              // portable cluster size
+template <int BN> struct ClTile {
+    static constexpr int MAX_STAGES = BN == 64 ? 8 : 6;
+    static constexpr int B_BYTES = BN * BK * 2, STAGE = A_BYTES + (BN + 16) * BK * 2;   // filters, carry-through rows
+    static constexpr int PITCH = BN + 4;                 // partial row: BN channels, the checksum column
+    static constexpr int TMEM = BN == 64 ? 128 : 256;    // accumulator columns (BN + 16) allocated
+    // Z partials of ceil(BM / Z) rows (at most BM + Z - 1 rows), beside the stages or in their place
+    static constexpr int PART = (BM + CL_MAX_Z - 1) * PITCH * 4;
+    static constexpr bool apart(int stages) { return 1024 + 144 + stages * STAGE + PART <= 227 * 1024; }
+    static constexpr size_t smem(int stages) {
+        return 1024 + 144 + (apart(stages) ? stages * STAGE + PART : stages * STAGE > PART ? stages * STAGE : PART);
+    }
+};
+
+__device__ __forceinline__ void st_cluster4(uint32_t addr, float x, float y, float z, float w) {
+    asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(x), "f"(y), "f"(z), "f"(w) : "memory");
+}
+__device__ __forceinline__ void st_cluster1(uint32_t addr, float x) {
+    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(x) : "memory");
+}
+
+template <int BN>
+__global__ void __launch_bounds__(CL_THREADS, 1)
+conv_tc_cluster_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ CUtensorMap bmap,
+                       const __grid_constant__ ConvArgs a, const __grid_constant__ TcGeom g, int nst) {
+    using T = ClTile<BN>;
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    // barriers, then the stages [nst][A | B | carry-through rows]
+    uint64_t *full = (uint64_t *)smem_raw;
+    uint64_t *empty = full + T::MAX_STAGES, *done = empty + T::MAX_STAGES;
+    uint32_t *tmem_holder = (uint32_t *)(done + 1);
+    static_assert(8 * (2 * T::MAX_STAGES + 1) + 4 <= 144, "barriers");
+    uint8_t *smem = smem_raw + ((1024u - ((smem_u32(smem_raw) + 144u) & 1023u)) & 1023u) + 144u;
+    const bool apart = T::apart(nst);
+    float *part = (float *)(smem + (apart ? nst * T::STAGE : 0));   // [Z][rows of this CTA][PITCH]
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int Z = g.splits, rank = (int)cluster_ctarank(), tile = (int)blockIdx.x / Z;
+    const int m0 = (tile / g.n_tiles) * BM, n_tile = tile % g.n_tiles, n0 = n_tile * BN;
+    const int kb_lo = min(g.n_kb, rank * g.kps), kb_hi = min(g.n_kb, kb_lo + g.kps);
+    const bool ct_here = g.ct_mode != CT_NONE_ && n_tile == 0;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < nst; ++s) {
+            mbar_init(smem_u32(&full[s]), 1);
+            mbar_init(smem_u32(&empty[s]), 1);
+        }
+        mbar_init(smem_u32(done), 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == CL_MMA_WARP) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_holder)),
+                     "r"((uint32_t)T::TMEM));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    }
+    if (warp >= CL_EPI_WARP0 && ct_here) {
+        // constant carry-through rows after each stage's filters: row 0 = coef, rows 1..15 = 0
+        const uint32_t coef2 = (uint32_t)g.coef_h | ((uint32_t)g.coef_h << 16);
+        for (int s = 0; s < nst; ++s) {
+            uint32_t *rows = (uint32_t *)(smem + s * T::STAGE + A_BYTES + T::B_BYTES);
+            for (int i = threadIdx.x - 32 * CL_EPI_WARP0; i < 16 * BK / 2; i += 128) rows[i] = (i < BK / 2) ? coef2 : 0u;
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmem = *tmem_holder;
+    bool mma_ok = false;
+    const int n_kb = kb_hi - kb_lo;
+    if (apart) cluster_arrive();                          // this CTA has started
+
+    if (warp < CL_NPROD) {
+        // ---------------- TMA producers: K blocks warp, warp + CL_NPROD, ... ----------------
+        // nst is a multiple of CL_NPROD or covers every K block, so a slot belongs to one warp
+        if (elect_one()) {
+            asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&amap) : "memory");
+            asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&bmap) : "memory");
+            const int nimg = m0 / g.PQ, rem = m0 % g.PQ;
+            const int w0 = (rem % g.Q) * g.stride - g.pad, h0 = (rem / g.Q) * g.stride - g.pad;
+            auto load_b = [&](int it) {
+                const int kb = kb_lo + it, s = it % nst;
+                const uint32_t fb = smem_u32(&full[s]);
+                mbar_arrive_expect_tx(fb, A_BYTES + T::B_BYTES);
+                tma_load_2d(smem_u32(smem + s * T::STAGE + A_BYTES), &bmap, fb,
+                            tap_of(kb / g.cpb, g.ctr_tap) * g.C + (kb % g.cpb) * BK, n0);
+            };
+            const bool early = a.weights_stable != 0;
+            if (early)
+                for (int it = warp; it < min(nst, n_kb); it += CL_NPROD) load_b(it);
+            pdl_wait();
+            bool ok = true;
+            int it = warp;
+            for (; it < n_kb; it += CL_NPROD) {
+                const int kb = kb_lo + it, s = it % nst;
+                if (!mbar_wait(smem_u32(&empty[s]), ((uint32_t)(it / nst) & 1u) ^ 1u, a.err, 1u)) { ok = false; break; }
+                if (!early || it >= nst) load_b(it);
+                const int tap = tap_of(kb / g.cpb, g.ctr_tap);
+                tma_load_im2col(smem_u32(smem + s * T::STAGE), &amap, smem_u32(&full[s]), (kb % g.cpb) * BK, w0, h0, nimg,
+                                (uint16_t)(tap % g.S), (uint16_t)(tap / g.S));
+            }
+            // a wait gave up: copies in flight land before the stages are reused
+            if (!ok)
+                for (int i = max(warp, it - nst / CL_NPROD * CL_NPROD); i < it; i += CL_NPROD)
+                    mbar_wait(smem_u32(&full[i % nst]), (uint32_t)(i / nst) & 1u, a.err, 2u);
+        }
+        __syncwarp();
+        pdl_wait();
+        pdl_trigger();
+    } else if (warp == CL_MMA_WARP) {
+        pdl_wait();
+        pdl_trigger();
+        // ---------------- MMA issuer ----------------
+        if (elect_one()) {
+            const uint32_t id_main = idesc_f16(BM, BN), id_ct = idesc_f16(BM, BN + 16);
+            for (int it = 0; it < n_kb; ++it) {
+                const int s = it % nst;
+                if (!mbar_wait(smem_u32(&full[s]), (uint32_t)(it / nst) & 1u, a.err, 2u)) break;
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                const uint64_t ad = smem_desc_sw128(smem_u32(smem + s * T::STAGE));
+                const uint64_t bd = smem_desc_sw128(smem_u32(smem + s * T::STAGE + A_BYTES));
+                const uint32_t id = ct_here && kb_lo + it < g.cpb ? id_ct : id_main;
+#pragma unroll
+                for (int k16 = 0; k16 < BK / 16; ++k16)
+                    umma_f16(tmem, ad + 2 * k16, bd + 2 * k16, id, (it > 0 || k16) ? 1u : 0u);
+                umma_commit(smem_u32(&empty[s]));
+            }
+            umma_commit(smem_u32(done));                  // every MMA of this CTA has completed
+        }
+        __syncwarp();
+    } else {
+        pdl_wait();
+        pdl_trigger();
+        // this CTA's MMAs complete
+        mma_ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(done), 0u, a.err, 4u));
+    }
+    __syncwarp();
+    if (!apart) cluster_arrive();
+    cluster_wait();                                       // every CTA's partial buffer may be written
+    const int rows = (BM + Z - 1) / Z;
+    if (warp >= CL_EPI_WARP0 && mma_ok) {
+        // ---------------- partial rows to their owners ----------------
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const int row = (warp & 3) * 32 + lane, owner = row / rows;
+        const uint32_t trow = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+        const bool any = kb_lo < kb_hi, ct = ct_here && kb_lo < min(g.cpb, kb_hi);
+        const uint32_t dst = mapa_shared(smem_u32(part + (rank * rows + row - owner * rows) * T::PITCH), (uint32_t)owner);
+#pragma unroll
+        for (int c = 0; c < BN; c += 32) {
+            uint32_t t0[16], t1[16];
+            float v[32];
+            tmem_ld16_nw(trow + c, t0);
+            tmem_ld16_nw(trow + c + 16, t1);
+            tmem_wait_ld();
+            tmem_done16(t0, v);
+            tmem_done16(t1, v + 16);
+#pragma unroll
+            for (int i = 0; i < 32; i += 4) {
+                if (any) st_cluster4(dst + (uint32_t)(c + i) * 4u, v[i], v[i + 1], v[i + 2], v[i + 3]);
+                else st_cluster4(dst + (uint32_t)(c + i) * 4u, 0.f, 0.f, 0.f, 0.f);
+            }
+        }
+        uint32_t r;
+        tmem_ld1_nw(trow + BN, r);                        // undefined unless ct: not used then
+        tmem_wait_ld();
+        const float cv = tmem_done(r);
+        st_cluster1(dst + BN * 4u, ct ? cv : 0.f);
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncwarp();
+    cluster_arrive();
+    // residual and bias of this thread's first items, in flight during the barrier
+    const int r_lo = rank * rows, r_n = min(min(BM, r_lo + rows), g.M - m0) - r_lo;
+    const __half *res = static_cast<const __half *>(a.res);
+    constexpr int U = 2;                                  // items (8 channels of a row) in flight per thread
+    uint4 rs[U];
+    float4 b0[U], b1[U];
+    auto load_items = [&](int e0) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int e = min(e0 + u * CL_THREADS, r_n * (BN / 8) - 1);
+            const int m = m0 + r_lo + e / (BN / 8), k0 = n0 + (e % (BN / 8)) * 8;
+            b0[u] = __ldg(reinterpret_cast<const float4 *>(a.bias + k0));
+            b1[u] = __ldg(reinterpret_cast<const float4 *>(a.bias + k0 + 4));
+            rs[u] = res ? __ldg(reinterpret_cast<const uint4 *>(res + (size_t)m * g.K + k0)) : make_uint4(0u, 0u, 0u, 0u);
+        }
+    };
+    if ((int)threadIdx.x < r_n * (BN / 8)) load_items(threadIdx.x);
+    cluster_wait();                                       // the partials of this CTA's rows are here
+    if (warp == CL_MMA_WARP) {
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)T::TMEM));
+    }
+    {
+        // ---------------- rows of this CTA: add the partials, epilogue ----------------
+        const FaultDelta &fd = a.fd;
+        const __half *x = static_cast<const __half *>(a.x);
+        auto fault_src = [&](int m) -> float {
+            const int ni = m / g.PQ, rm = m % g.PQ;
+            const int h = (rm / g.Q) * g.stride + fd.r - g.pad, w = (rm % g.Q) * g.stride + fd.s - g.pad;
+            if (h < 0 || h >= a.H || w < 0 || w >= a.W) return 0.f;
+            const size_t pix = ((size_t)ni * a.H + h) * a.W + w;
+            if (fd.cin < g.C) return ldh(x, pix * g.C + fd.cin);
+            return a.cs_in ? ldh(static_cast<const __half *>(a.cs_in), pix) : 0.f;
+        };
+        for (int e0 = threadIdx.x; e0 < r_n * (BN / 8); e0 += U * CL_THREADS) {
+            if (e0 != (int)threadIdx.x) load_items(e0);
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int e = e0 + u * CL_THREADS;
+                if (e >= r_n * (BN / 8)) break;
+                const int r = e / (BN / 8), c = (e % (BN / 8)) * 8, m = m0 + r_lo + r, k0 = n0 + c;
+                float v[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+                for (int z = 0; z < CL_MAX_Z; ++z)
+                    if (z < Z) {
+                        const float4 *p = reinterpret_cast<const float4 *>(part + (z * rows + r) * T::PITCH + c);
+                        const float4 p0 = p[0], p1 = p[1];
+                        v[0] += p0.x; v[1] += p0.y; v[2] += p0.z; v[3] += p0.w;
+                        v[4] += p1.x; v[5] += p1.y; v[6] += p1.z; v[7] += p1.w;
+                    }
+                const float bias[8] = {b0[u].x, b0[u].y, b0[u].z, b0[u].w, b1[u].x, b1[u].y, b1[u].z, b1[u].w};
+                const __half2 *rh = reinterpret_cast<const __half2 *>(&rs[u]);
+                const float fsrc = fd.active && fd.kout >= k0 && fd.kout < k0 + 8 ? fault_src(m) : 0.f;
+                uint32_t pk[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const float2 rf = __half22float2(rh[i]);
+                    float o[2] = {v[2 * i] + bias[2 * i], v[2 * i + 1] + bias[2 * i + 1]};
+#pragma unroll
+                    for (int j = 0; j < 2; ++j) {
+                        if (fd.active && fd.kout == k0 + 2 * i + j) o[j] += fd.dv * fsrc;
+                        if (res) o[j] += j ? rf.y : rf.x;
+                    }
+                    pk[i] = cvt_h2(o[0], o[1], a.relu != 0);
+                }
+                *reinterpret_cast<uint4 *>(static_cast<__half *>(a.y) + (size_t)m * g.K + k0) =
+                    make_uint4(pk[0], pk[1], pk[2], pk[3]);
+            }
+        }
+        if (a.cs_out != nullptr && n_tile == 0)
+            for (int r = threadIdx.x; r < r_n; r += CL_THREADS) {
+                const int m = m0 + r_lo + r;
+                const int ni = m / g.PQ, rm = m % g.PQ;
+                const CsIn csv = load_cs_inputs(a, g, m, ni, rm / g.Q, rm % g.Q);
+                float ctv = 0.f;
+                for (int z = 0; z < Z; ++z) ctv += part[(z * rows + r) * T::PITCH + BN];
+                store_checksum_pre(ctv, csv, a, g, m, fd.active && fd.kout == g.K ? fault_src(m) : 0.f);
+            }
     }
 }
 
@@ -1959,8 +2095,7 @@ bool load_encoders() {
 
 template <int BN, int STAGES, int SUB>
 size_t smem_bytes() {
-    return 1024 + (size_t)STAGES * SUB * (A_BYTES + (BN + 16) * BK * 2) + 16 * BK * 2 + 2 * BM * 4 +
-           8 * (2 * STAGES + 6) + 16 + 16 + 4 * BIAS_SMEM;
+    return 1024 + (size_t)STAGES * SUB * (A_BYTES + (BN + 16) * BK * 2) + 8 * (2 * STAGES + 4) + 16 + 16 + 4 * BIAS_SMEM;
 }
 
 uint16_t coef_half_bits(float c) {
@@ -1988,8 +2123,7 @@ struct TcPlan {
     TcGeom g;
     int BN, n_tiles, sms;
     size_t smem;
-    CUtensorMap bmap_pair;       // N = 256 over CTA pairs: 128-row weight halves
-    CUtensorMap bmap_pair64;     // 128-channel half tiles: 64-row weight quarters
+    CUtensorMap bmap64, bmap128; // weight boxes of 64 and 128 filters (bmap128: K >= 128)
     int pair_clusters;           // resident CTA pairs (0: no pair variant)
     size_t pair_smem;
     // launches that also run a shortcut: splits of the shortcut's items
@@ -2021,7 +2155,7 @@ TcPlan *tc_plan_create(const ConvArgs &a, int max_batch, const void *w_dev, cons
     g.cpb = a.C / BK;
     g.n_kb = a.R * a.S * g.cpb;
     g.ctr_tap = ((a.R - 1) / 2) * a.S + (a.S - 1) / 2;
-    g.ct_mode = a.role != CT_ROLE_CT ? CT_NONE_ : (pl->BN + 16 <= 256 && pl->n_tiles == 1 ? CT_MERGED : CT_SEPARATE);
+    g.ct_mode = a.role == CT_ROLE_CT ? CT_COLUMN : CT_NONE_;
     g.tmem_cols = 512;
     g.n_tiles = pl->n_tiles;
     g.coef_h = coef_half_bits(a.coef);
@@ -2048,7 +2182,21 @@ TcPlan *tc_plan_create(const ConvArgs &a, int max_batch, const void *w_dev, cons
                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) { if (why) *why = "weight tensor map"; delete pl; return nullptr; }
-    cudaError_t e;
+    for (int rows : {64, 128}) {
+        if (rows > a.K) continue;
+        cuuint32_t box_r[2] = {BK, (cuuint32_t)rows};
+        r = g_encode_tiled(rows == 64 ? &pl->bmap64 : &pl->bmap128, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2,
+                           const_cast<void *>(w_dev), bdim, bstr, box_r, bes, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                           CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+        if (r != CUDA_SUCCESS) { if (why) *why = "weight tensor map"; delete pl; return nullptr; }
+    }
+    cudaError_t e = cudaFuncSetAttribute(conv_tc_cluster_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)ClTile<64>::smem(ClTile<64>::MAX_STAGES));
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(conv_tc_cluster_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)ClTile<128>::smem(ClTile<128>::MAX_STAGES));
+    if (e != cudaSuccess) { if (why) *why = "shared memory attribute"; delete pl; return nullptr; }
     if (pl->BN == 64) {
         pl->smem = smem_bytes<64, 4, 2>();
         e = cudaFuncSetAttribute(conv_tc_kernel<64, 4, 2, 4, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -2060,10 +2208,6 @@ TcPlan *tc_plan_create(const ConvArgs &a, int max_batch, const void *w_dev, cons
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(conv_tc_kernel<128, 3, 2, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)pl->smem);
-    } else {
-        pl->smem = smem_bytes<256, 4, 1>();
-        e = cudaFuncSetAttribute(conv_tc_kernel<256, 4, 1, 1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)pl->smem);
     }
     if (e != cudaSuccess) { if (why) *why = "shared memory attribute"; delete pl; return nullptr; }
     // N = 256 over CTA pairs (cta_group::2): each CTA copies half of the
@@ -2071,15 +2215,6 @@ TcPlan *tc_plan_create(const ConvArgs &a, int max_batch, const void *w_dev, cons
     // kernel: on CTA pairs they ran 10-30% slower, measured.)
     pl->pair_clusters = 0;
     if (pl->BN == 256) {
-        cuuint32_t box_h[2] = {BK, (cuuint32_t)BM};
-        r = g_encode_tiled(&pl->bmap_pair, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<void *>(w_dev), bdim, bstr,
-                           box_h, bes, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                           CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-        cuuint32_t box_q[2] = {BK, (cuuint32_t)(BM / 2)};
-        if (r == CUDA_SUCCESS)
-            r = g_encode_tiled(&pl->bmap_pair64, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<void *>(w_dev), bdim,
-                               bstr, box_q, bes, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
         pl->pair_smem = pair_smem_bytes();
         cudaError_t pe = cudaSuccess;
         for (auto kern : {conv_tc_pair_kernel<false, false>, conv_tc_pair_kernel<true, false>,
@@ -2180,22 +2315,90 @@ ScSplit cached_split(TcPlan *pl, int batch, int n2, F &&make) {
     return sp;
 }
 
+// Estimated microseconds of a layer, for the choice between the persistent
+// kernels (whole-K tiles) and a K split over clusters.  Per K block and CTA:
+// 0.35 us for 128 x 128 tiles and 0.31 us for a CTA pair's (clock traces,
+// shared-memory bound), 0.22 us for 128 x 64; per launch about 3 us of copy
+// and store latency, 6 us with the epilogue of a 256 x 256 tile.  Measured at
+// the sizes where the choice falls, either side of the line, within 15%.
+struct ClPick {
+    int BN, Z;                   // tile width and cluster size (0: persistent kernel)
+    double us;
+};
+constexpr double KB_US_64 = 0.20, KB_US_128 = 0.38, KB_US_PAIR = 0.31;
+
+// Clusters of Z CTAs that are resident together (a cluster stays inside one
+// GPC, so sizes that do not divide its SMs leave some of them idle).
+struct ClResident {
+    int n[2][CL_MAX_Z + 1];
+};
+const ClResident &cluster_resident() {
+    static const ClResident r = [] {
+        ClResident t;
+        for (int v = 0; v < 2; ++v)
+            for (int Z = 0; Z <= CL_MAX_Z; ++Z) {
+                t.n[v][Z] = 0;
+                if (Z == 0) continue;
+                cudaLaunchConfig_t cfg = {};
+                cfg.gridDim = dim3(Z * 64);
+                cfg.blockDim = dim3(CL_THREADS);
+                cfg.dynamicSmemBytes = v ? ClTile<128>::smem(ClTile<128>::MAX_STAGES) : ClTile<64>::smem(ClTile<64>::MAX_STAGES);
+                cudaLaunchAttribute at[1];
+                at[0].id = cudaLaunchAttributeClusterDimension;
+                at[0].val.clusterDim.x = Z;
+                at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+                cfg.attrs = at;
+                cfg.numAttrs = 1;
+                int n = 0;
+                const cudaError_t e = v ? cudaOccupancyMaxActiveClusters(&n, conv_tc_cluster_kernel<128>, &cfg)
+                                        : cudaOccupancyMaxActiveClusters(&n, conv_tc_cluster_kernel<64>, &cfg);
+                if (e != cudaSuccess) cudaGetLastError();
+                else t.n[v][Z] = n;
+            }
+        return t;
+    }();
+    return r;
+}
+
+ClPick cluster_pick(int m_tiles, int K, int n_kb) {
+    const ClResident &res = cluster_resident();
+    ClPick best{0, 0, 1e30};
+    for (int BN = 64; BN <= 128 && BN <= K; BN *= 2)
+        for (int Z = 1; Z <= CL_MAX_Z && Z <= n_kb; ++Z) {
+            const int kps = (n_kb + Z - 1) / Z;
+            if (Z > 1 && (Z - 1) * kps >= n_kb) continue;        // an empty share
+            const long long cls = (long long)m_tiles * (K / BN), fit = res.n[BN == 128][Z];
+            if (fit < 1) continue;
+            const double rounds = (double)((cls + fit - 1) / fit);
+            const double us = 3.0 + 0.15 * Z + rounds * (2.5 + kps * (BN == 64 ? KB_US_64 : KB_US_128));
+            if (us < best.us) best = ClPick{BN, Z, us};
+        }
+    return best;
+}
+double persistent_us(const TcPlan *pl, const TcGeom &g, bool pairs) {
+    if (pairs) {
+        const int items = ((g.m_tiles + 1) / 2) * g.n_tiles, P = pl->pair_clusters, rem = items % P;
+        const double rounds = items / P + (rem == 0 ? 0.0 : 2 * rem <= P ? 0.92 : 1.0);
+        return 6.0 + rounds * g.n_kb * KB_US_PAIR;
+    }
+    const int tiles = g.m_tiles * g.n_tiles;
+    return 5.5 + (double)((tiles + pl->sms - 1) / pl->sms) * g.n_kb * (pl->BN == 64 ? 0.22 : 0.35);
+}
+
 // Geometry of one launch of plan pl: output tiles, K split, CTA pairs.
-TcGeom tc_launch_geom(const ConvArgs &a, const TcPlan *pl, bool *pairs) {
+TcGeom tc_launch_geom(const ConvArgs &a, const TcPlan *pl, bool *pairs, ClPick *cl) {
     TcGeom g = pl->g;
     g.M = a.N * a.P * a.Q;
     g.m_tiles = (g.M + BM - 1) / BM;
-    const int tiles = g.m_tiles * g.n_tiles;
-    // split K when the output tiles leave most SMs idle (at least 4 K blocks
-    // per split; about half the SMs busy: more splits cost more in partial
-    // sums than they gain, measured on 4-16 image batches)
-    g.ws_ld = (g.K + 1 + 3) & ~3;
-    g.splits = (a.K % 8 == 0) ? splitk_choose(tiles, g.n_kb, 4, pl->sms / 2, g.M, g.ws_ld, a.ws ? a.ws_bytes : 0) : 1;
-    g.kps = (g.n_kb + g.splits - 1) / g.splits;
+    g.splits = 1;
+    g.kps = g.n_kb;
     g.sc_items = 0;
     g.sc_s0 = 0;
     g.sc_x = 0;
-    *pairs = pl->pair_clusters > 0 && g.splits == 1 && g.m_tiles >= 2;
+    *pairs = pl->pair_clusters > 0 && g.m_tiles >= 2;
+    // N = 256 plans have no persistent kernel on single CTAs
+    *cl = cluster_pick(g.m_tiles, g.K, g.n_kb);
+    if (cl->Z > 0 && (pl->BN != 256 || *pairs) && cl->us > 0.85 * persistent_us(pl, g, *pairs)) cl->Z = 0;
     return g;
 }
 
@@ -2206,10 +2409,11 @@ bool tc_shortcut_fits(const ConvArgs &a, const void *plan, const void *plan2) {
     const TcPlan *pl2 = static_cast<const TcPlan *>(plan2);
     if (!pl || !pl2) return false;
     bool pairs = false;
-    const TcGeom g = tc_launch_geom(a, pl, &pairs);
+    ClPick cl;
+    tc_launch_geom(a, pl, &pairs, &cl);
     // both layers whole (unsplit) N = 128 tiles on single CTAs, or N = 256
     // tiles on CTA pairs; the shortcut's K blocks are the centre tap's
-    return g.splits == 1 && pl2->BN == pl->BN && pl2->n_tiles == pl->n_tiles && pl2->g.n_kb == pl->g.cpb &&
+    return cl.Z == 0 && pl2->BN == pl->BN && pl2->n_tiles == pl->n_tiles && pl2->g.n_kb == pl->g.cpb &&
            ((pl->BN == 128 && !pairs) || (pl->BN == 256 && pairs));
 }
 
@@ -2219,7 +2423,23 @@ cudaError_t launch_conv_tc(const ConvArgs &a, const void *plan, cudaStream_t st,
     const TcPlan *pl2 = static_cast<const TcPlan *>(plan2);
     if (merged) *merged = false;
     bool pairs = false;
-    TcGeom g = tc_launch_geom(a, pl, &pairs);
+    ClPick cl;
+    TcGeom g = tc_launch_geom(a, pl, &pairs, &cl);
+    if (n_kernels) *n_kernels = 1;
+    if (cl.Z > 0) {
+        g.splits = cl.Z;
+        g.kps = (g.n_kb + cl.Z - 1) / cl.Z;
+        g.n_tiles = g.K / cl.BN;
+        const dim3 grid(g.m_tiles * g.n_tiles * cl.Z);
+        const int nst = std::min(g.kps, cl.BN == 64 ? ClTile<64>::MAX_STAGES : ClTile<128>::MAX_STAGES);
+        if (cl.BN == 64)
+            pdl_launch_cluster(conv_tc_cluster_kernel<64>, grid, CL_THREADS, ClTile<64>::smem(nst), st, cl.Z, pl->amap,
+                               pl->bmap64, a, g, nst);
+        else
+            pdl_launch_cluster(conv_tc_cluster_kernel<128>, grid, CL_THREADS, ClTile<128>::smem(nst), st, cl.Z, pl->amap,
+                               pl->bmap128, a, g, nst);
+        return cudaGetLastError();
+    }
     const int tiles = g.m_tiles * g.n_tiles;
     // a 1x1 shortcut of the same input (a2, plan2) joins this launch when the
     // tiles allow; the caller launches it on its own otherwise
@@ -2228,14 +2448,13 @@ cudaError_t launch_conv_tc(const ConvArgs &a, const void *plan, cudaStream_t st,
     if (sc) {
         g2.M = g.M;
         g2.m_tiles = g.m_tiles;
-        g2.ws_ld = g.ws_ld;
         g2.splits = 1;
         g2.kps = g2.n_kb;
         g2.t_first = g2.units = 0;
         g2.sc_items = g2.sc_s0 = g2.sc_x = 0;
     }
     const ConvArgs &b = sc ? *a2 : a;
-    const CUtensorMap &bm2 = sc ? (pairs ? pl2->bmap_pair : pl2->bmap) : (pairs ? pl->bmap_pair : pl->bmap);
+    const CUtensorMap &bm2 = sc ? (pairs ? pl2->bmap128 : pl2->bmap) : (pairs ? pl->bmap128 : pl->bmap);
     if (pairs) {
         // tiles over CTA pairs: 256 pixels x 256 channels per pair
         const int items = ((g.m_tiles + 1) / 2) * g.n_tiles;
@@ -2264,18 +2483,18 @@ cudaError_t launch_conv_tc(const ConvArgs &a, const void *plan, cudaStream_t st,
         }
         if (halves && sc)
             pdl_launch_cluster(conv_tc_pair_kernel<true, true>, dim3(2 * ncl), PR_THREADS, pl->pair_smem, st, 2,
-                               pl->amap, pl->bmap_pair, pl->bmap_pair64, a, g, bm2, b, g2);
+                               pl->amap, pl->bmap128, pl->bmap64, a, g, bm2, b, g2);
         else if (sc)
             pdl_launch_cluster(conv_tc_pair_kernel<false, true>, dim3(2 * ncl), PR_THREADS, pl->pair_smem, st, 2,
-                               pl->amap, pl->bmap_pair, pl->bmap_pair64, a, g, bm2, b, g2);
+                               pl->amap, pl->bmap128, pl->bmap64, a, g, bm2, b, g2);
         else if (halves)
             pdl_launch_cluster(conv_tc_pair_kernel<true, false>, dim3(2 * ncl), PR_THREADS, pl->pair_smem, st, 2,
-                               pl->amap, pl->bmap_pair, pl->bmap_pair64, a, g, bm2, b, g2);
+                               pl->amap, pl->bmap128, pl->bmap64, a, g, bm2, b, g2);
         else
             pdl_launch_cluster(conv_tc_pair_kernel<false, false>, dim3(2 * ncl), PR_THREADS, pl->pair_smem, st, 2,
-                               pl->amap, pl->bmap_pair, pl->bmap_pair64, a, g, bm2, b, g2);
+                               pl->amap, pl->bmap128, pl->bmap64, a, g, bm2, b, g2);
     } else {
-        const int items = tiles * g.splits;
+        const int items = tiles;
         const int n2 = sc ? g2.m_tiles * g2.n_tiles : 0;
         const int ncl = items + n2 < pl->sms ? items + n2 : pl->sms;
         dim3 grid(ncl);
@@ -2288,25 +2507,19 @@ cudaError_t launch_conv_tc(const ConvArgs &a, const void *plan, cudaStream_t st,
             });
             g.sc_s0 = sp.s0;
             g.sc_x = sp.x;
-            pdl_launch(conv_tc_kernel<128, 3, 2, 1, true>, grid, tc_threads(128, 3), pl->smem, st, pl->amap, pl->bmap,
+            pdl_launch(conv_tc_kernel<128, 3, 2, 1, true>, grid, tc_threads(3), pl->smem, st, pl->amap, pl->bmap,
                        a, g, bm2, b, g2);
         } else if (pl->BN == 64) {
-            pdl_launch(conv_tc_kernel<64, 4, 2, 4, false>, grid, tc_threads(64, 4), pl->smem, st, pl->amap, pl->bmap, a,
+            pdl_launch(conv_tc_kernel<64, 4, 2, 4, false>, grid, tc_threads(4), pl->smem, st, pl->amap, pl->bmap, a,
                        g, bm2, b, g2);
-        } else if (pl->BN == 128) {
-            pdl_launch(conv_tc_kernel<128, 3, 2, 1, false>, grid, tc_threads(128, 3), pl->smem, st, pl->amap, pl->bmap,
-                       a, g, bm2, b, g2);
         } else {
-            pdl_launch(conv_tc_kernel<256, 4, 1, 1, false>, grid, tc_threads(256, 4), pl->smem, st, pl->amap, pl->bmap,
+            pdl_launch(conv_tc_kernel<128, 3, 2, 1, false>, grid, tc_threads(3), pl->smem, st, pl->amap, pl->bmap,
                        a, g, bm2, b, g2);
         }
     }
-    cudaError_t e = cudaGetLastError();
-    if (n_kernels) *n_kernels = 1;
+    const cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess && merged) *merged = sc;
-    if (e != cudaSuccess || g.splits == 1) return e;
-    if (n_kernels) *n_kernels = 2;
-    return launch_splitk_reduce(a, g.splits, g.ws_ld, true, st);
+    return e;
 }
 
 bool tc_small_supported(int C, int K, int R, int S, int stride, int pad) {

@@ -970,6 +970,7 @@ ct_status infer_impl(ct_model *m, const float *input, int batch, float *logits, 
         a.stride = d.stride; a.pad = d.pad; a.P = l.P; a.Q = l.Q;
         a.role = l.role; a.relu = d.relu; a.coef = l.coef; a.err = m->d_err;
         a.ws = m->ws; a.ws_bytes = SPLITK_WS_BYTES; a.sk_flags = m->sk_flags;
+        a.weights_stable = !armed;       // a fault's bit flips are kernels of this inference
         const bool wfault = armed && m->f_kind == CT_BUF_WEIGHT && m->f_layer == (int)li;
         if (wfault) {
             wf = resolve_weight_fault(m, l, m->f_elem, m->f_bit);
@@ -1062,7 +1063,7 @@ ct_status infer_impl(ct_model *m, const float *input, int batch, float *logits, 
             a.N = batch; a.H = a.W = 1; a.C = l.n_in; a.K = l.n_out; a.R = a.S = 1;
             a.stride = 1; a.pad = 0; a.P = a.Q = 1;
             a.role = m->protect ? CT_ROLE_CT : CT_ROLE_NONE; a.relu = d.relu; a.coef = l.coef;
-            a.err = m->d_err; a.cs_rowsum = l.n_cs;
+            a.err = m->d_err; a.cs_rowsum = l.n_cs; a.weights_stable = !armed;
             a.ws = m->ws; a.ws_bytes = SPLITK_WS_BYTES;
             const double flops = 2.0 * batch * (double)l.n_in * l.n_out;
             int nk = 1;

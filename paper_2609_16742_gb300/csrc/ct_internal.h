@@ -45,6 +45,8 @@ struct ConvArgs {
                           // is the sum of cs_in[m * cs_rowsum .. m * cs_rowsum + cs_rowsum)
     float *ws;            // split-K workspace (null: never split)
     size_t ws_bytes;
+    int weights_stable;   // nothing earlier in the stream that may still run writes this layer's
+                          // weights: they may be read before the previous kernel ends
     uint32_t *sk_flags;   // SK_FLAGS words, 0 between launches (partial sums exchanged between CTAs)
     const void *x2;       // first layer only: images n >= n_split are image n - n_split of x2
     int n_split;          // (null x2: every image comes from x)
@@ -185,7 +187,7 @@ inline cudaError_t pdl_launch_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 
 
 // kernel launchers; each returns cudaGetLastError()
 // conv launchers report in *n_kernels (may be null) how many kernels they
-// launched: 2 when K is split (the conv kernel and the split-K reduction)
+// launched: 2 when the CUDA-core kernel splits K (it and the reduction)
 cudaError_t launch_conv_simt(const ConvArgs &a, bool half, cudaStream_t st, int *n_kernels);
 // a2 / tc_plan2: a 1x1 shortcut convolution of the same input at the same
 // stride whose pixel is the first layer's centre tap; it runs in the same

@@ -1,11 +1,11 @@
-// Split-K for convolutions whose output tiles cannot fill the GPU (small
-// batches: re-execution of flagged images, deep layers with few pixels, FC
-// layers run as 1x1 convolutions).  The conv kernels then write FP32 partial
-// sums of their K range to a workspace [splits][M][ws_ld] (data channels in
-// columns 0..K-1, the carry-through partial, already scaled by coef, in
-// column K), and this kernel adds the partials in split order and applies
-// the epilogue of Sec. II-A to data and checksum alike: bias (0 on the
-// checksum), fault delta, residual, ReLU, store in the storage type.
+// Split-K for the CUDA-core convolutions of conv_simt.cu whose output tiles
+// cannot fill the GPU (small batches, deep layers with few pixels).  The conv
+// kernel then writes FP32 partial sums of its K ranges to a workspace
+// [splits][M][ws_ld] (data channels in columns 0..K-1, the carry-through
+// partial, already scaled by coef, in column K), and this kernel adds the
+// partials in split order and applies the epilogue of Sec. II-A to data and
+// checksum alike: bias (0 on the checksum), fault delta, residual, ReLU,
+// store in the storage type.
 #include "ct_internal.h"
 
 namespace ct {
@@ -111,9 +111,7 @@ __global__ void splitk_reduce_kernel(const ConvArgs a, int splits, int ws_ld) {
                 for (int u = 0; u < 4; ++u) ctv += c[u];
             }
             float cin = 0.f;
-            if (a.cs_in && a.cs_rowsum > 0) {            // FC layer: every incoming checksum feature
-                for (int i = 0; i < a.cs_rowsum; ++i) cin += ld<T>(a.cs_in, (size_t)m * a.cs_rowsum + i);
-            } else if (a.cs_in) {
+            if (a.cs_in) {
                 const int hc = p * a.stride + (a.R - 1) / 2 - a.pad, wc = q * a.stride + (a.S - 1) / 2 - a.pad;
                 if (hc >= 0 && hc < a.H && wc >= 0 && wc < a.W) cin = ld<T>(a.cs_in, ((size_t)n * a.H + hc) * a.W + wc);
             }

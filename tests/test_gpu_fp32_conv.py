@@ -15,7 +15,7 @@ from _gpu import TOL, ct, run, same_class
 pytestmark = pytest.mark.gpu
 
 
-def net_of(C, K, k, stride, H, cin=3, depthwise=False, residual=False):
+def net_of(C, K, k, stride, H, cin=3, depthwise=False, residual=False, prec="fp32"):
     Ly = synth.Layer
     L = [Ly("conv", 0, 1, cin=cin, cout=C, k=3, pad=1, relu=True)]
     s = 1
@@ -29,7 +29,7 @@ def net_of(C, K, k, stride, H, cin=3, depthwise=False, residual=False):
     L.append(Ly("conv", s, s + 1, cin=C, cout=K, k=k, stride=stride, pad=k // 2, relu=True))
     L.append(Ly("gap", s + 1, s + 2))
     L.append(Ly("fc", s + 2, s + 3, cin=K, cout=10, final=True))
-    wl = synth.Workload("edge", L, (cin, H, H), 10, 1, "fp32", 7, "normal")
+    wl = synth.Workload("edge", L, (cin, H, H), 10, 1, prec, 7, "normal")
     return wl, synth.make_params(L, 7), s
 
 
@@ -43,7 +43,7 @@ def check(wl, params, batch, sel, fault=None):
     assert ct().ct_device_error(m) == 0
     f = None if fault is None else oracle.Fault(*fault)
     o = oracle.forward(net, x[sel], f, keep=fault is None)
-    tol = TOL["fp32"]
+    tol = TOL[wl.precision]
     for j, i in enumerate(sel):
         ref = np.append(o["logits"][j], o["S"][j])
         got = np.append(lg[i], S[i])

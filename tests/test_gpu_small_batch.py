@@ -1,0 +1,58 @@
+"""FP16 layers with few output tiles (K split over a cluster of CTAs) and FC
+layers at the edges of their tiles, against the oracle: pixels that do not
+fill a tile, cluster sizes that do not divide its rows, every tile width,
+residuals, shortcuts, faults in stored and implicit weights, hidden FC layers
+on the tensor cores and on the CUDA cores."""
+import numpy as np
+import pytest
+
+import synth
+from test_gpu_fp32_conv import check, net_of
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("C,K,k,stride,H,batch", [
+    (64, 64, 3, 1, 8, 1),       # 64 channels, half a tile of pixels
+    (64, 128, 3, 2, 15, 2),     # 128 channels, 128 pixels exactly
+    (128, 256, 3, 1, 9, 3),     # 243 pixels
+    (256, 512, 3, 1, 7, 1),     # 49 pixels, 36 K blocks
+    (512, 512, 3, 1, 4, 5),     # 72 K blocks
+    (512, 256, 1, 1, 5, 2),     # 8 K blocks
+    (64, 256, 1, 2, 14, 1),     # one K block: nothing to split
+])
+def test_few_tiles_match_oracle(C, K, k, stride, H, batch):
+    wl, p, _ = net_of(C, K, k, stride, H, prec="fp16")
+    check(wl, p, batch, sorted({0, batch - 1}))
+
+
+@pytest.mark.parametrize("C,H,batch", [(64, 9, 1), (256, 6, 2)])
+def test_residual_block_matches_oracle(C, H, batch):
+    wl, p, _ = net_of(C, 128, 1, 1, H, residual=True, prec="fp16")
+    check(wl, p, batch, sorted({0, batch - 1}))
+
+
+def test_faults_match_oracle():
+    C, K, batch = 64, 128, 2
+    wl, p, _ = net_of(C, K, 3, 1, 10, prec="fp16")
+    Ct = C + 1
+    for f in [(0, 1, (5 * Ct + 3) * 9 + 4, 13), (0, 1, (9 * Ct + C) * 9 + 4, 13), (0, 1, (K * Ct + 2) * 9 + 4, 13),
+              (0, 1, (K * Ct + C) * 9 + 0, 12), (0, 1, (77 * Ct + 63) * 9 + 8, 13), (1, 1, 3 * 100 + 5, 13),
+              (1, 1, C * 100 + 7, 13)]:
+        check(wl, p, batch, [0, batch - 1], f)
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp16"])
+@pytest.mark.parametrize("C,H,hidden,classes,batch", [
+    (6, 5, 33, 10, 1),          # 150 inputs: rows not 16-byte aligned
+    (16, 6, 40, 3, 33),         # 576 inputs, one image and one neuron past a tile
+    (64, 8, 256, 1000, 70),     # 4096 inputs: tensor cores (FP16), K split
+    (64, 2, 128, 65, 2),
+])
+def test_fc_layers_match_oracle(prec, C, H, hidden, classes, batch):
+    Ly = synth.Layer
+    L = [Ly("conv", 0, 1, cin=3, cout=C, k=3, pad=1, relu=True),
+         Ly("fc", 1, 2, cin=C * H * H, cout=hidden, relu=True),
+         Ly("fc", 2, 3, cin=hidden, cout=classes, final=True)]
+    wl = synth.Workload("fc", L, (3, H, H), classes, 1, prec, 11, "normal")
+    check(wl, synth.make_params(L, 11), batch, sorted({0, batch // 2, batch - 1}))
