@@ -68,6 +68,10 @@ class FaultDesc(ctypes.Structure):
                 ("bit", ctypes.c_int32)]
 
 
+_FAULT_DTYPE = np.dtype([("kind", np.int32), ("layer", np.int32), ("element", np.int64), ("bit", np.int32)], align=True)
+assert _FAULT_DTYPE.itemsize == ctypes.sizeof(FaultDesc)
+
+
 class BuildOpts(ctypes.Structure):
     _fields_ = [("precision", ctypes.c_int32), ("protect", ctypes.c_int32),
                 ("ds_mode", ctypes.c_int32), ("device", ctypes.c_int32),
@@ -329,11 +333,14 @@ def ct_campaign_batched(m: Model, input_dev, batch: int, faults, S_dev, top1_dev
     """Many faults in one launch.  faults: rows (kind, layer, element, bit);
     outputs [n_faults, batch] device tensors (float32, int32, uint8)."""
     f = np.asarray(faults, dtype=np.int64).reshape(-1, 4)
-    arr = (FaultDesc * max(len(f), 1))()
-    for i, (kind, layer, el, bit) in enumerate(f.tolist()):
-        arr[i] = FaultDesc(kind, layer, el, bit)
-    _check(lib().ct_campaign_batched(m.handle, _ptr(input_dev), batch, arr, len(f), _ptr(S_dev), _ptr(top1_dev),
-                                     _ptr(flag_dev), _stream(stream)), "ct_campaign_batched")
+    # the records of FaultDesc, filled column by column (a Python loop over
+    # 2,048 faults took 0.85 ms); 32-bit fields wrap as ctypes' do
+    arr = np.zeros(max(len(f), 1), dtype=_FAULT_DTYPE)
+    for j, name in enumerate(_FAULT_DTYPE.names):
+        arr[name][:len(f)] = f[:, j]
+    _check(lib().ct_campaign_batched(m.handle, _ptr(input_dev), batch,
+                                     arr.ctypes.data_as(ctypes.POINTER(FaultDesc)), len(f), _ptr(S_dev),
+                                     _ptr(top1_dev), _ptr(flag_dev), _stream(stream)), "ct_campaign_batched")
 
 
 def ct_reexecute_noalloc(m: Model, input_dev, batch: int, flag_dev, logits_dev, S_dev=None,

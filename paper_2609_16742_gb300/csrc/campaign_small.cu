@@ -17,13 +17,28 @@
 // output, checksum plane included) for one image, and only that image's CTA
 // runs.  FC weights are never faulted and are read from global memory.
 //
-// Arithmetic follows the per-layer kernels: each convolution output is an
-// FFMA chain over the K index (r, s, c) in that order, then + bias, fault
-// delta, ReLU; the carry-through channel is coef * (sum of the centre-tap
-// input channels + incoming checksum); max-pool propagates NaN; each FC
-// neuron is a dot product (warp-parallel here, so its summation order
-// differs from the FC kernel's), the carry-through neuron coef * (sum of
-// data inputs + sum of checksum inputs); the verdict is NOT(|S - r| <= tau).
+// Arithmetic: each convolution output is an FFMA chain over the K index
+// (c, r, s), then + bias, fault delta, ReLU; the carry-through channel is
+// coef * (sum of the centre-tap input channels + incoming checksum); max-pool
+// propagates NaN; an FC neuron is a dot product over eight threads, the
+// carry-through neuron coef * (sum of data inputs + sum of checksum inputs);
+// the verdict is NOT(|S - r| <= tau).
+//
+// What bounds it: latency at small batches, issue slots in the campaign.
+// LeNet-5: one to 64 images 36.5 -> 9.3 us (the host needs 8.6 us for a
+// call), 1,024 images 199 -> 48 us, 2,048 faults on 8 images 1.9 -> 0.30 ms,
+// against one conv output per thread with the unpooled tensors in shared
+// memory and a warp per FC neuron.
+// A convolution and its pool are one step: a task is one pooled output, whose
+// thread computes the window's four convolution outputs from two rolling
+// input rows in registers (four FFMAs per weight read), so the unpooled
+// tensors are never stored.  FC weights: an inference that gives every image
+// an SM copies them into shared memory behind the convolutions (they are
+// never written, so the copy starts before the previous kernel ends); with
+// more images, and in the campaign, where several CTAs share an SM, they are
+// read through L1.
+#include <algorithm>
+
 #include "ct_internal.h"
 
 namespace ct {
@@ -37,47 +52,187 @@ __device__ __forceinline__ float flip_f32(float v, int bit) {
     return __uint_as_float(__float_as_uint(v) ^ (1u << bit));
 }
 
-// warp dot product of w[0..n) and x[0..n); every lane returns the sum
-__device__ __forceinline__ float warp_dot(const float *__restrict__ w, const float *x, int n, int lane) {
-    float s = 0.f;
-    for (int i = lane; i < n; i += 32) s = fmaf(__ldg(w + i), x[i], s);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    return s;
-}
-
-__device__ __forceinline__ float warp_sum(const float *x, int n, int lane) {
-    float s = 0.f;
-    for (int i = lane; i < n; i += 32) s += x[i];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    return s;
-}
+// Filters in shared memory: [k][c][r] rows of R taps, padded to whole 16 bytes.
+__host__ __device__ inline int w_row(int R) { return (R + 3) & ~3; }
 
 // shared-memory layout (floats), from the shapes
 struct SmLayout {
-    int w1, w2, img, a1, c1, p1, q1, a2, c2, p2, q2, f1, f2, f3, total;
+    int w1, w2, img, p1, q1, p2, q2, f1, f2, f3, v1, v2, v3, total;
 };
-__host__ __device__ inline SmLayout sm_layout(const SmallNet &g) {
+__host__ __device__ inline SmLayout sm_layout(const SmallNet &g, bool fc_smem) {
     SmLayout L;
     int o = 0;
     auto take = [&](int n) { int at = o; o += (n + 3) & ~3; return at; };
-    L.w1 = take(g.K1 * g.R1 * g.R1 * g.C0);
-    L.w2 = take(g.K2 * g.R2 * g.R2 * g.K1);
+    L.w1 = take(g.K1 * g.C0 * g.R1 * w_row(g.R1));
+    L.w2 = take(g.K2 * g.K1 * g.R2 * w_row(g.R2));
     L.img = take(g.C0 * g.H0 * g.W0);
-    L.a1 = take(g.K1 * g.H1 * g.W1);
-    L.c1 = take(g.H1 * g.W1);
     L.p1 = take(g.K1 * g.Hp1 * g.Wp1);
     L.q1 = take(g.Hp1 * g.Wp1);
-    L.a2 = take(g.K2 * g.H2 * g.W2);
-    L.c2 = take(g.H2 * g.W2);
     L.p2 = take(g.NIN1);                 // NHWC flatten order: (h, w, c)
     L.q2 = take(g.Hp2 * g.Wp2);
     L.f1 = take(g.N1 + 1);               // data neurons, then the carry-through neuron
     L.f2 = take(g.N2 + 1);
     L.f3 = take(g.N3 + 1);               // logits, then S
+    L.v1 = take(fc_smem ? g.N1 * g.NIN1 : 0);
+    L.v2 = take(fc_smem ? g.N2 * g.N1 : 0);
+    L.v3 = take(fc_smem ? g.N3 * g.N2 : 0);
     L.total = o;
     return L;
+}
+
+// The four convolution outputs under pooling window (pp, pq) of one filter:
+// acc[2 i + j] += sum over (c, r, s) of in[c][2 pp + i + r][2 pq + j + s] *
+// wk[c][r][s].  RT > 0: the filter size at compile time and an even row pitch
+// (8-byte reads of the input rows); else any.
+template <int RT>
+__device__ __forceinline__ void conv_window(const float *in, int C, int H, int W, const float *wk, int R, int pp, int pq,
+                                            float (&acc)[4]) {
+    if constexpr (RT > 0) {
+        static_assert(RT % 2 == 1, "an input row of RT + 1 values is read in pairs");
+        constexpr int WR = (RT + 3) & ~3;
+        for (int c = 0; c < C; ++c) {
+            const float *src = in + (c * H + 2 * pp) * W + 2 * pq;
+            float row[2][RT + 1];
+            auto load = [&](float (&d)[RT + 1], const float *p) {
+#pragma unroll
+                for (int i = 0; i < RT + 1; i += 2) {
+                    const float2 v = *reinterpret_cast<const float2 *>(p + i);
+                    d[i] = v.x;
+                    d[i + 1] = v.y;
+                }
+            };
+            load(row[0], src);
+#pragma unroll
+            for (int r = 0; r < RT; ++r) {
+                load(row[(r + 1) & 1], src + (r + 1) * W);
+                float w[WR];
+#pragma unroll
+                for (int i = 0; i < WR; i += 4) {
+                    const float4 v = *reinterpret_cast<const float4 *>(wk + (c * RT + r) * WR + i);
+                    w[i] = v.x; w[i + 1] = v.y; w[i + 2] = v.z; w[i + 3] = v.w;
+                }
+#pragma unroll
+                for (int s = 0; s < RT; ++s)
+#pragma unroll
+                    for (int o = 0; o < 4; ++o) acc[o] = fmaf(row[(r + (o >> 1)) & 1][s + (o & 1)], w[s], acc[o]);
+            }
+        }
+    } else {
+        for (int c = 0; c < C; ++c)
+            for (int r = 0; r < R; ++r)
+                for (int s = 0; s < R; ++s) {
+                    const float w = wk[(c * R + r) * w_row(R) + s];
+                    const float *src = in + (c * H + 2 * pp + r) * W + 2 * pq + s;
+#pragma unroll
+                    for (int o = 0; o < 4; ++o) acc[o] = fmaf(src[(o >> 1) * W + (o & 1)], w, acc[o]);
+                }
+    }
+}
+
+// One convolution and its 2x2 max-pool: data channels to out[k][pq] (or, for
+// the FC input, out[pq * K + k]), the checksum channel to cs_out[pq].  cs_in
+// is the incoming checksum plane (null: none).
+template <int NT, int RT, bool FLAT>
+__device__ __forceinline__ void conv_pool(const float *in, const float *cs_in, int C, int H, int W, const float *w,
+                                          const float *bias, int K, int R, int Hp, int Wp, float coef, int pc,
+                                          bool fault, const FaultDelta &fd, float *out, float *cs_out) {
+    const int HWp = Hp * Wp, ctr = (R - 1) / 2;
+    for (int e = threadIdx.x; e < (K + pc) * HWp; e += NT) {
+        const int k = e / HWp, pq = e - k * HWp, pp = pq / Wp, pw = pq - pp * Wp;
+        float o4[4] = {0.f, 0.f, 0.f, 0.f};
+        if (k < K) {
+            conv_window<RT>(in, C, H, W, w + k * C * R * w_row(R), R, pp, pw, o4);
+            const float b = __ldg(bias + k);
+#pragma unroll
+            for (int o = 0; o < 4; ++o) o4[o] += b;
+        } else {
+#pragma unroll
+            for (int o = 0; o < 4; ++o) {
+                const int at = (2 * pp + (o >> 1) + ctr) * W + 2 * pw + (o & 1) + ctr;
+                float cs = 0.f;
+                for (int c = 0; c < C; ++c) cs += in[c * H * W + at];
+                o4[o] = coef * (cs_in ? cs + cs_in[at] : cs);
+            }
+        }
+        if (fault && fd.kout == k && (fd.cin < C || cs_in)) {
+#pragma unroll
+            for (int o = 0; o < 4; ++o) {
+                const int at = (2 * pp + (o >> 1) + fd.r) * W + 2 * pw + (o & 1) + fd.s;
+                o4[o] += fd.dv * (fd.cin < C ? in[fd.cin * H * W + at] : cs_in[at]);
+            }
+        }
+        float mx = -INFINITY;
+#pragma unroll
+        for (int o = 0; o < 4; ++o) vmax_nan(mx, relu_nan(o4[o]));
+        if (k == K) cs_out[pq] = mx;
+        else if (FLAT) out[pq * K + k] = mx;
+        else out[k * HWp + pq] = mx;
+    }
+}
+
+// FC layer of n_out neurons (weights w, rows of n_in) and, with pc, the
+// carry-through neuron over the inputs x and their n_cs checksums xcs; eight
+// threads per neuron.  Calls put(j, value before any ReLU) for every neuron,
+// j = n_out for the carry-through one.
+template <int NT, typename Put>
+__device__ __forceinline__ void fc_layer(const float *w, const float *bias, const float *x, const float *xcs, int n_in,
+                                         int n_cs, int n_out, float coef, int pc, Put &&put) {
+    const int sub = threadIdx.x & 7;
+    const bool vec = (n_in & 3) == 0;
+    // whole groups of eight threads stay together: the shuffles below name the full warp
+    for (int j = threadIdx.x >> 3; j < ((n_out + pc + 3) & ~3); j += NT / 8) {
+        float s = 0.f;
+        if (j < n_out) {
+            const float *wj = w + (size_t)j * n_in;
+            if (vec) {
+                float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 8
+                for (int k = 4 * sub; k < n_in; k += 32) {
+                    const float4 wv = *reinterpret_cast<const float4 *>(wj + k), xv = *reinterpret_cast<const float4 *>(x + k);
+                    a.x = fmaf(wv.x, xv.x, a.x); a.y = fmaf(wv.y, xv.y, a.y);
+                    a.z = fmaf(wv.z, xv.z, a.z); a.w = fmaf(wv.w, xv.w, a.w);
+                }
+                s = (a.x + a.y) + (a.z + a.w);
+            } else {
+                for (int k = sub; k < n_in; k += 8) s = fmaf(wj[k], x[k], s);
+            }
+        } else if (j == n_out && pc) {
+            float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (vec)
+                for (int k = 4 * sub; k < n_in; k += 32) {
+                    const float4 xv = *reinterpret_cast<const float4 *>(x + k);
+                    a.x += xv.x; a.y += xv.y; a.z += xv.z; a.w += xv.w;
+                }
+            else
+                for (int k = sub; k < n_in; k += 8) a.x += x[k];
+            for (int k = sub; k < n_cs; k += 8) s += xcs[k];
+            s += (a.x + a.y) + (a.z + a.w);
+        }
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (sub == 0 && j < n_out + pc) put(j, j < n_out ? s + __ldg(bias + j) : coef * s);
+    }
+}
+
+__device__ __forceinline__ void copy_async(float *dst, const float *src, int n, int nt) {
+    if ((n & 3) == 0) {
+        for (int i = threadIdx.x; i < n / 4; i += nt)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst + 4 * i)),
+                         "l"(src + 4 * i)
+                         : "memory");
+    } else {
+        for (int i = threadIdx.x; i < n; i += nt) dst[i] = src[i];
+    }
+}
+
+// filters [k][r][s][c] of global memory to the shared layout [k][c][r][s]
+template <int NT>
+__device__ __forceinline__ void stage_filters(float *dst, const float *src, int K, int R, int C) {
+    const int n = K * R * R * C, wr = w_row(R);
+    for (int i = threadIdx.x; i < n; i += NT) {
+        const int c = i % C, t = i / C, sx = t % R, t2 = t / R, r = t2 % R, k = t2 / R;
+        dst[((k * C + c) * R + r) * wr + sx] = src[i];
+    }
 }
 
 // faults == null: inference -- one fault, `single` (kind 2: none), and every
@@ -87,39 +242,46 @@ __host__ __device__ inline SmLayout sm_layout(const SmallNet &g) {
 // flag).  logits_out, top1_out may be null.  Without protection
 // (g.protect == 0) no checksum channel or neuron is computed, S is NaN and
 // the flag 0, as for the per-layer kernels.
-__global__ void __launch_bounds__(1024) campaign_small_kernel(const SmallNet g, const CampFault *faults,
-                                                               const CampFault single, int ipc, float *S_out,
-                                                               int32_t *top1_out, uint8_t *flag_out, float *logits_out,
-                                                               const SmallRerun rr) {
+// R5: both filters are 5x5 and both input rows have an even pitch.  FCS: the
+// FC weights are copied to shared memory.
+template <int NT, bool R5, bool FCS>
+__global__ void __launch_bounds__(NT, NT == 256 ? 4 : 1) campaign_small_kernel(const SmallNet g, const CampFault *faults,
+                                                            const CampFault single, int ipc, float *S_out,
+                                                            int32_t *top1_out, uint8_t *flag_out, float *logits_out,
+                                                            const SmallRerun rr) {
+    extern __shared__ __align__(16) float sm[];
+    const SmLayout L = sm_layout(g, FCS);
+    float *w1 = sm + L.w1, *w2 = sm + L.w2, *img = sm + L.img;
+    float *p1 = sm + L.p1, *q1 = sm + L.q1, *p2 = sm + L.p2, *q2 = sm + L.q2;
+    float *f1 = sm + L.f1, *f2 = sm + L.f2, *f3 = sm + L.f3;
+    const int tid = threadIdx.x;
+    if (faults) {                                // a campaign's activation fault: only the hit image's CTA works
+        pdl_wait();
+        const CampFault &cf = faults[blockIdx.x];
+        const int lo = blockIdx.y * ipc;
+        if (cf.kind == 1 && (cf.img < lo || cf.img >= lo + ipc)) return;
+    }
+    // the weights are never written by a kernel: read before the previous one ends
+    stage_filters<NT>(w1, g.w1, g.K1, g.R1, g.C0);
+    stage_filters<NT>(w2, g.w2, g.K2, g.R2, g.K1);
+    if (FCS) {
+        copy_async(sm + L.v1, g.wf1, g.N1 * g.NIN1, NT);
+        copy_async(sm + L.v2, g.wf2, g.N2 * g.N1, NT);
+        copy_async(sm + L.v3, g.wf3, g.N3 * g.N2, NT);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    const float *v1 = FCS ? sm + L.v1 : g.wf1, *v2 = FCS ? sm + L.v2 : g.wf2, *v3 = FCS ? sm + L.v3 : g.wf3;
     pdl_wait();
     pdl_trigger();
     const CampFault f = faults ? faults[blockIdx.x] : single;
     const bool campaign = faults != nullptr;
     const int pc = g.protect ? 1 : 0;            // checksum channels / neurons
     const int n_lo = blockIdx.y * ipc, n_hi = min(g.B + (campaign ? 0 : rr.n), n_lo + ipc);
-    // a campaign's activation fault: only the hit image's CTA works
-    if (campaign && f.kind == 1 && (f.img < n_lo || f.img >= n_hi)) return;
-    extern __shared__ __align__(16) float sm[];
-    const SmLayout L = sm_layout(g);
-    float *w1 = sm + L.w1, *w2 = sm + L.w2, *img = sm + L.img, *a1 = sm + L.a1, *c1 = sm + L.c1;
-    float *p1 = sm + L.p1, *q1 = sm + L.q1, *a2 = sm + L.a2, *c2 = sm + L.c2, *p2 = sm + L.p2, *q2 = sm + L.q2;
-    float *f1 = sm + L.f1, *f2 = sm + L.f2, *f3 = sm + L.f3;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int nw1 = g.K1 * g.R1 * g.R1 * g.C0, nw2 = g.K2 * g.R2 * g.R2 * g.K1;
-    for (int i = tid; i < nw1; i += blockDim.x) w1[i] = g.w1[i];
-    for (int i = tid; i < nw2; i += blockDim.x) w2[i] = g.w2[i];
-    __syncthreads();
-    if (tid == 0 && f.kind == 0 && f.word >= 0) {
-        float *w = f.layer == 0 ? w1 : w2;
-        w[f.word] = flip_f32(w[f.word], f.bit);
-    }
-    const bool fd1 = f.kind == 0 && f.layer == 0 && f.fd.active;
-    const bool fd2 = f.kind == 0 && f.layer == 1 && f.fd.active;
-    __syncthreads();
     const int n_first = (campaign && f.kind == 1) ? f.img : n_lo;
     const int n_last = (campaign && f.kind == 1) ? f.img + 1 : n_hi;
-    const int ctr1 = (g.R1 - 1) / 2, ctr2 = (g.R2 - 1) / 2;
-    const int HW0 = g.H0 * g.W0, HW1 = g.H1 * g.W1, HWp1 = g.Hp1 * g.Wp1, HW2 = g.H2 * g.W2, HWp2 = g.Hp2 * g.Wp2;
+    const bool fd1 = f.kind == 0 && f.layer == 0 && f.fd.active;
+    const bool fd2 = f.kind == 0 && f.layer == 1 && f.fd.active;
+    const int HW0 = g.H0 * g.W0, HWp1 = g.Hp1 * g.Wp1, HWp2 = g.Hp2 * g.Wp2;
     for (int n = n_first; n < n_last; ++n) {
         // ---- image [C0][H0][W0] ----
         const bool rerun = n >= g.B;             // a row of the re-run list
@@ -127,166 +289,146 @@ __global__ void __launch_bounds__(1024) campaign_small_kernel(const SmallNet g, 
         const float *xn = rerun ? rr.x + (size_t)src_n * g.C0 * HW0
                         : (g.x2 && n >= g.n_split) ? g.x2 + (size_t)(n - g.n_split) * g.C0 * HW0
                                                    : g.x + (size_t)n * g.C0 * HW0;
-        for (int i = tid; i < g.C0 * HW0; i += blockDim.x) img[i] = __ldg(xn + i);
+        for (int i = tid; i < g.C0 * HW0; i += NT) img[i] = __ldg(xn + i);
         __syncthreads();
-        // ---- conv1 + ReLU, its carry-through channel ----
-        for (int e = tid; e < (g.K1 + pc) * HW1; e += blockDim.x) {
-            const int k = e / HW1, pq = e % HW1, p = pq / g.W1, q = pq % g.W1;
-            float o;
-            if (k < g.K1) {
-                float acc = 0.f;
-                const float *wk = w1 + k * g.R1 * g.R1 * g.C0;
-                for (int r = 0; r < g.R1; ++r)
-                    for (int s = 0; s < g.R1; ++s)
-                        for (int c = 0; c < g.C0; ++c)
-                            acc = fmaf(img[(c * g.H0 + p + r) * g.W0 + q + s], wk[(r * g.R1 + s) * g.C0 + c], acc);
-                o = acc + __ldg(g.b1 + k);
-            } else {
-                float cs = 0.f;
-                for (int c = 0; c < g.C0; ++c) cs += img[(c * g.H0 + p + ctr1) * g.W0 + q + ctr1];
-                o = g.coef1 * cs;                       // the image carries no checksum
+        if (n == n_first && f.kind == 0 && f.word >= 0) {
+            // this CTA's copy of the faulted filter: device word (k, r, s, c)
+            if (tid == 0) {
+                float *w = f.layer == 0 ? w1 : w2;
+                const int C = f.layer == 0 ? g.C0 : g.K1, R = f.layer == 0 ? g.R1 : g.R2;
+                const int wd = (int)f.word, c = wd % C, t = wd / C, sx = t % R, t2 = t / R, r = t2 % R, k = t2 / R;
+                float &v = w[((k * C + c) * R + r) * w_row(R) + sx];
+                v = flip_f32(v, f.bit);
             }
-            if (fd1 && f.fd.kout == k && f.fd.cin < g.C0)
-                o += f.fd.dv * img[(f.fd.cin * g.H0 + p + f.fd.r) * g.W0 + q + f.fd.s];
-            o = relu_nan(o);
-            if (k < g.K1) a1[k * HW1 + pq] = o; else c1[pq] = o;
+            __syncthreads();
         }
+        // ---- conv1 + ReLU + pool (the image carries no checksum); an activation flip of this image ----
+        conv_pool<NT, R5 ? 5 : 0, false>(img, nullptr, g.C0, g.H0, g.W0, w1, g.b1, g.K1, g.R1, g.Hp1, g.Wp1, g.coef1, pc,
+                                         fd1, f.fd, p1, q1);
         __syncthreads();
-        // ---- 2x2 max-pool (data and checksum); an activation flip of this image ----
-        for (int e = tid; e < (g.K1 + pc) * HWp1; e += blockDim.x) {
-            const int k = e / HWp1, pq = e % HWp1, p = pq / g.Wp1, q = pq % g.Wp1;
-            const float *src = k < g.K1 ? a1 + k * HW1 : c1;
-            float mx = -INFINITY;
-            for (int i = 0; i < 2; ++i)
-                for (int j = 0; j < 2; ++j) vmax_nan(mx, src[(2 * p + i) * g.W1 + 2 * q + j]);
-            if (f.kind == 1 && n == f.img && f.act_c == k && f.act_hw == pq) mx = flip_f32(mx, f.bit);
-            if (k < g.K1) p1[k * HWp1 + pq] = mx; else q1[pq] = mx;
-        }
-        __syncthreads();
-        // ---- conv2 + ReLU (the checksum input is skipped by data filters),
-        // carry-through channel over data and checksum inputs ----
-        for (int e = tid; e < (g.K2 + pc) * HW2; e += blockDim.x) {
-            const int k = e / HW2, pq = e % HW2, p = pq / g.W2, q = pq % g.W2;
-            float o;
-            if (k < g.K2) {
-                float acc = 0.f;
-                const float *wk = w2 + k * g.R2 * g.R2 * g.K1;
-                for (int r = 0; r < g.R2; ++r)
-                    for (int s = 0; s < g.R2; ++s)
-                        for (int c = 0; c < g.K1; ++c)
-                            acc = fmaf(p1[(c * g.Hp1 + p + r) * g.Wp1 + q + s], wk[(r * g.R2 + s) * g.K1 + c], acc);
-                o = acc + __ldg(g.b2 + k);
-            } else {
-                float cs = 0.f;
-                for (int c = 0; c < g.K1; ++c) cs += p1[(c * g.Hp1 + p + ctr2) * g.Wp1 + q + ctr2];
-                o = g.coef2 * (cs + q1[(p + ctr2) * g.Wp1 + q + ctr2]);
+        if (f.kind == 1 && n == f.img) {
+            if (tid == 0) {
+                float &v = f.act_c < g.K1 ? p1[f.act_c * HWp1 + f.act_hw] : q1[f.act_hw];
+                v = flip_f32(v, f.bit);
             }
-            if (fd2 && f.fd.kout == k) {
-                const int h = p + f.fd.r, w = q + f.fd.s;
-                o += f.fd.dv * (f.fd.cin < g.K1 ? p1[(f.fd.cin * g.Hp1 + h) * g.Wp1 + w] : q1[h * g.Wp1 + w]);
-            }
-            o = relu_nan(o);
-            if (k < g.K2) a2[k * HW2 + pq] = o; else c2[pq] = o;
+            __syncthreads();
         }
-        __syncthreads();
-        // ---- 2x2 max-pool into the FC input: data in (h, w, c) order, checksum plane ----
-        for (int e = tid; e < (g.K2 + pc) * HWp2; e += blockDim.x) {
-            const int k = e / HWp2, pq = e % HWp2, p = pq / g.Wp2, q = pq % g.Wp2;
-            const float *src = k < g.K2 ? a2 + k * HW2 : c2;
-            float mx = -INFINITY;
-            for (int i = 0; i < 2; ++i)
-                for (int j = 0; j < 2; ++j) vmax_nan(mx, src[(2 * p + i) * g.W2 + 2 * q + j]);
-            if (k < g.K2) p2[pq * g.K2 + k] = mx; else q2[pq] = mx;
-        }
+        // ---- conv2 + ReLU + pool into the FC input (h, w, c): data filters skip the
+        // checksum input, the carry-through channel sums data and checksum inputs ----
+        conv_pool<NT, R5 ? 5 : 0, true>(p1, q1, g.K1, g.Hp1, g.Wp1, w2, g.b2, g.K2, g.R2, g.Hp2, g.Wp2, g.coef2, pc, fd2,
+                                        f.fd, p2, q2);
+        if (FCS) asm volatile("cp.async.wait_all;" ::: "memory");
         __syncthreads();
         // ---- FC1 + ReLU; carry-through neuron ----
-        for (int j = warp; j < g.N1 + pc; j += blockDim.x / 32) {
-            float o;
-            if (j < g.N1) o = warp_dot(g.wf1 + (size_t)j * g.NIN1, p2, g.NIN1, lane) + __ldg(g.bf1 + j);
-            else o = g.coeff1 * (warp_sum(p2, g.NIN1, lane) + warp_sum(q2, HWp2, lane));
-            if (lane == 0) f1[j] = relu_nan(o);
-        }
+        fc_layer<NT>(v1, g.bf1, p2, q2, g.NIN1, HWp2, g.N1, g.coeff1, pc, [&](int j, float o) { f1[j] = relu_nan(o); });
         __syncthreads();
         // ---- FC2 + ReLU; carry-through neuron ----
-        for (int j = warp; j < g.N2 + pc; j += blockDim.x / 32) {
-            float o;
-            if (j < g.N2) o = warp_dot(g.wf2 + (size_t)j * g.N1, f1, g.N1, lane) + __ldg(g.bf2 + j);
-            else o = g.coeff2 * (warp_sum(f1, g.N1, lane) + f1[g.N1]);
-            if (lane == 0) f2[j] = relu_nan(o);
-        }
+        fc_layer<NT>(v2, g.bf2, f1, f1 + g.N1, g.N1, 1, g.N2, g.coeff2, pc, [&](int j, float o) { f2[j] = relu_nan(o); });
         __syncthreads();
-        // ---- classifier; accumulated-checksum neuron S ----
-        for (int j = warp; j < g.N3 + pc; j += blockDim.x / 32) {
-            float o;
-            if (j < g.N3) o = warp_dot(g.wf3 + (size_t)j * g.N2, f2, g.N2, lane) + __ldg(g.bf3 + j);
-            else o = g.coeff3 * (warp_sum(f2, g.N2, lane) + f2[g.N2]);
-            if (lane == 0) f3[j] = o;
-        }
-        __syncthreads();
+        // ---- classifier; accumulated-checksum neuron S and the verdict ----
         const size_t o = (size_t)blockIdx.x * g.B + n;
-        if (rerun) {
-            for (int j = tid; j < g.N3; j += blockDim.x) rr.logits[(size_t)src_n * g.N3 + j] = f3[j];
-            if (tid == 0 && rr.S) rr.S[src_n] = g.protect ? f3[g.N3] : __int_as_float(0x7fc00000);
-            __syncthreads();
-            continue;
-        }
-        if (logits_out)
-            for (int j = tid; j < g.N3; j += blockDim.x) logits_out[o * g.N3 + j] = f3[j];
-        if (tid == 0) {
-            // top-1: a NaN logit gives -1; ties go to the lowest index
-            int best = 0;
-            bool nan = false;
-            for (int j = 0; j < g.N3; ++j) {
-                if (f3[j] != f3[j]) nan = true;
-                else if (f3[j] > f3[best]) best = j;
+        fc_layer<NT>(v3, g.bf3, f2, f2 + g.N2, g.N2, 1, g.N3, g.coeff3, pc, [&](int j, float v) {
+            if (j < g.N3) {
+                if (top1_out) f3[j] = v;
+                if (rerun) rr.logits[(size_t)src_n * g.N3 + j] = v;
+                else if (logits_out) logits_out[o * g.N3 + j] = v;
+                return;
             }
-            const float S = g.protect ? f3[g.N3] : __int_as_float(0x7fc00000);
-            if (S_out) S_out[o] = S;
-            if (top1_out) top1_out[o] = nan ? -1 : best;
-            const uint8_t fv = g.protect ? !(fabs((double)S - g.ref) <= g.tau) : 0;
+            if (rerun) {
+                if (rr.S) rr.S[src_n] = v;
+                return;
+            }
+            const uint8_t fv = !(fabs((double)v - g.ref) <= g.tau);
+            if (S_out) S_out[o] = v;
             if (flag_out) flag_out[o] = fv;
             if (!campaign && g.flag2) g.flag2[n] = fv;
+        });
+        if (!pc && tid == 0) {
+            const float nan = __int_as_float(0x7fc00000);
+            if (rerun) {
+                if (rr.S) rr.S[src_n] = nan;
+            } else {
+                if (S_out) S_out[o] = nan;
+                if (flag_out) flag_out[o] = 0;
+                if (!campaign && g.flag2) g.flag2[n] = 0;
+            }
         }
-        __syncthreads();
+        if (top1_out) {
+            // a NaN logit gives -1; ties go to the lowest index
+            __syncthreads();
+            if (tid == 0) {
+                int best = 0;
+                bool nan = false;
+                for (int j = 0; j < g.N3; ++j) {
+                    if (f3[j] != f3[j]) nan = true;
+                    else if (f3[j] > f3[best]) best = j;
+                }
+                top1_out[o] = nan ? -1 : best;
+            }
+        }
+        if (n + 1 < n_last) __syncthreads();
     }
+    if (FCS) asm volatile("cp.async.wait_all;" ::: "memory");
+}
+
+// whether the unrolled 5x5 path applies
+bool is_r5(const SmallNet &g) { return g.R1 == 5 && g.R2 == 5 && g.W0 % 2 == 0 && g.Wp1 % 2 == 0; }
+
+template <int NT, bool R5, bool FCS>
+cudaError_t small_go(const SmallNet &g, const CampFault *faults, const CampFault &single, dim3 grid, int ipc, float *S,
+                     int32_t *top1, uint8_t *flag, float *logits, const SmallRerun &rr, cudaStream_t st) {
+    const size_t smem = sizeof(float) * (size_t)sm_layout(g, FCS).total;
+    if (smem > 48 * 1024) {
+        cudaError_t e = cudaFuncSetAttribute(campaign_small_kernel<NT, R5, FCS>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+    }
+    pdl_launch(campaign_small_kernel<NT, R5, FCS>, grid, NT, smem, st, g, faults, single, ipc, S, top1, flag, logits, rr);
+    return cudaGetLastError();
 }
 
 }  // namespace
 
-size_t campaign_small_smem(const SmallNet &g) { return sizeof(float) * (size_t)sm_layout(g).total; }
+// One image's tensors, unpooled ones included, and the filters: the size that
+// decides whether a network runs whole in one CTA.
+size_t campaign_small_smem(const SmallNet &g) {
+    auto r4 = [](size_t n) { return (n + 3) & ~(size_t)3; };
+    return sizeof(float) *
+           (r4((size_t)g.K1 * g.R1 * g.R1 * g.C0) + r4((size_t)g.K2 * g.R2 * g.R2 * g.K1) + r4((size_t)g.C0 * g.H0 * g.W0) +
+            r4((size_t)g.K1 * g.H1 * g.W1) + r4((size_t)g.H1 * g.W1) + r4((size_t)g.K1 * g.Hp1 * g.Wp1) +
+            r4((size_t)g.Hp1 * g.Wp1) + r4((size_t)g.K2 * g.H2 * g.W2) + r4((size_t)g.H2 * g.W2) + r4(g.NIN1) +
+            r4((size_t)g.Hp2 * g.Wp2) + r4(g.N1 + 1) + r4(g.N2 + 1) + r4(g.N3 + 1));
+}
 
 cudaError_t launch_campaign_small(const SmallNet &g, const CampFault *faults, int n_faults, float *S, int32_t *top1,
                                   uint8_t *flag, cudaStream_t st) {
     if (n_faults <= 0) return cudaSuccess;
-    constexpr int IPC = 8;
-    const size_t smem = campaign_small_smem(g);
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(campaign_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem);
-        if (e != cudaSuccess) return e;
-    }
+    constexpr int IPC = 4;                       // images per CTA of a weight fault
     dim3 grid(n_faults, (g.B + IPC - 1) / IPC);
     CampFault none{};
     none.kind = 2;
-    SmallRerun rr{};
-    pdl_launch(campaign_small_kernel, grid, 256, smem, st, g, faults, none, IPC, S, top1, flag, (float *)nullptr, rr);
-    return cudaGetLastError();
+    const SmallRerun rr{};
+    if (is_r5(g)) return small_go<256, true, false>(g, faults, none, grid, IPC, S, top1, flag, nullptr, rr, st);
+    return small_go<256, false, false>(g, faults, none, grid, IPC, S, top1, flag, nullptr, rr, st);
 }
 
 cudaError_t launch_small_infer(const SmallNet &g, const CampFault &fault, float *logits, float *S, uint8_t *flag,
                                const SmallRerun &rr, cudaStream_t st) {
-    const size_t smem = campaign_small_smem(g);
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(campaign_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem);
-        if (e != cudaSuccess) return e;
+    // one image per CTA: the images of a batch (and the re-run list) run side
+    // by side.  Up to one image per SM: 1024 threads and the FC weights in
+    // shared memory, when they fit; more images: several CTAs of 256 threads
+    // per SM (152 images 12 us wide, 153 images 18 us; a second round of wide
+    // CTAs would take 24 us).
+    static const int sms = device_sm_count();
+    const int images = g.B + rr.n;
+    dim3 grid(1, images);
+    const bool wide = images <= sms && sizeof(float) * (size_t)sm_layout(g, true).total <= 220 * 1024;
+    if (is_r5(g)) {
+        if (wide) return small_go<1024, true, true>(g, nullptr, fault, grid, 1, S, nullptr, flag, logits, rr, st);
+        return small_go<256, true, false>(g, nullptr, fault, grid, 1, S, nullptr, flag, logits, rr, st);
     }
-    // one image per CTA of 1024 threads: the images of a batch (and the
-    // re-run list) run side by side
-    dim3 grid(1, g.B + rr.n);
-    pdl_launch(campaign_small_kernel, grid, 1024, smem, st, g, (const CampFault *)nullptr, fault, 1, S,
-               (int32_t *)nullptr, flag, logits, rr);
-    return cudaGetLastError();
+    if (wide) return small_go<1024, false, true>(g, nullptr, fault, grid, 1, S, nullptr, flag, logits, rr, st);
+    return small_go<256, false, false>(g, nullptr, fault, grid, 1, S, nullptr, flag, logits, rr, st);
 }
 
 }  // namespace ct

@@ -1,0 +1,71 @@
+"""The whole-network kernel (the LeNet-5 shape) at shapes other than LeNet-5:
+filter sizes with and without the unrolled path, odd row pitches, several
+image channels, FC rows that are not whole 16-byte vectors, more images than
+SMs, and faults; logits, S and the batched campaign against the oracle."""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+from _gpu import TOL, ct, run, same_class
+
+pytestmark = pytest.mark.gpu
+
+
+def shape(C0, H, R1, K1, R2, K2, n1, n2, n3):
+    Ly = synth.Layer
+    hp1 = (H - R1 + 1) // 2
+    hp2 = (hp1 - R2 + 1) // 2
+    L = [Ly("conv", 0, 1, cin=C0, cout=K1, k=R1, relu=True), Ly("maxpool", 1, 2, k=2, stride=2),
+         Ly("conv", 2, 3, cin=K1, cout=K2, k=R2, relu=True), Ly("maxpool", 3, 4, k=2, stride=2),
+         Ly("fc", 4, 5, cin=K2 * hp2 * hp2, cout=n1, relu=True), Ly("fc", 5, 6, cin=n1, cout=n2, relu=True),
+         Ly("fc", 6, 7, cin=n2, cout=n3, final=True)]
+    wl = synth.Workload("small", L, (C0, H, H), n3, 1, "fp32", 13, "normal")
+    return wl, synth.make_params(L, 13), (K1 + 1) * hp1 * hp1
+
+
+SHAPES = [((1, 28, 5, 6, 5, 16, 120, 84, 10), 160),     # more images than SMs
+          ((3, 32, 5, 4, 5, 7, 30, 9, 3), 5),           # 5x5, 175 FC inputs
+          ((2, 17, 3, 5, 3, 6, 33, 20, 11), 3),         # 3x3, odd pitches
+          ((1, 21, 2, 3, 4, 4, 130, 6, 2), 2)]          # even filters, more neurons than thread groups
+
+
+@pytest.mark.parametrize("dims,batch", SHAPES)
+def test_small_net_matches_oracle(dims, batch):
+    wl, p, per_img = shape(*dims)
+    m = ct().ct_build_workload(wl, p, max_batch=batch)
+    net = oracle.build_workload(wl, params=p)
+    x = synth.make_input(wl, batch=batch)
+    sel = sorted({0, batch // 2, batch - 1})
+    lg, S, _ = run(m, x)
+    assert ct().ct_launches_per_infer(m) == 1
+    o = oracle.forward(net, x[sel])
+    tol = TOL["fp32"]
+    assert (np.abs(lg[sel] - o["logits"]) <= tol * np.abs(o["logits"]).max(axis=1, keepdims=True)).all()
+    assert (np.abs(S[sel] - o["S"]) <= tol * np.abs(o["S"])).all()
+    # weight flips (stored filters, carry-through row, zero slice) and an
+    # activation flip, one by one and as a batched campaign
+    import torch
+    C0, H, R1, K1, R2, K2 = dims[:6]
+    Ct = K1 + 1
+    faults = [(0, 0, 1 * C0 * R1 * R1 + R1 + 1, 29), (0, 0, K1 * C0 * R1 * R1 + 1, 28),
+              (0, 2, (2 * Ct + 1) * R2 * R2 + 2, 29), (0, 2, (1 * Ct + K1) * R2 * R2 + 1, 28),
+              (0, 2, (K2 * Ct + 1) * R2 * R2 + 3, 28), (1, 2, (batch - 1) * per_img + per_img - 3, 29),
+              (1, 2, (batch - 1) * per_img + 4, 28)]
+    n = len(faults)
+    Sb = torch.full((n, batch), float("nan"), device="cuda")
+    tb = torch.zeros(n, batch, dtype=torch.int32, device="cuda")
+    fb = torch.zeros(n, batch, dtype=torch.uint8, device="cuda")
+    ct().ct_campaign_batched(m, torch.from_numpy(x).cuda(), batch, faults, Sb, tb, fb)
+    Sb = Sb.cpu().numpy()
+    i = batch - 1
+    for k, f in enumerate(faults):
+        ct().ct_inject(m, *f)
+        _, Sf, _ = run(m, x)
+        so = float(oracle.forward(net, x[[i]], oracle.Fault(f[0], f[1], f[2] - (i * per_img if f[0] else 0), f[3]))["S"][0])
+        for got in (Sf[i], Sb[k, i]):
+            assert same_class(got, so), (f, got, so)
+            if np.isfinite(so):
+                assert abs(got - so) <= tol * max(abs(so), 1e-6), (f, got, so)
+    assert ct().ct_device_error(m) == 0
+    m.close()
