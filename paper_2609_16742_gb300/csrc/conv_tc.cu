@@ -1406,17 +1406,28 @@ conv_tc_pair_kernel(const __grid_constant__ CUtensorMap amap, const __grid_const
 // First layers with at most 4 input channels (the image): the input is
 // stored NHWC with its channels padded to 4 (8 bytes per pixel) and the GEMM
 // K index runs over (tap, channel of 4), 16 taps per 64-wide K block.  TMA
-// im2col cannot fetch 8-byte pixels, so four producer warps build the A tile
-// in shared memory: each thread owns one output pixel, loads one 8-byte
-// input pixel per tap and writes the 128-byte swizzled row the MMA reads.
+// im2col cannot fetch 8-byte pixels, so producer warps build the A tile in
+// shared memory: each thread owns one output pixel, loads one 8-byte input
+// pixel per tap and writes the 128-byte swizzled row the MMA reads.
 // Output channels: 64.  The carry-through row is coef at the centre tap's
-// real channels: 16 constant rows after the 64 weight rows of every B stage,
+// real channels: 16 constant rows after the 64 weight rows of every K block,
 // used (N = 80) on the centre tap's K block, which the loop visits first.
-// Persistent, double-buffered accumulators, as above.
+//
+// Bound by the bytes written when every stage overlaps: two groups of four
+// producer warps take alternate tiles and load a tile's pixels while they
+// store the tile before; the weights (at most four K blocks) stay resident;
+// two accumulators alternate, each read by its own four epilogue warps, which
+// store whole 128-byte lines.  Columns past the last tap are zero from the
+// start and not rewritten, and K steps that hold no tap are not issued.  64
+// images of 224 x 224 (411 MB written): 297 us with one group of each, weights
+// copied per tile and 16-byte stores.
 // ---------------------------------------------------------------------------
-constexpr int SM_THREADS = 288;     // warps 0-3 producers, 4 MMA, 5-8 epilogue
+constexpr int SM_PROD = 8, SM_EPI_WARP0 = SM_PROD + 1;   // producer warps, the MMA warp, epilogue warps
+constexpr int SM_THREADS = 32 * (SM_EPI_WARP0 + 8);
 constexpr int SM_STAGES = 8;
 constexpr int SM_BN = 64;
+constexpr int SM_MAX_KB = 4;
+constexpr int SM_B_BYTES = (SM_BN + 16) * BK * 2;        // a K block's weights and carry-through rows
 
 struct TcGeomS {
     int M, PQ, Q, stride, pad, C, H, W, R, S;
@@ -1426,51 +1437,54 @@ struct TcGeomS {
 };
 
 __global__ void __launch_bounds__(SM_THREADS, 1)
-conv_tc_small_kernel(const __grid_constant__ CUtensorMap bmap, const ConvArgs a, const TcGeomS g) {
-    constexpr int B_ROWS = SM_BN + 16;
-    constexpr int B_BYTES_STAGE = B_ROWS * BK * 2;
-    constexpr int B_TMA_BYTES = SM_BN * BK * 2;
-    constexpr int NCH = 4;                                // accumulator chains (see conv_tc_kernel)
+conv_tc_small_kernel(const __grid_constant__ CUtensorMap bmap, const __grid_constant__ ConvArgs a, const TcGeomS g) {
+    constexpr int NCH = 3;                                // accumulator chains (see conv_tc_kernel)
     constexpr int CH = SM_BN + 16;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
-    uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    uint8_t *As = smem;
-    uint8_t *Bs = As + SM_STAGES * A_BYTES;
-    uint64_t *full = (uint64_t *)(Bs + SM_STAGES * B_BYTES_STAGE);
+    uint8_t *smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+    uint8_t *As = smem;                                   // [SM_STAGES][A_BYTES]
+    uint8_t *Bs = As + SM_STAGES * A_BYTES;               // [n_kb][SM_B_BYTES], in visiting order
+    float *bias_s = (float *)(Bs + SM_MAX_KB * SM_B_BYTES);
+    uint64_t *full = (uint64_t *)(bias_s + SM_BN);
     uint64_t *empty = full + SM_STAGES;
-    uint64_t *acc_full = empty + SM_STAGES;
-    uint64_t *acc_empty = acc_full + 1;
-    uint32_t *tmem_holder = (uint32_t *)(acc_empty + 1);
+    uint64_t *acc_full = empty + SM_STAGES;               // [2]
+    uint64_t *acc_empty = acc_full + 2;                   // [2]
+    uint64_t *b_full = acc_empty + 2;
+    uint32_t *tmem_holder = (uint32_t *)(b_full + 1);
     volatile uint32_t *abort_flag = tmem_holder + 1;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int taps = g.R * g.S;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < SM_STAGES; ++s) {
             mbar_init(smem_u32(&full[s]), 128);
             mbar_init(smem_u32(&empty[s]), 1);
         }
-        mbar_init(smem_u32(acc_full), 1);
-        mbar_init(smem_u32(acc_empty), 4);
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(smem_u32(&acc_full[b]), 1);
+            mbar_init(smem_u32(&acc_empty[b]), 4);
+        }
+        mbar_init(smem_u32(b_full), 1);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == 4) {
+    if (warp == SM_PROD) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_holder)),
                      "r"((uint32_t)g.tmem_cols));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
-    if (warp >= 5) {
-        // constant rows 64..79 of every B stage: row 64 = coef at the centre
-        // tap's real channels (columns col_ct .. col_ct + C - 1), the rest 0;
-        // rows whose index is a multiple of 8 are not permuted by the swizzle
-        const int t = threadIdx.x - 160;
+    {
+        // every A stage starts as zeros (the columns of absent taps stay so)
+        for (int i = threadIdx.x; i < SM_STAGES * A_BYTES / 16; i += SM_THREADS)
+            reinterpret_cast<uint4 *>(As)[i] = make_uint4(0u, 0u, 0u, 0u);
+        // constant rows 64..79 of the first K block (the centre tap's): row 64 =
+        // coef at its real channels (columns col_ct .. col_ct + C - 1), the rest
+        // 0; rows whose index is a multiple of 8 are not permuted by the swizzle
         const __half ch = __ushort_as_half(g.coef_h);
-        for (int s = 0; s < SM_STAGES; ++s) {
-            __half *rows = (__half *)(Bs + s * B_BYTES_STAGE + SM_BN * BK * 2);
-            for (int i = t; i < 16 * BK; i += 128)
-                rows[i] = (g.ct && i >= g.col_ct && i < g.col_ct + g.C) ? ch : __ushort_as_half((unsigned short)0);
-        }
+        __half *rows = (__half *)(Bs + SM_BN * BK * 2);
+        for (int i = threadIdx.x; i < 16 * BK; i += SM_THREADS)
+            rows[i] = (g.ct && i >= g.col_ct && i < g.col_ct + g.C) ? ch : __ushort_as_half((unsigned short)0);
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -1481,138 +1495,192 @@ conv_tc_small_kernel(const __grid_constant__ CUtensorMap bmap, const ConvArgs a,
     pdl_wait();
     pdl_trigger();
     const __half *x = static_cast<const __half *>(a.x);
+    // this CTA's tiles: lt = 0, 1, .. is tile blockIdx.x + lt * gridDim.x; K
+    // block i of it uses ring slot (lt * n_kb + i) % SM_STAGES
 
-    if (warp < 4) {
-        // ---------------- software im2col producers ----------------
-        const int row = threadIdx.x;
-        if (row == 0) asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&bmap) : "memory");
-        const int taps = g.R * g.S;
-        int it = 0;
-        for (int tile = blockIdx.x; tile < g.m_tiles && !*abort_flag; tile += gridDim.x) {
-            const int m = tile * BM + row;
+    if (warp < SM_PROD) {
+        // ---------------- software im2col producers: tiles lt = grp, grp + 2, .. ----------------
+        const int grp = warp >> 2, row = threadIdx.x & 127;
+        if (threadIdx.x == 0) {
+            mbar_arrive_expect_tx(smem_u32(b_full), g.n_kb * SM_BN * BK * 2);
+            for (int i = 0; i < g.n_kb; ++i)
+                tma_load_2d(smem_u32(Bs + i * SM_B_BYTES), &bmap, smem_u32(b_full), (i + g.kb_ct) % g.n_kb * BK, 0);
+        }
+        const int n_it = g.n_kb * ((g.m_tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x);
+        uint2 v[2][16];
+        // the pixels of K block i of local tile lt; 16 taps in flight together
+        auto fetch = [&](uint2 (&d)[16], int lt, int i) {
+            const int m = ((int)blockIdx.x + lt * (int)gridDim.x) * BM + row;
             const bool valid = m < g.M;
             const int mm = valid ? m : 0;
             const int nimg = mm / g.PQ, rem = mm % g.PQ, p = rem / g.Q, q = rem % g.Q;
             const int h0 = p * g.stride - g.pad, w0 = q * g.stride - g.pad;
             const __half *ximg = x + (size_t)nimg * g.H * g.W * 4;
-            for (int i = 0; i < g.n_kb; ++i, ++it) {
-                const int kb = (i + g.kb_ct) % g.n_kb;
-                // all 16 taps of this K block are fetched before any shared-memory
-                // store, so their global-load latencies overlap
-                uint2 v[16];
-                int r = (kb * 16) / g.S, sx = (kb * 16) % g.S;
+            const int t0 = (i + g.kb_ct) % g.n_kb * 16;
+            int r = t0 / g.S, sx = t0 % g.S;
 #pragma unroll
-                for (int u = 0; u < 16; ++u) {
-                    v[u] = make_uint2(0u, 0u);
-                    const int h = h0 + r, w = w0 + sx;
-                    if (valid && kb * 16 + u < taps && h >= 0 && h < g.H && w >= 0 && w < g.W)
-                        v[u] = __ldg(reinterpret_cast<const uint2 *>(ximg + ((size_t)h * g.W + w) * 4));
-                    if (++sx == g.S) { sx = 0; ++r; }
-                }
-                const int s = it % SM_STAGES;
-                const uint32_t ph = (uint32_t)(it / SM_STAGES) & 1u;
-                if (!mbar_wait(smem_u32(&empty[s]), ph ^ 1u, a.err, 1u)) { *abort_flag = 1; break; }
-                const uint32_t fb = smem_u32(&full[s]);
-                if (row == 0) {
-                    mbar_expect_tx_only(fb, B_TMA_BYTES);
-                    tma_load_2d(smem_u32(Bs + s * B_BYTES_STAGE), &bmap, fb, kb * BK, 0);
-                }
-                uint8_t *arow = As + s * A_BYTES + row * 128;
-#pragma unroll
-                for (int j = 0; j < 8; ++j)
-                    *reinterpret_cast<uint4 *>(arow + ((j ^ (row & 7)) << 4)) =
-                        make_uint4(v[2 * j].x, v[2 * j].y, v[2 * j + 1].x, v[2 * j + 1].y);
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                mbar_arrive(fb);
+            for (int u = 0; u < 16; ++u) {
+                if (t0 + u >= taps) break;
+                d[u] = make_uint2(0u, 0u);
+                const int h = h0 + r, w = w0 + sx;
+                if (valid && h >= 0 && h < g.H && w >= 0 && w < g.W)
+                    d[u] = __ldg(reinterpret_cast<const uint2 *>(ximg + ((size_t)h * g.W + w) * 4));
+                if (++sx == g.S) { sx = 0; ++r; }
             }
+        };
+        auto put = [&](uint2 (&d)[16], int lt, int i) -> bool {
+            const int it = lt * g.n_kb + i, s = it % SM_STAGES;
+            if (!mbar_wait(smem_u32(&empty[s]), ((uint32_t)(it / SM_STAGES) & 1u) ^ 1u, a.err, 1u)) return false;
+            const int nt = min(16, taps - (i + g.kb_ct) % g.n_kb * 16);   // taps of this K block
+            uint8_t *arow = As + s * A_BYTES + row * 128;
+            // a slot is only ever used by K blocks of as many taps when n_kb == 1;
+            // with several, absent taps are written as zeros
+            const int nw = g.n_kb == 1 ? nt : 16;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                if (2 * j >= nw) break;
+                const uint2 lo = 2 * j < nt ? d[2 * j] : make_uint2(0u, 0u);
+                const uint2 hi = 2 * j + 1 < nt ? d[2 * j + 1] : make_uint2(0u, 0u);
+                *reinterpret_cast<uint4 *>(arow + ((j ^ (row & 7)) << 4)) = make_uint4(lo.x, lo.y, hi.x, hi.y);
+            }
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            mbar_arrive(smem_u32(&full[s]));
+            return true;
+        };
+        // this group's K blocks in order: (lt, i), the next one fetched before
+        // the current one is stored
+        int lt = grp, i = 0;
+        const int n_lt = n_it / g.n_kb;
+        auto step = [&](int &l, int &k) {
+            if (++k == g.n_kb) { k = 0; l += 2; }
+        };
+        if (lt < n_lt) fetch(v[0], lt, i);
+        bool ok = true;
+        while (ok && lt < n_lt) {
+            int l2 = lt, k2 = i;
+            step(l2, k2);
+            if (l2 < n_lt) fetch(v[1], l2, k2);
+            ok = put(v[0], lt, i) && !*abort_flag;
+            if (!ok || l2 >= n_lt) break;
+            lt = l2;
+            i = k2;
+            step(l2, k2);
+            if (l2 < n_lt) fetch(v[0], l2, k2);
+            ok = put(v[1], lt, i) && !*abort_flag;
+            lt = l2;
+            i = k2;
         }
-    } else if (warp == 4) {
+        if (!ok) *abort_flag = 1;
+    } else if (warp == SM_PROD) {
         // ---------------- MMA issuer (whole warp, one lane issues) ----------------
         const uint32_t id_main = idesc_f16(BM, SM_BN);
         const uint32_t id_merged = idesc_f16(BM, SM_BN + 16);
         int it = 0, lt = 0;
-        for (int tile = blockIdx.x; tile < g.m_tiles; tile += gridDim.x, ++lt) {
+        bool ok = warp_wait(smem_u32(b_full), 0u, a.err, 2u);
+        if (!ok && lane == 0) *abort_flag = 1;
+        for (int tile = blockIdx.x; tile < g.m_tiles && ok; tile += gridDim.x, ++lt) {
             if (__any_sync(0xffffffffu, *abort_flag)) break;
-            if (!warp_wait(smem_u32(acc_empty), ((uint32_t)lt & 1u) ^ 1u, a.err, 8u)) {
+            const int ab = lt & 1;
+            if (!warp_wait(smem_u32(&acc_empty[ab]), ((uint32_t)(lt >> 1) & 1u) ^ 1u, a.err, 8u)) {
                 if (lane == 0) *abort_flag = 1;
                 break;
             }
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            bool ok = true;
             for (int i = 0; i < g.n_kb; ++i, ++it) {
-                const uint32_t d = tmem + (uint32_t)((i % NCH) * CH);
+                const uint32_t d = tmem + (uint32_t)(ab * 256 + (i % NCH) * CH);
                 const int s = it % SM_STAGES;
-                const uint32_t ph = (uint32_t)(it / SM_STAGES) & 1u;
-                if (!warp_wait(smem_u32(&full[s]), ph, a.err, 2u)) { ok = false; break; }
+                if (!warp_wait(smem_u32(&full[s]), (uint32_t)(it / SM_STAGES) & 1u, a.err, 2u)) { ok = false; break; }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t a_base = smem_u32(As + s * A_BYTES);
-                const uint32_t b_base = smem_u32(Bs + s * B_BYTES_STAGE);
-                const bool leader = elect_one();
-#pragma unroll
-                for (int k16 = 0; k16 < BK / 16; ++k16) {
-                    const uint64_t ad = smem_desc_sw128(a_base + k16 * 32);
-                    const uint64_t bd = smem_desc_sw128(b_base + k16 * 32);
-                    const uint32_t acc = (i >= NCH || k16 > 0) ? 1u : 0u;   // first use of the chain
-                    if (leader) umma_f16(d, ad, bd, (i == 0 && g.ct) ? id_merged : id_main, acc);
+                const int steps = (min(16, taps - (i + g.kb_ct) % g.n_kb * 16) + 3) / 4;   // K steps that hold taps
+                if (elect_one()) {
+                    const uint64_t ad = smem_desc_sw128(smem_u32(As + s * A_BYTES));
+                    const uint64_t bd = smem_desc_sw128(smem_u32(Bs + i * SM_B_BYTES));
+                    for (int k16 = 0; k16 < steps; ++k16)
+                        umma_f16(d, ad + 2 * k16, bd + 2 * k16, (i == 0 && g.ct) ? id_merged : id_main,
+                                 (i >= NCH || k16 > 0) ? 1u : 0u);
+                    umma_commit(smem_u32(&empty[s]));
                 }
-                if (leader) umma_commit(smem_u32(&empty[s]));
                 __syncwarp();
             }
             if (!ok) { if (lane == 0) *abort_flag = 1; break; }
-            if (elect_one()) umma_commit(smem_u32(acc_full));
+            if (elect_one()) umma_commit(smem_u32(&acc_full[ab]));
             __syncwarp();
         }
     } else {
-        // ---------------- epilogue: warps 5..8 ----------------
-        const int quad = warp & 3;
-        const int row = quad * 32 + lane;
-        const FaultDelta fd = a.fd;
+        // ---------------- epilogue: two groups of four warps, one per accumulator ----------------
+        const int quad = warp & 3, grp = (warp - SM_EPI_WARP0) >> 2;
+        const FaultDelta &fd = a.fd;
         const int chains = min(NCH, g.n_kb);
-        int lt = 0;
-        for (int tile = blockIdx.x; tile < g.m_tiles; tile += gridDim.x, ++lt) {
-            bool ok = mbar_wait(smem_u32(acc_full), (uint32_t)lt & 1u, a.err, 4u) && !*abort_flag;
+        const bool fast = !fd.active && a.res == nullptr;
+        const int et = threadIdx.x - 32 * SM_EPI_WARP0;
+        if (et < SM_BN) bias_s[et] = __ldg(a.bias + et);
+        asm volatile("bar.sync 1, 256;" ::: "memory");
+        int lt = grp;
+        for (int tile = blockIdx.x + grp * gridDim.x; tile < g.m_tiles; tile += 2 * gridDim.x, lt += 2) {
+            bool ok = mbar_wait(smem_u32(&acc_full[grp]), (uint32_t)(lt >> 1) & 1u, a.err, 4u) && !*abort_flag;
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint32_t trow = tmem + ((uint32_t)(quad * 32) << 16);
+            const uint32_t trow = tmem + (uint32_t)(grp * 256) + ((uint32_t)(quad * 32) << 16);
             float vals[SM_BN];
+            uint32_t ctr = 0u;
+            const bool ld_ct = a.cs_out != nullptr && g.ct;
+            {
+                uint32_t tv[SM_BN / 16][16];
 #pragma unroll
-            for (int c = 0; c < SM_BN; c += 16) {
-                tmem_ld16(trow + c, vals + c);
-                for (int ch = 1; ch < chains; ++ch) {
+                for (int c = 0; c < SM_BN; c += 16) tmem_ld16_nw(trow + c, tv[c / 16]);
+                if (ld_ct) tmem_ld1_nw(trow + SM_BN, ctr);          // chain 0 only
+                tmem_wait_ld();
+#pragma unroll
+                for (int c = 0; c < SM_BN; c += 16) tmem_done16(tv[c / 16], vals + c);
+            }
+            for (int ch = 1; ch < chains; ++ch)
+#pragma unroll
+                for (int c = 0; c < SM_BN; c += 16) {
                     float t[16];
                     tmem_ld16(trow + ch * CH + c, t);
 #pragma unroll
                     for (int i = 0; i < 16; ++i) vals[c + i] += t[i];
                 }
-            }
-            const float ctv = (a.cs_out != nullptr && g.ct) ? tmem_ld1(trow + SM_BN) : 0.f;   // chain 0 only
+            const float ctv = ld_ct ? tmem_done(ctr) : 0.f;
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(acc_empty));
-            const int m = tile * BM + row;
-            if (m < g.M) {
+            if (lane == 0) mbar_arrive(smem_u32(&acc_empty[grp]));
+            const int mw = tile * BM + quad * 32, m = mw + lane;
+            float fsrc = 0.f;
+            if (fd.active && m < g.M) {
                 const int nimg = m / g.PQ, rem = m % g.PQ, p = rem / g.Q, q = rem % g.Q;
-                float fsrc = 0.f;
-                if (fd.active) {
-                    const int h = p * g.stride + fd.r - g.pad, w = q * g.stride + fd.s - g.pad;
-                    if (fd.cin < g.C && h >= 0 && h < g.H && w >= 0 && w < g.W)
-                        fsrc = ldh(x, (((size_t)nimg * g.H + h) * g.W + w) * 4 + fd.cin);
+                const int h = p * g.stride + fd.r - g.pad, w = q * g.stride + fd.s - g.pad;
+                if (fd.cin < g.C && h >= 0 && h < g.H && w >= 0 && w < g.W)
+                    fsrc = ldh(x, (((size_t)nimg * g.H + h) * g.W + w) * 4 + fd.cin);
+            }
+            if (fast) {
+                // whole lines: the lanes of each group of four swap their 16-channel pieces
+                uint32_t pk[4][8];
+#pragma unroll
+                for (int c = 0; c < 4; ++c) pack16(vals + 16 * c, bias16_at(bias_s, a.bias, true, 16 * c), a.relu != 0, pk[c]);
+                transpose4_pieces(pk, lane & 3);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const int mk = mw + (lane & ~3) + k;
+                    if (mk < g.M)
+                        st_global_v8(static_cast<__half *>(a.y) + (size_t)mk * SM_BN + 16 * (lane & 3), pk[k]);
                 }
+            } else if (m < g.M) {
 #pragma unroll
                 for (int c = 0; c < SM_BN; c += 16) store_chunk(vals + c, a, SM_BN, (size_t)m, c, fsrc);
-                if (a.cs_out != nullptr) {
-                    float o = (a.role == CT_ROLE_CT) ? ctv : 0.f;
-                    if (fd.active && fd.kout == SM_BN) o += fd.dv * fsrc;
-                    if (a.relu) o = relu_keep_nan(o);
-                    static_cast<__half *>(a.cs_out)[m] = __float2half_rn(o);
-                }
+            }
+            if (a.cs_out != nullptr && m < g.M) {
+                float o = (a.role == CT_ROLE_CT) ? ctv : 0.f;
+                if (fd.active && fd.kout == SM_BN) o += fd.dv * fsrc;
+                if (a.relu) o = relu_keep_nan(o);
+                static_cast<__half *>(a.cs_out)[m] = __float2half_rn(o);
             }
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    if (warp == 4) {
+    if (warp == SM_PROD) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)g.tmem_cols));
     }
@@ -2545,6 +2613,7 @@ TcSmallPlan *tc_small_plan_create(const ConvArgs &a, const void *w_dev, std::str
     g.H = a.H; g.W = a.W; g.R = a.R; g.S = a.S;
     const int kp = tc_small_kpad(a.R, a.S);
     g.n_kb = kp / BK;
+    static_assert((7 * 7 * 4 + BK - 1) / BK <= SM_MAX_KB, "resident weights");
     const int ctr_tap = ((a.R - 1) / 2) * a.S + (a.S - 1) / 2;
     g.kb_ct = (ctr_tap * 4) / BK;
     g.col_ct = (ctr_tap * 4) % BK;
@@ -2559,7 +2628,7 @@ TcSmallPlan *tc_small_plan_create(const ConvArgs &a, const void *w_dev, std::str
                                 box, bes, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                                 CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) { if (why) *why = "weight tensor map"; delete pl; return nullptr; }
-    pl->smem = 1024 + (size_t)SM_STAGES * (A_BYTES + (SM_BN + 16) * BK * 2) + 8 * (2 * SM_STAGES + 2) + 16;
+    pl->smem = 1024 + (size_t)SM_STAGES * A_BYTES + SM_MAX_KB * SM_B_BYTES + 4 * SM_BN + 8 * (2 * SM_STAGES + 5) + 16;
     if (cudaFuncSetAttribute(conv_tc_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl->smem) !=
         cudaSuccess) {
         if (why) *why = "shared memory attribute";

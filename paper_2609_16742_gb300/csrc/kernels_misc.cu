@@ -373,20 +373,18 @@ __global__ void maxpool_scalar_kernel(PoolArgs a) {
 }
 
 // Global average pool: float [N, C] features (+ float [N] checksum feature).
-// A block takes 256 / SPLIT channels of one image, SPLIT threads per channel
-// with every SPLIT-th pixel each, whose sums meet in shared memory.  Bound by
-// the chain of a thread's loads: with eight threads per channel 37 images of
-// 7 x 7 x 512 take 5.7 us (launch included, cold) instead of 7.0 with one; on
-// 4 x 4 maps (16 loads) one thread is better, 3.8 us for 128 images instead
-// of 5.5.  The block past the channels sums the checksum plane.
-template <typename T, int SPLIT>
+// A block takes 16 vectors of 16 bytes of channels of one image, 16 threads
+// per vector with every 16th pixel each, whose sums meet in shared memory.
+// Bound by the chain of a thread's loads and, at large batches, by bytes: one
+// channel per thread and all pixels in its chain took 7.6 us for 256 images of
+// 7 x 7 x 512 (12.8 MB).  The block past the channels sums the checksum plane.
+template <typename T>
 __global__ void __launch_bounds__(256) gap_kernel(PoolArgs a) {
     pdl_wait();
     pdl_trigger();
-    constexpr int CH = 256 / SPLIT;
-    __shared__ float red[SPLIT][CH + 1];
-    const int HW = a.H * a.W, n = blockIdx.y, ci = threadIdx.x % CH, part = threadIdx.x / CH;
-    const int c = blockIdx.x * CH + ci;
+    constexpr int VE = 16 / (int)sizeof(T), CH = 16 * VE;
+    __shared__ float red[16][CH + 1];
+    const int HW = a.H * a.W, n = blockIdx.y, ci = threadIdx.x % 16, part = threadIdx.x / 16;
     if ((int)blockIdx.x * CH >= a.C) {
         if (threadIdx.x >= 32) return;
         const T *cs = static_cast<const T *>(a.cs_in) + (size_t)n * HW;
@@ -397,27 +395,50 @@ __global__ void __launch_bounds__(256) gap_kernel(PoolArgs a) {
         if (threadIdx.x == 0) static_cast<float *>(a.cs_out)[n] = s / (float)HW;
         return;
     }
-    float s = 0.f;
-    if (c < a.C) {
-        const T *x = static_cast<const T *>(a.x) + (size_t)n * HW * a.C + c;
-#pragma unroll 8
-        for (int i = part; i < HW; i += SPLIT) s += to_f(x[(size_t)i * a.C]);
-    }
-    if constexpr (SPLIT > 1) {
-        red[part][ci] = s;
-        __syncthreads();
-        if (part > 0) return;
-        s = 0.f;
+    const int c0 = blockIdx.x * CH + ci * VE;
+    float s[VE];
 #pragma unroll
-        for (int w = 0; w < SPLIT; ++w) s += red[w][ci];
+    for (int j = 0; j < VE; ++j) s[j] = 0.f;
+    if (c0 < a.C) {
+        const T *x = static_cast<const T *>(a.x) + (size_t)n * HW * a.C + c0;
+#pragma unroll 4
+        for (int i = part; i < HW; i += 16) {
+            const uint4 v = *reinterpret_cast<const uint4 *>(x + (size_t)i * a.C);
+            const T *tv = reinterpret_cast<const T *>(&v);
+#pragma unroll
+            for (int j = 0; j < VE; ++j) s[j] += to_f(tv[j]);
+        }
     }
-    if (c < a.C) static_cast<float *>(a.y)[(size_t)n * a.C + c] = s / (float)HW;
+#pragma unroll
+    for (int j = 0; j < VE; ++j) red[part][ci * VE + j] = s[j];
+    __syncthreads();
+    const int c = blockIdx.x * CH + threadIdx.x;
+    if ((int)threadIdx.x >= CH || c >= a.C) return;
+    float t = 0.f;
+#pragma unroll
+    for (int w = 0; w < 16; ++w) t += red[w][threadIdx.x];
+    static_cast<float *>(a.y)[(size_t)n * a.C + c] = t / (float)HW;
 }
 
-template <typename T, int SPLIT>
-void gap_go(const PoolArgs &a, cudaStream_t st) {
-    dim3 grid((a.C + 256 / SPLIT - 1) / (256 / SPLIT) + (a.cs_in ? 1 : 0), a.N);
-    pdl_launch(gap_kernel<T, SPLIT>, grid, 256, 0, st, a);
+// Channel counts that are not whole 16-byte vectors: a thread per channel.
+template <typename T>
+__global__ void gap_scalar_kernel(PoolArgs a) {
+    pdl_wait();
+    pdl_trigger();
+    const int HW = a.H * a.W;
+    const int n = blockIdx.y;
+    const int c = blockIdx.x * blockDim.x + threadIdx.x;
+    const T *x = static_cast<const T *>(a.x);
+    if (c < a.C) {
+        float s = 0.f;
+        for (int i = 0; i < HW; ++i) s += to_f(x[((size_t)n * HW + i) * a.C + c]);
+        static_cast<float *>(a.y)[(size_t)n * a.C + c] = s / (float)HW;
+    } else if (c == a.C && a.cs_in) {
+        const T *cs = static_cast<const T *>(a.cs_in);
+        float s = 0.f;
+        for (int i = 0; i < HW; ++i) s += to_f(cs[(size_t)n * HW + i]);
+        static_cast<float *>(a.cs_out)[n] = s / (float)HW;
+    }
 }
 
 // NCHW fp32 -> NHWC storage type, one thread per pixel; channels C..Cp-1
@@ -434,6 +455,35 @@ __global__ void convert_input_kernel(const float *in, T *out, int N, int C, int 
         T *dst = out + (size_t)e * Cp;
         for (int c = 0; c < Cp; ++c) dst[c] = from_f<T>(c < C ? src[(size_t)c * HW] : 0.f);
     }
+}
+
+// The same to FP16 pixels of four channels (C <= 4), four pixels per thread:
+// 16-byte loads of each plane, 32 bytes stored.  HW a multiple of 4 and the
+// images 16-byte aligned.  Bound by HBM: 64 images of 3 x 224 x 224 (64 MB)
+// 33 us with a thread per pixel.
+template <int C>
+__global__ void __launch_bounds__(256) convert_input4_kernel(const float *in, uint2 *out, int groups, int gpi,
+                                                             const int32_t *idx) {
+    pdl_wait();
+    pdl_trigger();
+    const int e = blockIdx.x * 256 + threadIdx.x;        // group of four pixels
+    if (e >= groups) return;
+    const int n = e / gpi, g = e - n * gpi;
+    const float4 *src = reinterpret_cast<const float4 *>(in) + (size_t)(idx ? idx[n] : n) * C * gpi + g;
+    float4 v[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) v[c] = c < C ? __ldcs(src + (size_t)c * gpi) : make_float4(0.f, 0.f, 0.f, 0.f);
+    const float *f[4] = {&v[0].x, &v[1].x, &v[2].x, &v[3].x};
+    uint32_t o[8];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const __half2 a = __floats2half2_rn(f[0][i], f[1][i]), b = __floats2half2_rn(f[2][i], f[3][i]);
+        o[2 * i] = *reinterpret_cast<const uint32_t *>(&a);
+        o[2 * i + 1] = *reinterpret_cast<const uint32_t *>(&b);
+    }
+    uint4 *dst = reinterpret_cast<uint4 *>(out + (size_t)e * 4);
+    dst[0] = make_uint4(o[0], o[1], o[2], o[3]);
+    dst[1] = make_uint4(o[4], o[5], o[6], o[7]);
 }
 
 __global__ void xor_bit_kernel(void *base, int64_t word, int bit, int word_bytes) {
@@ -529,15 +579,31 @@ cudaError_t launch_maxpool(const PoolArgs &a, bool half, cudaStream_t st) {
 }
 
 cudaError_t launch_gap(const PoolArgs &a, bool half, cudaStream_t st) {
-    const bool many = a.H * a.W >= 32;
-    if (half) many ? gap_go<__half, 8>(a, st) : gap_go<__half, 1>(a, st);
-    else many ? gap_go<float, 8>(a, st) : gap_go<float, 1>(a, st);
+    const int ve = half ? 8 : 4;
+    if (a.C % ve == 0) {
+        dim3 grid((a.C + 16 * ve - 1) / (16 * ve) + (a.cs_in ? 1 : 0), a.N);
+        if (half) pdl_launch(gap_kernel<__half>, grid, 256, 0, st, a);
+        else pdl_launch(gap_kernel<float>, grid, 256, 0, st, a);
+    } else {
+        dim3 grid((a.C + 1 + 127) / 128, a.N);
+        if (half) pdl_launch(gap_scalar_kernel<__half>, grid, 128, 0, st, a);
+        else pdl_launch(gap_scalar_kernel<float>, grid, 128, 0, st, a);
+    }
     return cudaGetLastError();
 }
 
 cudaError_t launch_convert_input(const float *in, void *out, int N, int C, int Cp, int H, int W, bool half,
                                  cudaStream_t st, const int32_t *idx) {
     const int64_t n = (int64_t)N * H * W;
+    if (half && Cp == 4 && C >= 1 && C <= 4 && H * W % 4 == 0 && n < (1ll << 31) && reinterpret_cast<uintptr_t>(in) % 16 == 0) {
+        const int groups = (int)(n / 4), gpi = H * W / 4, grid = (groups + 255) / 256;
+        uint2 *o = static_cast<uint2 *>(out);
+        if (C == 1) pdl_launch(convert_input4_kernel<1>, grid, 256, 0, st, in, o, groups, gpi, idx);
+        else if (C == 2) pdl_launch(convert_input4_kernel<2>, grid, 256, 0, st, in, o, groups, gpi, idx);
+        else if (C == 3) pdl_launch(convert_input4_kernel<3>, grid, 256, 0, st, in, o, groups, gpi, idx);
+        else pdl_launch(convert_input4_kernel<4>, grid, 256, 0, st, in, o, groups, gpi, idx);
+        return cudaGetLastError();
+    }
     if (half) pdl_launch(convert_input_kernel<__half>, grid_for(n, 256), 256, 0, st, in, (__half *)out, N, C, Cp, H, W, idx);
     else pdl_launch(convert_input_kernel<float>, grid_for(n, 256), 256, 0, st, in, (float *)out, N, C, Cp, H, W, idx);
     return cudaGetLastError();
