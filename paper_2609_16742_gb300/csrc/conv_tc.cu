@@ -68,7 +68,6 @@ using namespace tc;
 constexpr int BM = 128;            // output pixels per tile (TMEM lanes)
 constexpr int BK = 64;             // channels per K block (128 bytes of fp16)
 constexpr int A_BYTES = BM * BK * 2;
-constexpr int NTHREADS = 320;      // 1 TMA warp, 1 MMA warp, 8 epilogue warps
 constexpr int N_EPI_WARPS = 8;
 // conv_tc_kernel: TMA producer warps (each owning whole ring slots), one MMA
 // warp, 8 epilogue warps.  There are as few producers as the ring allows: a
@@ -1702,6 +1701,8 @@ conv_tc_small_kernel(const __grid_constant__ CUtensorMap bmap, const __grid_cons
 // carry-through row is merged into the centre tap's MMAs as in
 // conv_tc_kernel; two TMEM accumulators alternate between tiles.
 // ---------------------------------------------------------------------------
+constexpr int HT_THREADS = 352;                         // TMA warp, MMA warp, 8 epilogue warps, second MMA warp
+constexpr int HT_MMA2 = 10;                             // the second MMA warp
 constexpr int HT_TH = 16, HT_TW = 8;                    // output tile
 constexpr int HT_PH = HT_TH + 2, HT_PW = HT_TW + 2;     // input patch with a one-pixel halo
 constexpr int HT_A_BYTES = HT_PH * HT_PW * BK * 2;      // 23040
@@ -1788,11 +1789,19 @@ __host__ __device__ constexpr int halo_bres_off(int i) {
     return i == 0 ? 0 : (BN + 16) * BK * 2 + (i - 1) * BN * BK * 2;
 }
 
+// Two MMA warps take alternate tiles (and accumulators), so that one's barrier
+// waits pass while the other's MMAs are queued: with one warp the tensor core
+// idled for about 1,200 of the 3,400 cycles of an N = 64 tile, 73 us a layer
+// (256 images of 56 x 56 x 64), 50 us with two (56 us with a residual).
+// Sharing each streamed weight stage of N = 128 between two tiles (both
+// accumulators then belong to the current pair, and its epilogue stalls the
+// next) was slower: 236 -> 255 us for 64 images of 112 x 112 x 128.
+//
 // POOL: the 2 x 2 stride-2 max-pool that follows the convolution is applied
 // in the epilogue (data and checksum alike); a.y / a.cs_out are then the
 // pooled tensor [N, H / 2, W / 2, K] and its checksum plane.
 template <int BN, bool BRES, int NA, int NB, int NR, bool POOL>
-__global__ void __launch_bounds__(NTHREADS, 1)
+__global__ void __launch_bounds__(HT_THREADS, 1)
 conv_tc_halo_kernel(const __grid_constant__ HaloMaps maps, const ConvArgs a, const HaloGeom hg, const TcGeom g) {
     constexpr int B_ROWS = BN + 16;                       // 16 constant carry-through rows
     constexpr int B_STAGE = B_ROWS * BK * 2;
@@ -1847,7 +1856,7 @@ conv_tc_halo_kernel(const __grid_constant__ HaloMaps maps, const ConvArgs a, con
                      "r"((uint32_t)hg.tmem_cols));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
-    if (warp >= 2) {
+    if (warp >= 2 && warp < HT_MMA2) {
         // constant carry-through rows after the BN weight rows of every B stage:
         // row 0 = coef, rows 1..15 = 0 (swizzle-invariant)
         const uint32_t coef2 = (uint32_t)hg.coef_h | ((uint32_t)hg.coef_h << 16);
@@ -1904,9 +1913,9 @@ conv_tc_halo_kernel(const __grid_constant__ HaloMaps maps, const ConvArgs a, con
                         uint8_t *st = Rs + rs * R::STAGE;
                         mbar_arrive_expect_tx(rb, r_bytes);
                         if (hg.res)
-                            for (int cb = 0; cb < BN / 64; ++cb)
-                                tma_load_4d(smem_u32(st + cb * 128 * 128), &maps.rmap, rb, ht.nt * BN + cb * 64, ht.x0,
-                                            ht.y0, ht.n);
+                            for (int c64 = 0; c64 < BN / 64; ++c64)
+                                tma_load_4d(smem_u32(st + c64 * 128 * 128), &maps.rmap, rb, ht.nt * BN + c64 * 64,
+                                            ht.x0, ht.y0, ht.n);
                         if (hg.csin) tma_load_3d(smem_u32(st + R::RES), &maps.cmap, rb, ht.x0, ht.y0, ht.n);
                         if (hg.rescs) tma_load_3d(smem_u32(st + R::RES + R::CS), &maps.qmap, rb, ht.x0, ht.y0, ht.n);
                     }
@@ -1932,80 +1941,69 @@ conv_tc_halo_kernel(const __grid_constant__ HaloMaps maps, const ConvArgs a, con
             }
         }
         if (!ok && lane == 0) *abort_flag = 1;
-    } else if (warp == 1) {
-        // ---------------- MMA issuer (whole warp, one lane issues) ----------------
+    } else if (warp == 1 || warp == HT_MMA2) {
+        // ---------------- MMA issuers (whole warps, one lane issues) ----------------
         const uint32_t id_main = idesc_f16(BM, BN);
         const uint32_t id_merged = idesc_f16(BM, BN + 16);
-        int ai = 0, bi = 0, lt = 0;
+        // this warp's tiles: every second one of the CTA's, lt = w, w + 2, ..
+        const int w = warp == HT_MMA2 ? 1 : 0;
         bool ok = true;
         if (BRES) {
-            // resident weights: wait for all nine tiles once
+            // resident weights (one channel block): wait for all nine tiles once
             for (int i = 0; i < 9 && ok; ++i) ok = warp_wait(smem_u32(&b_full[i]), 0u, a.err, 2u);
         }
-        for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x, ++lt) {
+        int lt = w;
+        for (int tile = blockIdx.x + w * gridDim.x; tile < num_tiles && ok; tile += 2 * gridDim.x, lt += 2) {
             if (__any_sync(0xffffffffu, *abort_flag)) break;
-            const HaloTile ht = halo_tile(tile, hg);
-            const bool ct_here = hg.ct && ht.nt == 0;
-            const int ab = lt & 1;
-            if (!warp_wait(smem_u32(&acc_empty[ab]), ((uint32_t)(lt >> 1) & 1u) ^ 1u, a.err, 8u)) { ok = false; break; }
-            const uint32_t d = tmem + (uint32_t)(ab * CH);
+            const bool ct_here = hg.ct && halo_tile(tile, hg).nt == 0;
+            if (!warp_wait(smem_u32(&acc_empty[w]), ((uint32_t)(lt >> 1) & 1u) ^ 1u, a.err, 8u)) { ok = false; break; }
+            const uint32_t d = tmem + (uint32_t)(w * CH);
             for (int cb = 0; cb < hg.ncb && ok; ++cb) {
-                const int as = ai % NA;
+                const int ai = lt * hg.ncb + cb, as = ai % NA;
                 if (!warp_wait(smem_u32(&a_full[as]), (uint32_t)(ai / NA) & 1u, a.err, 2u)) { ok = false; break; }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint32_t a_base = smem_u32(As + as * HT_A_STAGE);
                 if constexpr (BRES) {
                     // all 36 MMAs of the tile in one burst from one lane
+                    const uint32_t b0 = smem_u32(Bs);
                     if (elect_one()) {
-                        const uint32_t b0 = smem_u32(Bs);
 #pragma unroll
                         for (int i = 0; i < 9; ++i) {
                             const int tap = tap_of(i, 4);
                             const uint32_t a_tap = a_base + (uint32_t)(((tap / 3) * HT_PW + tap % 3) * BK * 2);
                             const uint32_t b_base = b0 + (uint32_t)halo_bres_off<BN>(i);
 #pragma unroll
-                            for (int k16 = 0; k16 < BK / 16; ++k16) {
-                                const uint64_t ad = smem_desc_sw128_sbo(a_tap + k16 * 32, HT_ROW);
-                                const uint64_t bd = smem_desc_sw128(b_base + k16 * 32);
-                                const uint32_t acc = (cb > 0 || i > 0 || k16 > 0) ? 1u : 0u;
-                                umma_f16(d, ad, bd, (ct_here && i == 0) ? id_merged : id_main, acc);
-                            }
+                            for (int k16 = 0; k16 < BK / 16; ++k16)
+                                umma_f16(d, smem_desc_sw128_sbo(a_tap + k16 * 32, HT_ROW),
+                                         smem_desc_sw128(b_base + k16 * 32), (ct_here && i == 0) ? id_merged : id_main,
+                                         (i > 0 || k16 > 0) ? 1u : 0u);
                         }
-                        umma_commit(smem_u32(&a_empty[as]));
                     }
-                    __syncwarp();
-                    ++ai;
                 } else {
-                for (int i = 0; i < 9; ++i) {
-                    const int bs = BRES ? i : bi % NBS;
-                    const uint32_t bph = BRES ? 0u : (uint32_t)(bi / NBS) & 1u;
-                    if (!warp_wait(smem_u32(&b_full[bs]), bph, a.err, 2u)) { ok = false; break; }
-                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    const int tap = tap_of(i, 4);
-                    const uint32_t a_tap = a_base + (uint32_t)(((tap / 3) * HT_PW + tap % 3) * BK * 2);
-                    const uint32_t b_base = smem_u32(Bs + bs * B_STAGE);
-                    const bool merged = ct_here && i == 0;
-                    if (elect_one()) {
+                    for (int i = 0; i < 9; ++i) {
+                        const int bi = ai * 9 + i, bs = bi % NBS;
+                        if (!warp_wait(smem_u32(&b_full[bs]), (uint32_t)(bi / NBS) & 1u, a.err, 2u)) { ok = false; break; }
+                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                        const int tap = tap_of(i, 4);
+                        if (elect_one()) {
+                            const uint64_t ad = smem_desc_sw128_sbo(
+                                a_base + (uint32_t)(((tap / 3) * HT_PW + tap % 3) * BK * 2), HT_ROW);
+                            const uint64_t bd = smem_desc_sw128(smem_u32(Bs + bs * B_STAGE));
 #pragma unroll
-                        for (int k16 = 0; k16 < BK / 16; ++k16) {
-                            const uint64_t ad = smem_desc_sw128_sbo(a_tap + k16 * 32, HT_ROW);
-                            const uint64_t bd = smem_desc_sw128(b_base + k16 * 32);
-                            const uint32_t acc = (cb > 0 || i > 0 || k16 > 0) ? 1u : 0u;
-                            umma_f16(d, ad, bd, merged ? id_merged : id_main, acc);
+                            for (int k16 = 0; k16 < BK / 16; ++k16)
+                                umma_f16(d, ad + 2 * k16, bd + 2 * k16, ct_here && i == 0 ? id_merged : id_main,
+                                         (cb > 0 || i > 0 || k16 > 0) ? 1u : 0u);
+                            umma_commit(smem_u32(&b_empty[bs]));
                         }
-                        if (!BRES) umma_commit(smem_u32(&b_empty[bs]));
+                        __syncwarp();
                     }
-                    __syncwarp();
-                    if (!BRES) ++bi;
+                    if (!ok) break;
                 }
-                if (!ok) break;
                 if (elect_one()) umma_commit(smem_u32(&a_empty[as]));
                 __syncwarp();
-                ++ai;
-                }
             }
             if (!ok) break;
-            if (elect_one()) umma_commit(smem_u32(&acc_full[ab]));   // fires when the tile's MMAs have completed
+            if (elect_one()) umma_commit(smem_u32(&acc_full[w]));   // fires when the tile's MMAs have completed
             __syncwarp();
         }
         if (!ok && lane == 0) *abort_flag = 1;
@@ -2784,7 +2782,7 @@ cudaError_t launch_conv_tc_halo(const ConvArgs &a, const HaloPlan *pl, cudaStrea
     const int tiles = halo_tiles(pl, a.N);
     dim3 grid(tiles < pl->sms ? tiles : pl->sms);
 #define HALO_LAUNCH(P, ...) \
-    pdl_launch(conv_tc_halo_kernel<__VA_ARGS__, P>, grid, NTHREADS, pl->smem, st, pl->maps, a, hg, g)
+    pdl_launch(conv_tc_halo_kernel<__VA_ARGS__, P>, grid, HT_THREADS, pl->smem, st, pl->maps, a, hg, g)
     if (pl->kind == 0) pl->pool ? HALO_LAUNCH(true, HK0) : HALO_LAUNCH(false, HK0);
     else if (pl->kind == 1) pl->pool ? HALO_LAUNCH(true, HK1) : HALO_LAUNCH(false, HK1);
     else pl->pool ? HALO_LAUNCH(true, HK2) : HALO_LAUNCH(false, HK2);
