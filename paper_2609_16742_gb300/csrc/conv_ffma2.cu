@@ -179,13 +179,14 @@ conv_ffma2_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constan
     static_assert(WM * WN * KW == F_WARPS, "four warps");
     static_assert(KW == 1 || WM * WN == 1, "warps split K or the tile");
     extern __shared__ __align__(1024) uint8_t smem_raw[];
-    uint8_t *smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+    uint8_t *smem = smem_raw;          // no static shared memory: the dynamic part starts 1024-byte aligned
     float *red = (float *)(smem + STAGES * ST_BYTES);            // [KW][F_TM * F_TN][32] (KW > 1)
     // running centre-tap sums of each thread's rows: [F_TM][F_THREADS] (they
     // are touched in centre-tap blocks only, and registers are short)
     float *csum = red + (KW > 1 ? KW * F_TM * F_TN * 32 : 0);
     uint64_t *full = (uint64_t *)(csum + F_TM * F_THREADS);
     uint64_t *empty = full + STAGES;
+    volatile int &abort_s = *(volatile int *)(empty + STAGES);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) {
@@ -194,7 +195,6 @@ conv_ffma2_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constan
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    __shared__ int abort_s;
     if (threadIdx.x == 0) abort_s = 0;
     __syncthreads();
     pdl_wait();
@@ -480,58 +480,67 @@ conv_ffma2_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constan
         for (int h = 0; h < F_TN / 4; ++h)
             bias[h] = nb + 4 * LN * h < g.K ? __ldg(reinterpret_cast<const float4 *>(a.bias + nb + 4 * LN * h))
                                             : make_float4(0.f, 0.f, 0.f, 0.f);
-        constexpr int RB = NI < 4 ? NI : 4;         // rows whose residual loads are in flight together
+        float4 rv[NI][F_TN / 4];                    // every residual load in flight together
 #pragma unroll
-        for (int ib = 0; ib < NI; ib += RB) {
-            float4 rv[RB][F_TN / 4];
+        for (int i = 0; i < NI; ++i) {
+            const int m = m0 + wrow + lm + (i0 + i) * LM;
 #pragma unroll
-            for (int i = 0; i < RB; ++i) {
-                const int m = m0 + wrow + lm + (i0 + ib + i) * LM;
+            for (int h = 0; h < F_TN / 4; ++h)
+                rv[i][h] = (res && m < g.M && nb + 4 * LN * h < g.K)
+                               ? __ldg(reinterpret_cast<const float4 *>(res + (size_t)m * g.K + nb + 4 * LN * h))
+                               : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
 #pragma unroll
-                for (int h = 0; h < F_TN / 4; ++h)
-                    rv[i][h] = (res && m < g.M && nb + 4 * LN * h < g.K)
-                                   ? __ldg(reinterpret_cast<const float4 *>(res + (size_t)m * g.K + nb + 4 * LN * h))
-                                   : make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int i = 0; i < NI; ++i) {
+            const int m = m0 + wrow + lm + (i0 + i) * LM;
+            if (m >= g.M) continue;
+            float fsrc = 0.f;
+            if (fd.active) {
+                const int nimg = m / g.PQ, rem = m % g.PQ;
+                fsrc = f_fault_source(a, nimg, rem / g.Q, rem % g.Q);
             }
 #pragma unroll
-            for (int i = 0; i < RB; ++i) {
-                const int m = m0 + wrow + lm + (i0 + ib + i) * LM;
-                if (m >= g.M) continue;
-                float fsrc = 0.f;
-                if (fd.active) {
-                    const int nimg = m / g.PQ, rem = m % g.PQ;
-                    fsrc = f_fault_source(a, nimg, rem / g.Q, rem % g.Q);
-                }
+            for (int h = 0; h < F_TN / 4; ++h) {
+                const int k = nb + 4 * LN * h;
+                const float *bp = reinterpret_cast<const float *>(&bias[h]);
+                const float *rp = reinterpret_cast<const float *>(&rv[i][h]);
+                float o[4];
 #pragma unroll
-                for (int h = 0; h < F_TN / 4; ++h) {
-                    const int k = nb + 4 * LN * h;
-                    const float *bp = reinterpret_cast<const float *>(&bias[h]);
-                    const float *rp = reinterpret_cast<const float *>(&rv[i][h]);
-                    float o[4];
+                for (int e = 0; e < 4; ++e) {
+                    o[e] = v[i][4 * h + e] + bp[e];
+                    if (fd.active && fd.kout == k + e) o[e] += fd.dv * fsrc;
+                    if (res) o[e] += rp[e];
+                    if (a.relu) o[e] = relu_keep_nan(o[e]);
+                }
+                if (k < g.K)
+                    *reinterpret_cast<float4 *>(y + (size_t)m * g.K + k) = make_float4(o[0], o[1], o[2], o[3]);
+            }
+        }
+        if (do_cs) {
+            // checksum outputs: the lanes that share a row take different ones
+            // (one row after another, a row's loads waited for the row before)
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        o[e] = v[ib + i][4 * h + e] + bp[e];
-                        if (fd.active && fd.kout == k + e) o[e] += fd.dv * fsrc;
-                        if (res) o[e] += rp[e];
-                        if (a.relu) o[e] = relu_keep_nan(o[e]);
-                    }
-                    if (k < g.K)
-                        *reinterpret_cast<float4 *>(y + (size_t)m * g.K + k) = make_float4(o[0], o[1], o[2], o[3]);
-                }
-                if (do_cs && ln == 0) {
-                    const float *csi = static_cast<const float *>(a.cs_in);
-                    const int nimg = m / g.PQ, rem = m % g.PQ, p = rem / g.Q, q = rem % g.Q;
-                    const int hc = p * a.stride + (a.R - 1) / 2 - a.pad, wc = q * a.stride + (a.S - 1) / 2 - a.pad;
-                    const bool inb = hc >= 0 && hc < a.H && wc >= 0 && wc < a.W;
-                    const float cin = (csi && inb) ? csi[((size_t)nimg * a.H + hc) * a.W + wc] : 0.f;
-                    float o = 0.f;
-                    if (a.role == CT_ROLE_CT) o = a.coef * (cs[ib + i] + cin);
-                    else if (a.role == CT_ROLE_PASS) o = cin;
-                    if (fd.active && fd.kout == g.K) o += fd.dv * fsrc;
-                    if (a.res_cs) o += static_cast<const float *>(a.res_cs)[m];
-                    if (a.relu) o = relu_keep_nan(o);
-                    static_cast<float *>(a.cs_out)[m] = o;
-                }
+            for (int ib = 0; ib < NI; ib += LN) {
+                const int i = ib + ln;
+                float ct = 0.f;
+#pragma unroll
+                for (int t = 0; t < NI; ++t)
+                    if (t == i) ct = cs[t];
+                const int m = m0 + wrow + lm + (i0 + i) * LM;
+                if (i >= NI || m >= g.M) continue;
+                const float *csi = static_cast<const float *>(a.cs_in);
+                const int nimg = m / g.PQ, rem = m % g.PQ, p = rem / g.Q, q = rem % g.Q;
+                const int hc = p * a.stride + (a.R - 1) / 2 - a.pad, wc = q * a.stride + (a.S - 1) / 2 - a.pad;
+                const bool inb = hc >= 0 && hc < a.H && wc >= 0 && wc < a.W;
+                const float cin = (csi && inb) ? csi[((size_t)nimg * a.H + hc) * a.W + wc] : 0.f;
+                const float rcs = a.res_cs ? static_cast<const float *>(a.res_cs)[m] : 0.f;
+                float o = 0.f;
+                if (a.role == CT_ROLE_CT) o = a.coef * (ct + cin);
+                else if (a.role == CT_ROLE_PASS) o = cin;
+                if (fd.active && fd.kout == g.K) o += fd.dv * f_fault_source(a, nimg, p, q);
+                if (a.res_cs) o += rcs;
+                if (a.relu) o = relu_keep_nan(o);
+                static_cast<float *>(a.cs_out)[m] = o;
             }
         }
         if (KW > 1) csync();               // the reduction buffer is reused by the next piece
@@ -557,16 +566,17 @@ bool f_load_encoders() {
     return ok;
 }
 
-// tile variants: lanes' rows LM, warps WM x WN over the tile, KW over K; ring
-// stages in about 110 KB (two CTAs per SM)
+// tile variants: lanes' rows LM, warps WM x WN over the tile, KW over K; as
+// many ring stages (at most six) as two CTAs per SM have room for
+constexpr int FS_MAX = 113 * 1024;      // 228 KB per SM less 1 KB of system memory per CTA, halved
 template <int LM_, int WM_, int WN_, int KW_>
 struct FTile {
     static constexpr int LM = LM_, WM = WM_, WN = WN_, KW = KW_;
     static constexpr int BM = LM * F_TM * WM, LN = 32 / LM, BN = LN * F_TN * WN;
     static constexpr int RED = (KW > 1 ? KW * F_TM * F_TN * 32 * 4 : 0) + F_TM * F_THREADS * 4;
-    static constexpr int FIT = (110 * 1024 - RED) / ((BM + BN) * 128);
+    static constexpr int FIT = (FS_MAX - RED - 16) / ((BM + BN) * 128 + 16);
     static constexpr int STAGES = FIT > 6 ? 6 : FIT;
-    static constexpr size_t SMEM = 1024 + (size_t)STAGES * (BM + BN) * 128 + RED + 16 * STAGES;
+    static constexpr size_t SMEM = (size_t)STAGES * (BM + BN) * 128 + RED + 16 * STAGES + 16;
     static bool maps(CUtensorMap *am, CUtensorMap *bm, const ConvArgs &a, int max_batch, const void *x, const void *w) {
         cuuint64_t gdim[4] = {(cuuint64_t)a.C, (cuuint64_t)a.W, (cuuint64_t)a.H, (cuuint64_t)max_batch};
         cuuint64_t gstr[3] = {(cuuint64_t)a.C * 4, (cuuint64_t)a.W * a.C * 4, (cuuint64_t)a.H * a.W * a.C * 4};

@@ -302,8 +302,8 @@ __device__ __forceinline__ uint32_t cvt_h2(float lo, float hi, bool relu) {
     else asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
     return r;
 }
-__device__ __forceinline__ void store16_fast(const float *v, const Bias16 &b, const Res16 &r, bool res, bool relu,
-                                             __half *dst) {
+__device__ __forceinline__ void pack16_res(const float *v, const Bias16 &b, const Res16 &r, bool res, bool relu,
+                                           uint32_t (&pk)[8]) {
     const float *bb = reinterpret_cast<const float *>(b.q);
     float t[16];
 #pragma unroll
@@ -317,9 +317,13 @@ __device__ __forceinline__ void store16_fast(const float *v, const Bias16 &b, co
             t[2 * i] += f0.x; t[2 * i + 1] += f0.y; t[8 + 2 * i] += f1.x; t[8 + 2 * i + 1] += f1.y;
         }
     }
-    uint32_t pk[8];
 #pragma unroll
     for (int i = 0; i < 8; ++i) pk[i] = cvt_h2(t[2 * i], t[2 * i + 1], relu);
+}
+__device__ __forceinline__ void store16_fast(const float *v, const Bias16 &b, const Res16 &r, bool res, bool relu,
+                                             __half *dst) {
+    uint32_t pk[8];
+    pack16_res(v, b, r, res, relu, pk);
     st_global_v8(dst, pk);          // 16 channels of one pixel: 32-byte aligned
 }
 
@@ -386,6 +390,16 @@ __device__ __forceinline__ float fmax_nan(float a, float b) {
     float r;
     asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
     return r;
+}
+// The same for two FP16 values: rounding is monotonic, so the maximum of the
+// rounded values is the rounded maximum, at half the shuffles.
+__device__ __forceinline__ uint32_t pool2x2_lanes_h2(uint32_t v) {
+#pragma unroll
+    for (int mk = 1; mk <= 8; mk *= 8) {
+        const uint32_t o = __shfl_xor_sync(0xffffffffu, v, mk);
+        asm("max.NaN.f16x2 %0, %0, %1;" : "+r"(v) : "r"(o));
+    }
+    return v;
 }
 __device__ __forceinline__ float pool2x2_lanes(float v) {
     v = fmax_nan(v, __shfl_xor_sync(0xffffffffu, v, 1));
@@ -1774,9 +1788,9 @@ struct HaloMaps {
 // c ^ (r & 7)): the epilogue lane of pixel r reads 16 bytes of its own
 // 128-byte row, and without the swizzle the 32 lanes of a warp would all hit
 // the same four banks.
-template <int BN>
+template <int BN, bool RRES>
 struct HaloR {
-    static constexpr int RES = 128 * BN * 2;
+    static constexpr int RES = RRES ? 128 * BN * 2 : 0;
     static constexpr int CS = 128 * 2;
     static constexpr int STAGE = (RES + 2 * CS + 1023) / 1024 * 1024;   // swizzle atoms stay 1024-byte aligned
 };
@@ -1800,7 +1814,12 @@ __host__ __device__ constexpr int halo_bres_off(int i) {
 // POOL: the 2 x 2 stride-2 max-pool that follows the convolution is applied
 // in the epilogue (data and checksum alike); a.y / a.cs_out are then the
 // pooled tensor [N, H / 2, W / 2, K] and its checksum plane.
-template <int BN, bool BRES, int NA, int NB, int NR, bool POOL>
+//
+// RRES: the operand ring holds a residual tile too; without one its room goes
+// to weight stages.  The copy latency of a weight stage (about 2,800 cycles)
+// bounds streamed weights: with four stages a K block takes 650 cycles against
+// 256 of MMA, with eight 350-400.
+template <int BN, bool BRES, int NA, int NB, int NR, bool RRES, bool POOL>
 __global__ void __launch_bounds__(HT_THREADS, 1)
 conv_tc_halo_kernel(const __grid_constant__ HaloMaps maps, const ConvArgs a, const HaloGeom hg, const TcGeom g) {
     constexpr int B_ROWS = BN + 16;                       // 16 constant carry-through rows
@@ -1809,7 +1828,7 @@ conv_tc_halo_kernel(const __grid_constant__ HaloMaps maps, const ConvArgs a, con
     constexpr int NBS = BRES ? 9 : NB;
     constexpr int B_AREA = BRES ? halo_bres_off<BN>(9) : NB * B_STAGE;
     constexpr int CH = BN + 16;
-    using R = HaloR<BN>;
+    using R = HaloR<BN, RRES>;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     uint8_t *As = smem;
@@ -1912,7 +1931,7 @@ conv_tc_halo_kernel(const __grid_constant__ HaloMaps maps, const ConvArgs a, con
                         const uint32_t rb = smem_u32(&r_full[rs]);
                         uint8_t *st = Rs + rs * R::STAGE;
                         mbar_arrive_expect_tx(rb, r_bytes);
-                        if (hg.res)
+                        if (RRES && hg.res)
                             for (int c64 = 0; c64 < BN / 64; ++c64)
                                 tma_load_4d(smem_u32(st + c64 * 128 * 128), &maps.rmap, rb, ht.nt * BN + c64 * 64,
                                             ht.x0, ht.y0, ht.n);
@@ -2015,7 +2034,7 @@ conv_tc_halo_kernel(const __grid_constant__ HaloMaps maps, const ConvArgs a, con
         const int row = quad * 32 + lane;
         const __half *x = static_cast<const __half *>(a.x);
         const FaultDelta fd = a.fd;
-        const bool has_res = hg.res != 0, relu = a.relu != 0;
+        const bool has_res = RRES && hg.res != 0, relu = a.relu != 0;
         // one N tile: this thread's channels are the same in every tile
         constexpr int NBIAS = BN <= 64 ? BN / 32 : 1;
         Bias16 bias_r[NBIAS];
@@ -2030,6 +2049,8 @@ conv_tc_halo_kernel(const __grid_constant__ HaloMaps maps, const ConvArgs a, con
             const int m = valid ? (ht.n * hg.H + p) * hg.W + q : 0;
             const int n0 = ht.nt * BN + half * (BN / 2);
             const bool do_cs = half == 0 && a.cs_out != nullptr && ht.nt == 0;
+            Res16 rs[BN / 32];
+            CsIn csv{0.f, 0, 0};
             bool ok = mbar_wait(smem_u32(&acc_full[ab]), (uint32_t)(lt >> 1) & 1u, a.err, 4u) && !*abort_flag;
             const int rsl = lt % NR;
             if (ring) ok = ok && mbar_wait(smem_u32(&r_full[rsl]), (uint32_t)(lt / NR) & 1u, a.err, 4u);
@@ -2053,10 +2074,9 @@ conv_tc_halo_kernel(const __grid_constant__ HaloMaps maps, const ConvArgs a, con
             if (lane == 0) mbar_arrive(smem_u32(&acc_empty[ab]));
             // epilogue operands from the R ring
             const uint8_t *rst = Rs + rsl * R::STAGE;
-            Res16 rs[BN / 32];
 #pragma unroll
             for (int c = 0; c < BN / 32; ++c) {
-                if (hg.res) {
+                if (RRES && hg.res) {
                     // channels ch .. ch + 15: 64-channel block ch / 64, chunks (ch % 64) / 8 and the next
                     const int ch = half * (BN / 2) + 16 * c;
                     const uint8_t *rrow = rst + (ch / 64) * 128 * 128 + row * 128;
@@ -2067,14 +2087,9 @@ conv_tc_halo_kernel(const __grid_constant__ HaloMaps maps, const ConvArgs a, con
                     rs[c].r0 = rs[c].r1 = make_uint4(0u, 0u, 0u, 0u);
                 }
             }
-            CsIn csv{0.f, 0, 0};
             if (do_cs) {
                 if (hg.csin) csv.cin_h = reinterpret_cast<const unsigned short *>(rst + R::RES)[row];
                 if (hg.rescs) csv.rcs_h = reinterpret_cast<const unsigned short *>(rst + R::RES + R::CS)[row];
-            }
-            if (ring) {
-                __syncwarp();
-                if (lane == 0) mbar_arrive(smem_u32(&r_empty[rsl]));
             }
             if (POOL) {
                 // every lane computes its pixel (the shuffles need the whole warp);
@@ -2091,13 +2106,18 @@ conv_tc_halo_kernel(const __grid_constant__ HaloMaps maps, const ConvArgs a, con
                 const size_t mp = ((size_t)ht.n * (hg.H / 2) + p / 2) * (hg.W / 2) + q / 2;
 #pragma unroll
                 for (int c = 0; c < BN / 2; c += 16) {
-                    float t[16];
-                    epi16_vals(vals + c, BN <= 64 ? bias_r[(c / 16) % NBIAS] : load_bias16(a.bias, n0 + c), rs[c / 16],
-                               has_res, relu, fd, n0 + c, fsrc, t);
+                    const Bias16 bias = BN <= 64 ? bias_r[(c / 16) % NBIAS] : load_bias16(a.bias, n0 + c);
                     uint32_t pk[8];
+                    if (!fd.active) {
+                        pack16_res(vals + c, bias, rs[c / 16], has_res, relu, pk);
+                    } else {
+                        float t[16];
+                        epi16_vals(vals + c, bias, rs[c / 16], has_res, relu, fd, n0 + c, fsrc, t);
 #pragma unroll
-                    for (int i = 0; i < 8; ++i)
-                        pk[i] = cvt_h2(pool2x2_lanes(t[2 * i]), pool2x2_lanes(t[2 * i + 1]), false);
+                        for (int i = 0; i < 8; ++i) pk[i] = cvt_h2(t[2 * i], t[2 * i + 1], false);
+                    }
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) pk[i] = pool2x2_lanes_h2(pk[i]);
                     if (writer) st_global_v8(static_cast<__half *>(a.y) + mp * hg.K + n0 + c, pk);
                 }
                 if (do_cs) {
@@ -2125,6 +2145,15 @@ conv_tc_halo_kernel(const __grid_constant__ HaloMaps maps, const ConvArgs a, con
                                      rs[c / 16], has_res, relu, yrow + c);
                 }
                 if (do_cs) store_checksum_pre(ctv, csv, a, g, m, fsrc);
+            }
+            // The ring slot is released only here, after the values read from it
+            // are in the stored results: released right after the reads, the
+            // compiler moved some of them down to their use, past the arrival,
+            // and a refill that came at once overwrote 16-byte pieces of a
+            // residual before they were read.
+            if (ring) {
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&r_empty[rsl]));
             }
         }
     }
@@ -2661,22 +2690,41 @@ struct HaloPlan {
     const void *res, *csin, *rescs;   // tensors the R-ring maps point at
 };
 
-template <int BN, bool BRES, int NA, int NB, int NR, bool POOL>
+template <int BN, bool BRES, int NA, int NB, int NR, bool RRES, bool POOL>
 size_t halo_smem() {
     const int nbs = BRES ? 9 : NB;
     const size_t b_area = BRES ? (size_t)halo_bres_off<BN>(9) : (size_t)NB * (BN + 16) * BK * 2;
-    return 1024 + (size_t)NA * HT_A_STAGE + b_area + (size_t)NR * HaloR<BN>::STAGE +
+    return 1024 + (size_t)NA * HT_A_STAGE + b_area + (size_t)NR * HaloR<BN, RRES>::STAGE +
            8 * (2 * NA + 2 * nbs + 2 * NR + 4) + 16;
 }
 
 // halo kernel variants <BN, resident weights, patch stages, weight stages,
-// operand-ring stages>; each also with the fused 2 x 2 max-pool
-#define HK0 64, true, 4, 0, 3
-#define HK1 64, false, 3, 6, 3
-#define HK2 128, false, 3, 4, 2
+// operand-ring stages, residual in the ring>; each also with the fused 2 x 2
+// max-pool.  Resident weights need one channel block; with 128 filters also no
+// residual tiles beside them.  64 images of 112 x 112: 64 -> 128 channels 126
+// us with four streamed stages, 83 us resident; 128 -> 128 (pooled) 241 us with
+// four stages, 191 us with eight.
+#define HK0 64, true, 4, 0, 3, true
+#define HK1 64, false, 3, 6, 3, true
+#define HK2 128, false, 3, 4, 2, true
+#define HK3 128, false, 3, 8, 2, false
+#define HK4 128, true, 3, 0, 2, false
+// f(pool, variant...) for the plan's variant
+#define HALO_DISPATCH(F)                                   \
+    do {                                                    \
+        switch (pl->kind) {                                 \
+            case 0: pl->pool ? F(true, HK0) : F(false, HK0); break; \
+            case 1: pl->pool ? F(true, HK1) : F(false, HK1); break; \
+            case 2: pl->pool ? F(true, HK2) : F(false, HK2); break; \
+            case 3: pl->pool ? F(true, HK3) : F(false, HK3); break; \
+            default: pl->pool ? F(true, HK4) : F(false, HK4); break; \
+        }                                                   \
+    } while (0)
 
 // Tiles that overhang the image waste MMA rows: require whole 8-column tiles
-// and at most one partly filled row of tiles on a tall image.
+// and at most one partly filled row of tiles on a tall image.  (Tiles of whole
+// image rows for other widths, 112 of 128 MMA rows on pixels at 28 x 28 x 128,
+// ran 59-61 us for 256 images against 57-59 on im2col tiles.)
 bool halo_supported(int C, int K, int R, int S, int stride, int pad, int H, int W) {
     return R == 3 && S == 3 && stride == 1 && pad == 1 && C % BK == 0 && (K == 64 || K == 128) && W % HT_TW == 0 &&
            (H % HT_TH == 0 || H >= 3 * HT_TH);
@@ -2753,15 +2801,13 @@ HaloPlan *halo_plan_create(const ConvArgs &a, int max_batch, const void *w_dev, 
         delete pl;
         return nullptr;
     }
-    cudaError_t e;
+    cudaError_t e = cudaSuccess;
     pl->pool = pool ? 1 : 0;
-    pl->kind = (pl->BN == 64 && hg.ncb == 1) ? 0 : pl->BN == 64 ? 1 : 2;
+    pl->kind = pl->BN == 64 ? (hg.ncb == 1 ? 0 : 1) : res_dev ? 2 : hg.ncb == 1 ? 4 : 3;
 #define HALO_ATTR(P, ...)                                                                                        \
-    (pl->smem = halo_smem<__VA_ARGS__, P>(),                                                                       \
-     cudaFuncSetAttribute(conv_tc_halo_kernel<__VA_ARGS__, P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl->smem))
-    if (pl->kind == 0) e = pool ? HALO_ATTR(true, HK0) : HALO_ATTR(false, HK0);
-    else if (pl->kind == 1) e = pool ? HALO_ATTR(true, HK1) : HALO_ATTR(false, HK1);
-    else e = pool ? HALO_ATTR(true, HK2) : HALO_ATTR(false, HK2);
+    (void)(pl->smem = halo_smem<__VA_ARGS__, P>(),                                                                 \
+           e = cudaFuncSetAttribute(conv_tc_halo_kernel<__VA_ARGS__, P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl->smem))
+    HALO_DISPATCH(HALO_ATTR);
 #undef HALO_ATTR
     if (e != cudaSuccess) { cudaGetLastError(); if (why) *why = "shared memory attribute"; delete pl; return nullptr; }
     return pl;
@@ -2782,10 +2828,8 @@ cudaError_t launch_conv_tc_halo(const ConvArgs &a, const HaloPlan *pl, cudaStrea
     const int tiles = halo_tiles(pl, a.N);
     dim3 grid(tiles < pl->sms ? tiles : pl->sms);
 #define HALO_LAUNCH(P, ...) \
-    pdl_launch(conv_tc_halo_kernel<__VA_ARGS__, P>, grid, HT_THREADS, pl->smem, st, pl->maps, a, hg, g)
-    if (pl->kind == 0) pl->pool ? HALO_LAUNCH(true, HK0) : HALO_LAUNCH(false, HK0);
-    else if (pl->kind == 1) pl->pool ? HALO_LAUNCH(true, HK1) : HALO_LAUNCH(false, HK1);
-    else pl->pool ? HALO_LAUNCH(true, HK2) : HALO_LAUNCH(false, HK2);
+    (void)pdl_launch(conv_tc_halo_kernel<__VA_ARGS__, P>, grid, HT_THREADS, pl->smem, st, pl->maps, a, hg, g)
+    HALO_DISPATCH(HALO_LAUNCH);
 #undef HALO_LAUNCH
     return cudaGetLastError();
 }

@@ -7,6 +7,8 @@ import numpy as np
 import pytest
 
 import synth
+from _cache import inputs
+from _gpu import ct, model
 from test_gpu_fp32_conv import check, net_of
 
 pytestmark = pytest.mark.gpu
@@ -56,3 +58,32 @@ def test_fc_layers_match_oracle(prec, C, H, hidden, classes, batch):
          Ly("fc", 2, 3, cin=hidden, cout=classes, final=True)]
     wl = synth.Workload("fc", L, (3, H, H), classes, 1, prec, 11, "normal")
     check(wl, synth.make_params(L, 11), batch, sorted({0, batch // 2, batch - 1}))
+
+
+@pytest.mark.parametrize("C,K,H,batch", [
+    (64, 128, 16, 80),          # resident weights, 128 filters
+    (128, 128, 16, 80),         # streamed weights
+    (128, 128, 56, 6),          # the last row of tiles of an image partly filled
+])
+def test_halo_tiles_match_oracle(C, K, H, batch):
+    wl, p, _ = net_of(C, K, 3, 1, H, prec="fp16")
+    check(wl, p, batch, sorted({0, batch // 2, batch - 1}))
+
+
+@pytest.mark.parametrize("batch", [64, 100])
+def test_repeated_inferences_give_the_same_bits(batch):
+    """Every stage's slots are read before they are refilled: the same batch
+    gives the same bits every time (256 to 1,500 tiles per layer, so that
+    CTAs run several)."""
+    import torch
+    m = model("resnet18_imagenet", max_batch=batch)
+    x = torch.from_numpy(inputs("resnet18_imagenet", batch)).cuda()
+    lg = torch.empty(batch, m.n_classes, device="cuda")
+    S = torch.empty(batch, device="cuda")
+    ct().ct_infer(m, x, batch, lg, S)
+    ref = lg.clone(), S.clone()
+    for _ in range(60):
+        ct().ct_infer(m, x, batch, lg, S)
+        assert torch.equal(lg, ref[0]) and torch.equal(S, ref[1])
+    assert ct().ct_device_error(m) == 0
+    m.close()
