@@ -29,20 +29,37 @@
 // their convolution rows in order, so a row shared by two units is computed
 // once (plus one row at the start of each CTA's range in an image).  Each
 // epilogue thread keeps the vertical maximum of its output column in
-// registers; when a convolution row completes a pooled row, those column
-// maxima go through a shared-memory row buffer for the 3-wide horizontal
-// maximum and the pooled row is written.
+// registers; when a convolution row completes a pooled row, the 3-wide
+// horizontal maximum of those column maxima is written.
+//
+// Overlapped columns (OVL, Q <= 112).  The 8-row groups of the A descriptor
+// are 7 columns apart (SBO = 112 bytes) and start at column -1, so MMA row
+// 8 g + j is column 7 g + j - 1 and the 32 rows a warp reads are columns
+// 28 w - 1 .. 28 w + 27: everything its 14 pooled columns need.  The
+// horizontal maximum is then two shuffles per register inside the warp, and
+// the epilogue warps never wait for each other.  Column -1 and columns past Q
+// read bytes beside the row and are never used.  Wider images use columns
+// 0 .. 127 and a shared-memory row buffer, with a barrier per row.  256 images
+// of 224 x 224: 179 us with the row buffer and its barrier, 152 us overlapped,
+// all else equal.
 //
 // Warp roles (512 threads): warps 0-5 fill ring rows (entry e goes to warp
 // e % 6), warps 6 and 7 issue tcgen05.mma (one elected lane each, for
-// alternate convolution rows: issuing one row's 14 MMAs and 3 commits takes
-// a thread about 900 cycles, so one issuer left the tensor core idle half the
-// time, measured), warp 6 also allocates TMEM, warps 8-15 are the epilogue:
-// each TMEM lane quadrant is read by two warps, each taking 32 of the 64
+// alternate convolution rows, so that one warp's waits overlap the other's
+// issue), warp 6 also allocates TMEM, warps 8-15 are the epilogue: each TMEM
+// lane quadrant is read by two warps, each taking 32 of the 64
 // channels.  Four TMEM accumulators rotate over
 // consecutive convolution rows, so the MMAs run up to three rows ahead of
 // the epilogue.  Every mbarrier wait is bounded; on
 // expiry the kernel records an error code, stops and frees TMEM.
+//
+// What bounds it: control, not data.  Of 178 us at 256 images of 224 x 224
+// (154 MB read, 23 us at the copy rate), 99 us remained without any copy,
+// conversion, pooling or all but two MMAs of a row.  Runs and windows found by
+// arithmetic, one lane per barrier and one commit per row instead of five:
+// 152 us.  Then the epilogue (140 us by itself): no selects for the row's
+// edges or the first row of a run, packed bias adds: 128 us.  The MMAs alone
+// now take 84 us and the producers 96.
 #include "ct_internal.h"
 #include "tc_common.cuh"
 
@@ -71,7 +88,11 @@ constexpr int ST_EPI0 = 32 * (ST_NPROD + ST_NMMA);   // first epilogue thread
 constexpr int ST_THREADS = ST_EPI0 + 256;
 constexpr int ST_EPI = 256;                  // epilogue threads
 constexpr int ST_NACC = 4;                   // TMEM accumulators (rows in flight between MMA and epilogue)
+// job-done barriers, in turn: the MMAs run at most 9 jobs ahead of the job a
+// producer waits for (the ring's rows) and 4 ahead of the epilogue
+constexpr int ST_NJOB = 16;
 constexpr int ST_TMEM_COLS = 128 * ST_NACC;
+constexpr int ST_PAD = 128;                  // bytes before the ring: column -1 of slot 0 starts 16 before it
 
 constexpr size_t ST_OFF_B = (size_t)ST_NSLOT * ST_SLOT_BYTES;
 constexpr size_t ST_OFF_ROW = ST_OFF_B + (size_t)ST_KSTEPS * ST_B_STEP;
@@ -79,14 +100,14 @@ constexpr size_t ST_OFF_CS = ST_OFF_ROW + 2ull * 128 * ST_PIX_H * 2;
 // staging of FP32 image rows (bulk copies): ST_STG_W per producer warp, up
 // to 4 channels of 256 pixels each.  Shared memory goes to ring depth first:
 // the producer, MMA and epilogue stages only overlap when the ring holds
-// several convolution rows beyond the 7-row window (16 slots: 275 us at 256
-// images, 24: 238 us; deeper staging gained nothing)
+// several convolution rows beyond the 7-row window (24 slots were 13% faster
+// than 16 when both were tried; deeper staging gained nothing)
 constexpr int ST_STG_W = 2;                  // staging slots per producer warp
 constexpr int ST_NSTG = ST_NPROD * ST_STG_W;
 constexpr int ST_STG_BYTES = 4 * 256 * 4;
 constexpr size_t ST_OFF_STG = ST_OFF_CS + 2ull * 128 * 2;
 constexpr size_t ST_OFF_BAR = ST_OFF_STG + (size_t)ST_NSTG * ST_STG_BYTES;
-constexpr size_t ST_SMEM = 1024 + ST_OFF_BAR + 8 * (2 * ST_NSLOT + 2 * ST_NACC + ST_NMMA + ST_NSTG) + 16;
+constexpr size_t ST_SMEM = 1024 + ST_PAD + ST_OFF_BAR + 8 * (ST_NSLOT + ST_NJOB + ST_NACC + ST_NMMA + ST_NSTG) + 16;
 
 struct StemGeom {
     int N, C, H, W, P, Q, P2, Q2;
@@ -94,35 +115,42 @@ struct StemGeom {
     uint16_t coef_h;
 };
 
-// Walks the convolution rows of one CTA's unit range [u, u_end) in order.
-struct StemJobs {
+// The runs of convolution rows of one CTA's unit range [u, u_end), one run
+// per image, in order.  Run rows are the jobs j0 .. j0 + nj - 1 (convolution
+// rows p0 ..); they read the ring entries e0 .. e0 + 2 nj + 4 (input rows
+// 2 p0 - 3 ..), job j the seven from e0 + 2 (j - j0) on.  Every role finds its
+// own jobs or entries by arithmetic: stepping through all rows to pick every
+// sixth cost a producer warp more than converting its row.
+struct StemRun {
     int u, u_end;
-    int n, p, p_end;
-    bool seg_start;      // first row of a run within one image
+    int n, p0, nj, j0, e0;
 
-    __device__ bool start_seg(const StemGeom &g) {
+    __device__ bool next(const StemGeom &g) {
         if (u >= u_end) return false;
+        if (nj) { j0 += nj; e0 += 2 * nj + 5; }
         n = u / g.P2;
-        const int ia = u % g.P2;
+        const int ia = u - n * g.P2;
         const int ib = min(g.P2 - 1, u_end - 1 - n * g.P2);
-        p = ia == 0 ? 0 : 2 * ia - 1;
-        p_end = min(2 * ib + 1, g.P - 1);
+        p0 = ia == 0 ? 0 : 2 * ia - 1;
+        nj = min(2 * ib + 1, g.P - 1) - p0 + 1;
         u = (n + 1) * g.P2;
-        seg_start = true;
         return true;
     }
-    __device__ bool first(int u0, int u1, const StemGeom &g) {
+    __device__ void init(int u0, int u1) {
         u = u0;
         u_end = u1;
-        return start_seg(g);
+        n = p0 = nj = j0 = e0 = 0;
     }
-    __device__ bool next(const StemGeom &g) {
-        if (p < p_end) {
-            ++p;
-            seg_start = false;
-            return true;
-        }
-        return start_seg(g);
+    // moves on to the run of job j / of entry e; false past the last run
+    __device__ bool at_job(int j, const StemGeom &g) {
+        while (j >= j0 + nj)
+            if (!next(g)) return false;
+        return true;
+    }
+    __device__ bool at_entry(int e, const StemGeom &g) {
+        while (nj == 0 || e >= e0 + 2 * nj + 5)
+            if (!next(g)) return false;
+        return true;
     }
 };
 
@@ -170,62 +198,18 @@ __device__ __forceinline__ float image_half(const float *img, const StemGeom &g,
     return __half2float(__float2half_rn(img[((size_t)c * g.H + h) * g.W + w]));
 }
 
-// The ring entries in production order: a CTA's convolution rows each need
-// the input rows not already in the ring (7 at the start of a run within an
-// image, then 2).  Entry e is produced by warp e % ST_NPROD.
-struct RowIter {
-    StemJobs jb;
-    bool have;
-    int ecount, t, n_new, y0;
-    int n_of_last;        // image of the entry last returned
-
-    __device__ void set_job() {
-        n_new = jb.seg_start ? 7 : 2;
-        y0 = jb.seg_start ? 2 * jb.p - 3 : 2 * jb.p + 2;
-    }
-    __device__ void init(int u0, int u1, const StemGeom &g) {
-        have = jb.first(u0, u1, g);
-        ecount = 0;
-        t = 0;
-        n_of_last = 0;
-        if (have) set_job();
-    }
-    // next entry of warp w: its index e and input row y
-    __device__ bool next(int w, int &e, int &y, const StemGeom &g) {
-        while (have) {
-            while (t < n_new) {
-                const int ee = ecount + t, tt = t;
-                ++t;
-                if (ee % ST_NPROD == w) {
-                    e = ee;
-                    y = y0 + tt;
-                    n_of_last = jb.n;
-                    return true;
-                }
-            }
-            ecount += n_new;
-            t = 0;
-            have = jb.next(g);
-            if (have) set_job();
-        }
-        return false;
-    }
-};
-
+template <bool OVL>
 __global__ void __launch_bounds__(ST_THREADS, 1)
 stem_pool_kernel(const ConvArgs a, const StemGeom g) {
-    pdl_wait();
-    pdl_trigger();
     extern __shared__ __align__(1024) uint8_t smem_raw[];
-    uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023) + ST_PAD;
     uint8_t *ring = smem;
     uint8_t *Bs = smem + ST_OFF_B;
     __half *rowbuf = (__half *)(smem + ST_OFF_ROW);
     __half *csbuf = (__half *)(smem + ST_OFF_CS);
     uint64_t *full = (uint64_t *)(smem + ST_OFF_BAR);
-    uint64_t *empty = full + ST_NSLOT;
-    uint64_t *acc_full = empty + ST_NSLOT;
-    uint64_t *acc_empty = acc_full + ST_NACC;
+    uint64_t *job_done = full + ST_NSLOT;                    // [ST_NJOB]
+    uint64_t *acc_empty = job_done + ST_NJOB;
     uint64_t *mma_done = acc_empty + ST_NACC;                // [ST_NMMA]
     uint64_t *stg_full = mma_done + ST_NMMA;                 // [ST_NSTG]
     float *stg = (float *)(smem + ST_OFF_STG);
@@ -239,8 +223,26 @@ stem_pool_kernel(const ConvArgs a, const StemGeom g) {
 
     // ---- set-up: zero the ring (its padding columns stay zero), weights to
     // the canonical no-swizzle layout, the carry-through row ----
-    for (int i = threadIdx.x; i < (int)(ST_OFF_B / 16); i += ST_THREADS)
-        reinterpret_cast<uint4 *>(ring)[i] = make_uint4(0u, 0u, 0u, 0u);
+    for (int i = threadIdx.x; i < (int)((ST_OFF_B + ST_PAD) / 16); i += ST_THREADS)
+        reinterpret_cast<uint4 *>(ring - ST_PAD)[i] = make_uint4(0u, 0u, 0u, 0u);
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < ST_NSLOT; ++s) mbar_init(smem_u32(&full[s]), 1);
+        for (int s = 0; s < ST_NJOB; ++s) mbar_init(smem_u32(&job_done[s]), 1);
+        for (int b = 0; b < ST_NACC; ++b) mbar_init(smem_u32(&acc_empty[b]), ST_EPI / 32);
+        for (int w = 0; w < ST_NMMA; ++w) mbar_init(smem_u32(&mma_done[w]), 1);
+        for (int s = 0; s < ST_NSTG; ++s) mbar_init(smem_u32(&stg_full[s]), 1);
+        *abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    // Everything above touches this CTA's own shared memory only.  TMEM is
+    // allocated after the wait: the kernel before may still have to allocate.
+    pdl_wait();
+    pdl_trigger();
+    if (warp == ST_MMA_WARP) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_holder)),
+                     "r"((uint32_t)ST_TMEM_COLS));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    }
     {
         const __half *w = static_cast<const __half *>(a.w);
         const __half coef = __ushort_as_half(g.coef_h);
@@ -266,25 +268,6 @@ stem_pool_kernel(const ConvArgs a, const StemGeom g) {
         }
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < ST_NSLOT; ++s) {
-            mbar_init(smem_u32(&full[s]), 32);
-            mbar_init(smem_u32(&empty[s]), ST_NMMA);      // one release per MMA warp
-        }
-        for (int b = 0; b < ST_NACC; ++b) {
-            mbar_init(smem_u32(&acc_full[b]), 1);
-            mbar_init(smem_u32(&acc_empty[b]), ST_EPI / 32);
-        }
-        for (int w = 0; w < ST_NMMA; ++w) mbar_init(smem_u32(&mma_done[w]), 1);
-        for (int s = 0; s < ST_NSTG; ++s) mbar_init(smem_u32(&stg_full[s]), 1);
-        *abort_flag = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    if (warp == ST_MMA_WARP) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_holder)),
-                     "r"((uint32_t)ST_TMEM_COLS));
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
-    }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -297,24 +280,25 @@ stem_pool_kernel(const ConvArgs a, const StemGeom g) {
         // row of W FP32 values) into its own staging slots; the warp then
         // converts a landed row to the two FP16 copies of its ring slot.
         // Rows outside the image are not copied (their slot reads as zero).
-        RowIter ri;
-        ri.init(u0, u1, g);
-        int ent_e[ST_STG_W], ent_y[ST_STG_W];
+        StemRun ri, rd, rw;                    // of the next entry to issue, to convert, and of the one it replaces
+        ri.init(u0, u1);
+        rd.init(u0, u1);
+        rw.init(u0, u1);
         int k_issue = 0, k_done = 0;
         bool ok = true, more = true;
         const uint32_t row_bytes = (uint32_t)g.W * 4u;
         while (ok) {
             // keep ST_STG_W entries in flight
             while (more && k_issue - k_done < ST_STG_W) {
-                int e, y;
-                more = ri.next(warp, e, y, g);
+                const int e = warp + k_issue * ST_NPROD;
+                more = ri.at_entry(e, g);
                 if (!more) break;
-                const int i = k_issue % ST_STG_W, sl = warp * ST_STG_W + i;
-                ent_e[i] = e; ent_y[i] = y;
+                const int y = 2 * ri.p0 - 3 + e - ri.e0;
+                const int sl = warp * ST_STG_W + k_issue % ST_STG_W;
                 if (lane == 0) {
                     const uint32_t bar = smem_u32(&stg_full[sl]);
                     if (y >= 0 && y < g.H) {
-                        const float *img = image_base(a, g, ri.n_of_last);
+                        const float *img = image_base(a, g, ri.n);
                         mbar_arrive_expect_tx(bar, row_bytes * (uint32_t)g.C);
                         for (int c = 0; c < g.C; ++c)
                             bulk_load(smem_u32(stg + (size_t)sl * (ST_STG_BYTES / 4) + c * g.W),
@@ -326,34 +310,50 @@ stem_pool_kernel(const ConvArgs a, const StemGeom g) {
                 ++k_issue;
             }
             if (k_done == k_issue) break;
-            if (__any_sync(0xffffffffu, *abort_flag)) { ok = false; break; }
-            const int i = k_done % ST_STG_W, sl = warp * ST_STG_W + i;
-            if (!warp_wait(smem_u32(&stg_full[sl]), (uint32_t)(k_done / ST_STG_W) & 1u, a.err, 1u)) { ok = false; break; }
-            const int e = ent_e[i], y = ent_y[i];
+            const int sl = warp * ST_STG_W + k_done % ST_STG_W;
+            const int e = warp + k_done * ST_NPROD;
             const int slot = e % ST_NSLOT;
-            if (!warp_wait(smem_u32(&empty[slot]), ((uint32_t)(e / ST_NSLOT) & 1u) ^ 1u, a.err, 1u)) { ok = false; break; }
+            // The slot is free when the last job that reads the entry it held
+            // is done, and the job before that (the other MMA warp's; a
+            // warp's jobs complete in order).  One lane per barrier.
+            int jw = -1;
+            if (e >= ST_NSLOT && rw.at_entry(e - ST_NSLOT, g))
+                jw = rw.j0 + min((e - ST_NSLOT - rw.e0) >> 1, rw.nj - 1);
+            bool mine = true;
+            if (lane == 0) mine = mbar_wait(smem_u32(&stg_full[sl]), (uint32_t)(k_done / ST_STG_W) & 1u, a.err, 1u);
+            else if (lane <= ST_NMMA && jw - lane + 1 >= 0)
+                mine = mbar_wait(smem_u32(&job_done[(jw - lane + 1) % ST_NJOB]),
+                                 (uint32_t)((jw - lane + 1) / ST_NJOB) & 1u, a.err, 1u);
+            ok = __all_sync(0xffffffffu, mine) && !__any_sync(0xffffffffu, *abort_flag);
+            if (!ok) break;
+            rd.at_entry(e, g);
+            const int y = 2 * rd.p0 - 3 + e - rd.e0;
             const bool row_ok = y >= 0 && y < g.H;
             const float *sr = stg + (size_t)sl * (ST_STG_BYTES / 4);
             uint8_t *E = ring + slot * ST_SLOT_BYTES;
             uint8_t *O = E + ST_ROW_BYTES;
+            // two pixels per lane (W is a multiple of 4)
 #pragma unroll
-            for (int it = 0; it < 8; ++it) {
-                const int col = lane + 32 * it;
+            for (int it = 0; it < 4; ++it) {
+                const int col = 2 * lane + 64 * it;
                 if (col < g.W) {
-                    float v[4];
+                    float2 v[4];
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) v[c] = (row_ok && c < g.C) ? sr[c * g.W + col] : 0.f;
-                    __half2 lo = __floats2half2_rn(v[0], v[1]);
-                    __half2 hi = __floats2half2_rn(v[2], v[3]);
-                    const uint2 pk = make_uint2(*reinterpret_cast<uint32_t *>(&lo), *reinterpret_cast<uint32_t *>(&hi));
-                    *reinterpret_cast<uint2 *>(E + (col + 3) * 8) = pk;
-                    *reinterpret_cast<uint2 *>(O + (col + 4) * 8) = pk;
+                    for (int c = 0; c < 4; ++c)
+                        v[c] = (row_ok && c < g.C) ? *reinterpret_cast<const float2 *>(sr + c * g.W + col)
+                                                   : make_float2(0.f, 0.f);
+                    __half2 h[4] = {__floats2half2_rn(v[0].x, v[1].x), __floats2half2_rn(v[2].x, v[3].x),
+                                    __floats2half2_rn(v[0].y, v[1].y), __floats2half2_rn(v[2].y, v[3].y)};
+                    const uint4 pk = *reinterpret_cast<uint4 *>(h);
+                    *reinterpret_cast<uint2 *>(E + (col + 3) * 8) = make_uint2(pk.x, pk.y);
+                    *reinterpret_cast<uint2 *>(E + (col + 4) * 8) = make_uint2(pk.z, pk.w);
+                    *reinterpret_cast<uint4 *>(O + (col + 4) * 8) = pk;
                 }
             }
             // the staging slot is refilled by a bulk copy (async proxy) after these reads
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncwarp();
-            mbar_arrive(smem_u32(&full[slot]));
+            if (lane == 0) mbar_arrive(smem_u32(&full[slot]));
             ++k_done;
         }
         if (!ok) {
@@ -365,91 +365,58 @@ stem_pool_kernel(const ConvArgs a, const StemGeom g) {
         }
     } else if (warp < ST_MMA_WARP + ST_NMMA) {
         // ---------------- MMA issuers: job j goes to MMA warp j % ST_NMMA ----------------
-        // One elected lane issues a job's 14 MMAs; the issue of one job and
-        // the barrier waits of the next overlap across the two warps.  A ring
-        // row is released once by each MMA warp, in row order, as soon as
-        // none of that warp's later jobs reads it: after its job j, the rows
-        // below the window of its next job j + 2 (all remaining rows after its
-        // last job).  The release is a commit, so it also waits for the MMAs.
+        // One elected lane issues a job's 14 MMAs and one commit, which tells
+        // both the epilogue (accumulator ready) and the producers (ring rows
+        // read) that the job is done.  The waits of one job overlap the issue
+        // of the other warp's.
         const int mw = warp - ST_MMA_WARP;
         const uint32_t id64 = idesc_f16(128, ST_K);
         const uint32_t id80 = idesc_f16(128, ST_NB);
         const uint32_t ring_base = smem_u32(ring), b_base = smem_u32(Bs);
-        // descriptors: the weights' are fixed; a ring row's is the ring base
-        // descriptor plus the row's offset in 16-byte units (the start
+        // descriptors: base plus an offset in 16-byte units (the start
         // address field of a no-swizzle descriptor is addr >> 4)
-        uint64_t bd[ST_KSTEPS];
-#pragma unroll
-        for (int t = 0; t < ST_KSTEPS; ++t) bd[t] = smem_desc_noswz(b_base + t * ST_B_STEP, ST_B_LBO, 128);
-        const uint64_t ad_base = smem_desc_noswz(ring_base, 16, 128);
-        // window starts of jobs j, j + 1, j + 2 (scanned ahead of the issue)
-        StemJobs scan;
-        bool scan_have = scan.first(u0, u1, g);
-        int scan_ec = 0;                       // ring entries of the jobs scanned so far
-        int ws[3];
-        bool hv[3];
-        auto scan_one = [&](int &w, bool &h) {
-            h = scan_have;
-            w = 0;
-            if (scan_have) {
-                w = scan.seg_start ? scan_ec : scan_ec - 5;
-                scan_ec += scan.seg_start ? 7 : 2;
-                scan_have = scan.next(g);
-            }
-        };
-        scan_one(ws[0], hv[0]);
-        scan_one(ws[1], hv[1]);
-        scan_one(ws[2], hv[2]);
-        int j = 0, waited = 0, rel = 0;
+        const uint64_t bd = smem_desc_noswz(b_base, ST_B_LBO, 128);
+        const uint64_t ad_base = OVL ? smem_desc_noswz(ring_base - 16, 16, 112) : smem_desc_noswz(ring_base, 16, 128);
+        StemRun rn;
+        rn.init(u0, u1);
         bool issued = false, ok = true;
-        while (hv[0]) {
-            if (j % ST_NMMA == mw) {
-                if (__any_sync(0xffffffffu, *abort_flag)) { ok = false; break; }
-                const int wstart = ws[0];
-                const int ab = j % ST_NACC;
-                const uint32_t use = (uint32_t)(j / ST_NACC) & 1u;
-                ok = warp_wait(smem_u32(&acc_empty[ab]), use ^ 1u, a.err, 8u);
-                // the rows of the window this warp has not waited for
-                for (int e = max(waited, wstart); e < wstart + ST_R && ok; ++e)
-                    ok = warp_wait(smem_u32(&full[e % ST_NSLOT]), (uint32_t)(e / ST_NSLOT) & 1u, a.err, 2u);
-                if (!ok) { if (lane == 0) *abort_flag = 1; break; }
-                waited = wstart + ST_R;
-                const int rel_end = hv[ST_NMMA] ? ws[ST_NMMA] : scan_ec;
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                if (elect_one()) {
-                    const uint32_t d = tmem + (uint32_t)(ab * 128);
-                    int slot = wstart % ST_NSLOT;
-                    uint64_t ad[ST_R];
+        for (int j = mw; rn.at_job(j, g); j += ST_NMMA) {
+            const int wstart = rn.e0 + 2 * (j - rn.j0);
+            const int ab = j % ST_NACC;
+            // the window's seven rows and the accumulator, one lane each
+            bool mine = true;
+            if (lane < ST_R)
+                mine = mbar_wait(smem_u32(&full[(wstart + lane) % ST_NSLOT]),
+                                 (uint32_t)((wstart + lane) / ST_NSLOT) & 1u, a.err, 2u);
+            else if (lane == ST_R)
+                mine = mbar_wait(smem_u32(&acc_empty[ab]), ((uint32_t)(j / ST_NACC) & 1u) ^ 1u, a.err, 8u);
+            ok = __all_sync(0xffffffffu, mine) && !__any_sync(0xffffffffu, *abort_flag);
+            if (!ok) { if (lane == 0) *abort_flag = 1; break; }
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            if (elect_one()) {
+                const uint32_t d = tmem + (uint32_t)(ab * 128);
+                int off = (wstart % ST_NSLOT) * (ST_SLOT_BYTES >> 4);
+                uint64_t ad[ST_R];
 #pragma unroll
-                    for (int r = 0; r < ST_R; ++r) {
-                        ad[r] = ad_base + (uint64_t)((slot * ST_SLOT_BYTES) >> 4);
-                        slot = slot + 1 == ST_NSLOT ? 0 : slot + 1;
-                    }
-#pragma unroll
-                    for (int i = 0; i < ST_R; ++i) {
-                        const int r = i == 0 ? 3 : (i <= 3 ? i - 1 : i);    // centre row first
-                        // the first MMA (centre row) writes all 80 columns when the
-                        // carry-through row is present
-                        umma_f16(d, ad[r], bd[2 * r], (i == 0 && g.ct) ? id80 : id64, i > 0 ? 1u : 0u);
-                        umma_f16(d, ad[r] + (uint64_t)((ST_ROW_BYTES + 32) >> 4), bd[2 * r + 1], id64, 1u);
-                    }
-                    umma_commit(smem_u32(&acc_full[ab]));
-                    for (int e = rel; e < rel_end; ++e) umma_commit(smem_u32(&empty[e % ST_NSLOT]));
+                for (int r = 0; r < ST_R; ++r) {
+                    ad[r] = ad_base + (uint64_t)off;
+                    off += ST_SLOT_BYTES >> 4;
+                    if (off == ST_NSLOT * (ST_SLOT_BYTES >> 4)) off = 0;
                 }
-                __syncwarp();
-                rel = max(rel, rel_end);
-                issued = true;
+#pragma unroll
+                for (int i = 0; i < ST_R; ++i) {
+                    const int r = i == 0 ? 3 : (i <= 3 ? i - 1 : i);    // centre row first
+                    // the first MMA (centre row) writes all 80 columns when the
+                    // carry-through row is present
+                    umma_f16(d, ad[r], bd + (uint64_t)((2 * r * ST_B_STEP) >> 4), (i == 0 && g.ct) ? id80 : id64,
+                             i > 0 ? 1u : 0u);
+                    umma_f16(d, ad[r] + (uint64_t)((ST_ROW_BYTES + 32) >> 4),
+                             bd + (uint64_t)(((2 * r + 1) * ST_B_STEP) >> 4), id64, 1u);
+                }
+                umma_commit(smem_u32(&job_done[j % ST_NJOB]));
             }
-            ws[0] = ws[1]; hv[0] = hv[1];
-            ws[1] = ws[2]; hv[1] = hv[2];
-            scan_one(ws[2], hv[2]);
-            ++j;
-        }
-        // a warp with no job after some rows (or none at all) still releases them
-        if (ok && rel < scan_ec) {
-            if (elect_one())
-                for (int e = rel; e < scan_ec; ++e) umma_commit(smem_u32(&empty[e % ST_NSLOT]));
             __syncwarp();
+            issued = true;
         }
         // every issued MMA has completed before TMEM can be freed
         if (issued) {
@@ -462,12 +429,22 @@ stem_pool_kernel(const ConvArgs a, const StemGeom g) {
         const int et = threadIdx.x - ST_EPI0;
         const int quad = warp & 3;
         const int half_id = (warp - ST_MMA_WARP - ST_NMMA) >> 2;     // channels 32 * half_id ..
-        const int q = quad * 32 + lane;                 // output column of this thread
+        // output column of this thread; OVL: columns -1 and past Q are not used
+        const int q = OVL ? 28 * quad + 7 * (lane >> 3) + (lane & 7) - 1 : quad * 32 + lane;
+        const bool in_row = q >= 0 && q < g.Q;
+        // OVL: the lane of an odd local column (28 quad + 2 t) is the centre of
+        // pooled column 14 quad + t.  Its neighbours' lanes (the last column of
+        // an 8-row group is the first of the next); a neighbour outside the row
+        // is replaced by the centre itself
+        const int cl = 7 * (lane >> 3) + (lane & 7), jp = 14 * quad + cl / 2;
+        const bool centre = (lane & 7) < 7 && (cl & 1) && jp < g.Q2;
+        const int left = q < 1 ? lane : (lane & 7) ? lane - 1 : max(lane - 2, 0);
+        const int right = q + 1 < g.Q ? min(lane + 1, 31) : lane;
         const int k0 = 32 * half_id;
         const FaultDelta fd = a.fd;
-        float bias[32];
+        float2 bias[16];
 #pragma unroll
-        for (int i = 0; i < 32; ++i) bias[i] = __ldg(a.bias + k0 + i);
+        for (int i = 0; i < 16; ++i) bias[i] = make_float2(__ldg(a.bias + k0 + 2 * i), __ldg(a.bias + k0 + 2 * i + 1));
         const bool has_cs = a.cs_out != nullptr;
         // pooling role: column jj, channels 8 cq .. 8 cq + 7 and 32 + 8 cq ..
         // 32 + 8 cq + 7 (16-byte chunks cq and cq + 4 of a 128-byte pixel):
@@ -482,24 +459,27 @@ stem_pool_kernel(const ConvArgs a, const StemGeom g) {
         // vertical max-pool state of this thread's column q, carried across
         // convolution rows: after an odd row p it holds row p (shared with
         // the next pooled row), after an even row the maximum of rows p - 1
-        // and p
+        // and p; -infinity at the start of a run
         uint32_t vs[16];
 #pragma unroll
         for (int i = 0; i < 16; ++i) vs[i] = 0xFC00FC00u;
         __half vs_cs = __ushort_as_half((unsigned short)0xFC00);
-        bool acc_valid = false, has_carry = false;
+        bool acc_valid = false;
         int n_st = 0;                                   // pooled rows written: row-buffer parity
-        StemJobs jb;
-        bool have = jb.first(u0, u1, g);
-        int j = 0;
-        while (have) {
+        StemRun jb;
+        jb.init(u0, u1);
+        for (int j = 0; jb.at_job(j, g); ++j) {
             const int ab = j % ST_NACC;
-            const uint32_t use = (uint32_t)(j / ST_NACC) & 1u;
-            bool ok = mbar_wait(smem_u32(&acc_full[ab]), use, a.err, 4u);
-            ok = __all_sync(0xffffffffu, ok) && !*abort_flag;
-            const int p = jb.p;
+            bool ok = mbar_wait(smem_u32(&job_done[j % ST_NJOB]), (uint32_t)(j / ST_NJOB) & 1u, a.err, 4u);
+            ok = __all_sync(0xffffffffu, ok);
+            const int p = jb.p0 + j - jb.j0;
             const bool close_even = (p & 1) == 0 && p == g.P - 1;
-            if (jb.seg_start) { acc_valid = false; has_carry = false; }
+            if (j == jb.j0) {
+                acc_valid = false;
+#pragma unroll
+                for (int i = 0; i < 16; ++i) vs[i] = 0xFC00FC00u;
+                vs_cs = __ushort_as_half((unsigned short)0xFC00);
+            }
             // this row completes pooled row i2 (uniform over the epilogue)
             const bool store = (p & 1) ? acc_valid : close_even;
             __half *rb = rowbuf + (size_t)(n_st & 1) * 128 * ST_PIX_H;
@@ -527,23 +507,27 @@ stem_pool_kernel(const ConvArgs a, const StemGeom g) {
                 if (!fd.active) {
                     if (a.relu) {
 #pragma unroll
-                        for (int i = 0; i < 16; ++i) u[i] = cvt_relu_h2(v[2 * i] + bias[2 * i], v[2 * i + 1] + bias[2 * i + 1]);
+                        for (int i = 0; i < 16; ++i) {
+                            const float2 o = __fadd2_rn(make_float2(v[2 * i], v[2 * i + 1]), bias[i]);
+                            u[i] = cvt_relu_h2(o.x, o.y);
+                        }
                     } else {
 #pragma unroll
                         for (int i = 0; i < 16; ++i) {
-                            __half2 hh = __floats2half2_rn(v[2 * i] + bias[2 * i], v[2 * i + 1] + bias[2 * i + 1]);
+                            const float2 o = __fadd2_rn(make_float2(v[2 * i], v[2 * i + 1]), bias[i]);
+                            __half2 hh = __floats2half2_rn(o.x, o.y);
                             u[i] = *reinterpret_cast<uint32_t *>(&hh);
                         }
                     }
                 } else {
-                    const float fsrc = q < g.Q
+                    const float fsrc = in_row
                         ? image_half(image_base(a, g, jb.n), g, fd.cin, 2 * p + fd.r - 3, 2 * q + fd.s - 3) : 0.f;
 #pragma unroll
                     for (int i = 0; i < 32; i += 2) {
                         float o[2];
 #pragma unroll
                         for (int t = 0; t < 2; ++t) {
-                            float s = v[i + t] + bias[i + t];
+                            float s = v[i + t] + (t ? bias[i / 2].y : bias[i / 2].x);
                             if (fd.kout == k0 + i + t) s += fd.dv * fsrc;
                             if (a.relu) s = relu_keep_nan(s);
                             o[t] = s;
@@ -557,31 +541,51 @@ stem_pool_kernel(const ConvArgs a, const StemGeom g) {
                 const __half u_cs = __float2half_rn(o_cs);
                 // vertical pooling in registers
                 uint32_t out[16];
-                __half out_cs = u_cs;
+                const __half out_cs = __hmax_nan(vs_cs, u_cs);
+#pragma unroll
+                for (int i = 0; i < 16; ++i) out[i] = hmax2u(vs[i], u[i]);
                 if (p & 1) {
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) { out[i] = hmax2u(vs[i], u[i]); vs[i] = u[i]; }
-                    out_cs = __hmax_nan(vs_cs, u_cs);
+                    for (int i = 0; i < 16; ++i) vs[i] = u[i];
                     vs_cs = u_cs;
                 } else {
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) { vs[i] = has_carry ? hmax2u(vs[i], u[i]) : u[i]; out[i] = vs[i]; }
-                    vs_cs = has_carry ? __hmax_nan(vs_cs, u_cs) : u_cs;
-                    out_cs = vs_cs;
+                    for (int i = 0; i < 16; ++i) vs[i] = out[i];
+                    vs_cs = out_cs;
                 }
-                if (store && q < g.Q) {
+                if (OVL && store) {
+                    const int i2 = (p & 1) ? (p - 1) / 2 : p / 2;
+                    const size_t px = ((size_t)jb.n * g.P2 + i2) * g.Q2 + jp;
+                    uint32_t h[2][8];
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) {
+                        const uint32_t l = __shfl_sync(0xffffffffu, out[i], left);
+                        const uint32_t r = __shfl_sync(0xffffffffu, out[i], right);
+                        h[i / 8][i % 8] = hmax2u(hmax2u(l, out[i]), r);
+                    }
+                    if (centre) {
+                        __half *dst = static_cast<__half *>(a.y) + px * ST_K + k0;
+                        st_global_v8(dst, h[0]);
+                        st_global_v8(dst + 16, h[1]);
+                    }
+                    if (keep_cs) {
+                        const __half l = __shfl_sync(0xffffffffu, out_cs, left), r = __shfl_sync(0xffffffffu, out_cs, right);
+                        if (centre) static_cast<__half *>(a.cs_out)[px] = __hmax_nan(__hmax_nan(l, out_cs), r);
+                    }
+                }
+                if (!OVL && store && q < g.Q) {
                     uint4 *dst = reinterpret_cast<uint4 *>(rb + q * ST_PIX_H + k0);
 #pragma unroll
                     for (int i = 0; i < 4; ++i) dst[i] = make_uint4(out[4 * i], out[4 * i + 1], out[4 * i + 2], out[4 * i + 3]);
                     if (keep_cs) cb[q] = out_cs;
                 }
             }
-            if (epi_bar_or(!ok)) {
-                if (et == 0) *abort_flag = 1;
+            if (OVL ? !ok : epi_bar_or(!ok)) {
+                if (OVL ? lane == 0 : et == 0) *abort_flag = 1;
                 break;
             }
             // ---- a completed pooled row: column max over 2jj - 1 .. 2jj + 1 ----
-            if (store) {
+            if (!OVL && store) {
                 const int i2 = (p & 1) ? (p - 1) / 2 : p / 2;
                 if (pool_data) {
                     uint32_t h[8];
@@ -613,10 +617,7 @@ stem_pool_kernel(const ConvArgs a, const StemGeom g) {
                 }
                 ++n_st;
             }
-            if (p & 1) { acc_valid = false; has_carry = true; }
-            else { acc_valid = !close_even; }
-            have = jb.next(g);
-            ++j;
+            acc_valid = (p & 1) == 0 && !close_even;
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -659,8 +660,10 @@ StemPlan *stem_plan_create(const ConvArgs &a, std::string *why) {
     __half h = __float2half_rn(a.coef);          // exact: coefficients are powers of two
     memcpy(&g.coef_h, &h, 2);
     pl->sms = device_sm_count();
-    if (cudaFuncSetAttribute(stem_pool_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ST_SMEM) !=
-        cudaSuccess) {
+    if (cudaFuncSetAttribute(stem_pool_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ST_SMEM) !=
+            cudaSuccess ||
+        cudaFuncSetAttribute(stem_pool_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ST_SMEM) !=
+            cudaSuccess) {
         cudaGetLastError();
         if (why) *why = "cannot reserve shared memory for the fused stem";
         delete pl;
@@ -676,7 +679,9 @@ cudaError_t launch_stem_pool(const ConvArgs &a, const StemPlan *pl, cudaStream_t
     g.N = a.N;
     const int units = g.N * g.P2;
     const int grid = std::min(pl->sms, units);
-    pdl_launch(stem_pool_kernel, grid, ST_THREADS, ST_SMEM, st, a, g);
+    // 16 groups of 7 columns cover 112
+    if (g.Q <= 112) pdl_launch(stem_pool_kernel<true>, grid, ST_THREADS, ST_SMEM, st, a, g);
+    else pdl_launch(stem_pool_kernel<false>, grid, ST_THREADS, ST_SMEM, st, a, g);
     return cudaGetLastError();
 }
 

@@ -94,3 +94,40 @@ def test_stem_weight_faults_match_oracle():
         # the fault is transient
         again = run(m, x)
         assert np.array_equal(again[0], g_lg) and np.array_equal(again[1], g_S)
+
+
+@pytest.mark.parametrize("C,H,W,batch", [
+    (3, 9, 4, 2),          # two output columns, one pooled
+    (1, 8, 12, 3),         # one channel, six columns; even number of rows
+    (4, 37, 60, 5),        # columns past the row in the second group of 28
+    (3, 30, 116, 2),       # 58 columns: two in the last group
+    (3, 33, 224, 11),      # 112 columns: all of the overlapped layout, runs that start inside an image
+    (3, 33, 228, 3),       # 114 columns: the row-buffer layout
+    (2, 21, 256, 40),      # its widest row
+])
+def test_image_sizes_match_oracle(C, H, W, batch):
+    Ly = synth.Layer
+    L = [Ly("conv", 0, 1, cin=C, cout=64, k=7, stride=2, pad=3, relu=True),
+         Ly("maxpool", 1, 2, k=3, stride=2, pad=1),
+         Ly("gap", 2, 3),
+         Ly("fc", 3, 4, cin=64, cout=5, final=True)]
+    wl = synth.Workload("stem", L, (C, H, W), 5, 1, "fp16", 13, "normal")
+    p = synth.make_params(L, 13)
+    m = ct().ct_build_workload(wl, p, max_batch=batch)
+    assert ct().ct_launches_per_infer(m) == len(L) - 1       # fused
+    net = oracle.build_workload(wl, params=p)
+    x = synth.make_input(wl, batch=batch)
+    sel = sorted({0, batch // 2, batch - 1})
+    # clean, the last filter's last tap (column 2 q + 3), a carry-through weight off the centre
+    for f in [None, (0, 0, 63 * C * 49 + 48, 14), (0, 0, 64 * C * 49 + 20, 14)]:
+        if f is not None:
+            ct().ct_inject(m, *f)
+        run(m, x)
+        assert ct().ct_device_error(m) == 0
+        gd, gc = ct().ct_copy_activation(m, 2, batch)
+        acts = oracle.forward(net, x[sel], None if f is None else oracle.Fault(*f), keep=True)["acts"]
+        for j, i in enumerate(sel):
+            a = acts[j][2]
+            assert np.abs(gd[i] - a[:64]).max() <= TOL["fp16"] * np.abs(a[:64]).max(), f
+            assert np.abs(gc[i] - a[64]).max() <= TOL["fp16"] * np.abs(a[64]).max(), f
+    m.close()
