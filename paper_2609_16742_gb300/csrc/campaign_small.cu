@@ -17,8 +17,9 @@
 // output, checksum plane included) for one image, and only that image's CTA
 // runs.  FC weights are never faulted and are read from global memory.
 //
-// Arithmetic: each convolution output is an FFMA chain over the K index
-// (c, r, s), then + bias, fault delta, ReLU; the carry-through channel is
+// Arithmetic: each convolution output is the sum over input channels of an
+// FFMA chain over (r, s) each (short chains: smaller rounding errors than one
+// chain over all of them), then + bias, fault delta, ReLU; the carry-through channel is
 // coef * (sum of the centre-tap input channels + incoming checksum); max-pool
 // propagates NaN; an FC neuron is a dot product over eight threads, the
 // carry-through neuron coef * (sum of data inputs + sum of checksum inputs);
@@ -92,6 +93,7 @@ __device__ __forceinline__ void conv_window(const float *in, int C, int H, int W
         constexpr int WR = (RT + 3) & ~3;
         for (int c = 0; c < C; ++c) {
             const float *src = in + (c * H + 2 * pp) * W + 2 * pq;
+            float sum[4] = {0.f, 0.f, 0.f, 0.f};         // of this channel
             float row[2][RT + 1];
             auto load = [&](float (&d)[RT + 1], const float *p) {
 #pragma unroll
@@ -114,18 +116,24 @@ __device__ __forceinline__ void conv_window(const float *in, int C, int H, int W
 #pragma unroll
                 for (int s = 0; s < RT; ++s)
 #pragma unroll
-                    for (int o = 0; o < 4; ++o) acc[o] = fmaf(row[(r + (o >> 1)) & 1][s + (o & 1)], w[s], acc[o]);
+                    for (int o = 0; o < 4; ++o) sum[o] = fmaf(row[(r + (o >> 1)) & 1][s + (o & 1)], w[s], sum[o]);
             }
+#pragma unroll
+            for (int o = 0; o < 4; ++o) acc[o] += sum[o];
         }
     } else {
-        for (int c = 0; c < C; ++c)
+        for (int c = 0; c < C; ++c) {
+            float sum[4] = {0.f, 0.f, 0.f, 0.f};
             for (int r = 0; r < R; ++r)
                 for (int s = 0; s < R; ++s) {
                     const float w = wk[(c * R + r) * w_row(R) + s];
                     const float *src = in + (c * H + 2 * pp + r) * W + 2 * pq + s;
 #pragma unroll
-                    for (int o = 0; o < 4; ++o) acc[o] = fmaf(src[(o >> 1) * W + (o & 1)], w, acc[o]);
+                    for (int o = 0; o < 4; ++o) sum[o] = fmaf(src[(o >> 1) * W + (o & 1)], w, sum[o]);
                 }
+#pragma unroll
+            for (int o = 0; o < 4; ++o) acc[o] += sum[o];
+        }
     }
 }
 
@@ -181,7 +189,7 @@ __device__ __forceinline__ void fc_layer(const float *w, const float *bias, cons
     const bool vec = (n_in & 3) == 0;
     // whole groups of eight threads stay together: the shuffles below name the full warp
     for (int j = threadIdx.x >> 3; j < ((n_out + pc + 3) & ~3); j += NT / 8) {
-        float s = 0.f;
+        float s = 0.f, cs = 0.f;
         if (j < n_out) {
             const float *wj = w + (size_t)j * n_in;
             if (vec) {
@@ -205,12 +213,18 @@ __device__ __forceinline__ void fc_layer(const float *w, const float *bias, cons
                 }
             else
                 for (int k = sub; k < n_in; k += 8) a.x += x[k];
-            for (int k = sub; k < n_cs; k += 8) s += xcs[k];
-            s += (a.x + a.y) + (a.z + a.w);
+            for (int k = sub; k < n_cs; k += 8) cs += xcs[k];
+            s = (a.x + a.y) + (a.z + a.w);
         }
 #pragma unroll
         for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (sub == 0 && j < n_out + pc) put(j, j < n_out ? s + __ldg(bias + j) : coef * s);
+        // the checksums' sum joins the data's last: it is the larger one, and
+        // every addition to it rounds at its size
+        if (j - ((threadIdx.x & 31) >> 3) + 4 > n_out) {
+#pragma unroll
+            for (int o = 4; o > 0; o >>= 1) cs += __shfl_xor_sync(0xffffffffu, cs, o);
+        }
+        if (sub == 0 && j < n_out + pc) put(j, j < n_out ? s + __ldg(bias + j) : coef * (s + cs));
     }
 }
 
