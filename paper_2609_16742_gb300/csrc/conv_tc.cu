@@ -828,6 +828,12 @@ template <int BN> struct ClTile {
     static constexpr size_t smem(int stages) {
         return 1024 + 144 + (apart(stages) ? stages * STAGE + PART : stages * STAGE > PART ? stages * STAGE : PART);
     }
+    // the most any launch takes: not the deepest ring's, whose partials share its room
+    static constexpr size_t max_smem() {
+        size_t m = 0;
+        for (int s = 1; s <= MAX_STAGES; ++s) m = smem(s) > m ? smem(s) : m;
+        return m;
+    }
 };
 
 __device__ __forceinline__ void st_cluster4(uint32_t addr, float x, float y, float z, float w) {
@@ -2287,10 +2293,10 @@ TcPlan *tc_plan_create(const ConvArgs &a, int max_batch, const void *w_dev, cons
         if (r != CUDA_SUCCESS) { if (why) *why = "weight tensor map"; delete pl; return nullptr; }
     }
     cudaError_t e = cudaFuncSetAttribute(conv_tc_cluster_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)ClTile<64>::smem(ClTile<64>::MAX_STAGES));
+                                         (int)ClTile<64>::max_smem());
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(conv_tc_cluster_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)ClTile<128>::smem(ClTile<128>::MAX_STAGES));
+                                 (int)ClTile<128>::max_smem());
     if (e != cudaSuccess) { if (why) *why = "shared memory attribute"; delete pl; return nullptr; }
     if (pl->BN == 64) {
         pl->smem = smem_bytes<64, 4, 2>();
@@ -2437,7 +2443,7 @@ const ClResident &cluster_resident() {
                 cudaLaunchConfig_t cfg = {};
                 cfg.gridDim = dim3(Z * 64);
                 cfg.blockDim = dim3(CL_THREADS);
-                cfg.dynamicSmemBytes = v ? ClTile<128>::smem(ClTile<128>::MAX_STAGES) : ClTile<64>::smem(ClTile<64>::MAX_STAGES);
+                cfg.dynamicSmemBytes = v ? ClTile<128>::max_smem() : ClTile<64>::max_smem();
                 cudaLaunchAttribute at[1];
                 at[0].id = cudaLaunchAttributeClusterDimension;
                 at[0].val.clusterDim.x = Z;

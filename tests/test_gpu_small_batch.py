@@ -28,6 +28,14 @@ def test_few_tiles_match_oracle(C, K, k, stride, H, batch):
     check(wl, p, batch, sorted({0, batch - 1}))
 
 
+@pytest.mark.parametrize("K", [64, 128, 256])
+def test_every_ring_depth_matches_oracle(K):
+    for C in range(64, 1025, 64):       # 1 to 16 K blocks: every share a CTA can have
+        wl, p, _ = net_of(C, K, 1, 1, 4, prec="fp16")
+        for batch in (1, 9):
+            check(wl, p, batch, [batch - 1])
+
+
 @pytest.mark.parametrize("C,H,batch", [(64, 9, 1), (256, 6, 2)])
 def test_residual_block_matches_oracle(C, H, batch):
     wl, p, _ = net_of(C, 128, 1, 1, H, residual=True, prec="fp16")
