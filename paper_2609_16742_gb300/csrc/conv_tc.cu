@@ -794,11 +794,17 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__
 // that read their peers' memory instead paid a remote round trip per eight
 // channels: the 128-channel tiles ran 20-30 us.)
 //
+// GEN: any input and output channels that are multiples of 8 (MobileNet's 16
+// to 1280).  The last K block of a tap may reach past C: its columns arrive as
+// zeros in both operands (the im2col copy's channel bound; the filters through
+// a 3-D map [K][taps][C], so that a block never reads the next tap's
+// weights, which a fault may have made infinite).  Filters past K arrive as
+// zeros and their columns are dropped.
+//
 // These layers are bound by latency: a launch, two or three copy round trips,
 // the exchange.  Splitting over a workspace with a reduction kernel per layer
 // took 12-20 us a layer on one ResNet-18/224 image (conv 7-11, reduction
-// 4-9).  Two CTAs fit an SM.  A 1x1 shortcut of the same input can share the
-// launch: clusters n1 .. run its tiles, on the centre-tap K blocks.
+// 4-9).
 //
 // The copy latency (about 1.5 us) bounds the K loop of these short tiles: with
 // three stages a K block took 0.46 us, so the ring takes up to six stages of
@@ -843,7 +849,7 @@ __device__ __forceinline__ void st_cluster1(uint32_t addr, float x) {
     asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(x) : "memory");
 }
 
-template <int BN>
+template <int BN, bool GEN = false>
 __global__ void __launch_bounds__(CL_THREADS, 1)
 conv_tc_cluster_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ CUtensorMap bmap,
                        const __grid_constant__ ConvArgs a, const __grid_constant__ TcGeom g, int nst) {
@@ -905,8 +911,9 @@ conv_tc_cluster_kernel(const __grid_constant__ CUtensorMap amap, const __grid_co
                 const int kb = kb_lo + it, s = it % nst;
                 const uint32_t fb = smem_u32(&full[s]);
                 mbar_arrive_expect_tx(fb, A_BYTES + T::B_BYTES);
-                tma_load_2d(smem_u32(smem + s * T::STAGE + A_BYTES), &bmap, fb,
-                            tap_of(kb / g.cpb, g.ctr_tap) * g.C + (kb % g.cpb) * BK, n0);
+                const int tap = tap_of(kb / g.cpb, g.ctr_tap), c0 = (kb % g.cpb) * BK;
+                if (GEN) tma_load_3d(smem_u32(smem + s * T::STAGE + A_BYTES), &bmap, fb, c0, tap, n0);
+                else tma_load_2d(smem_u32(smem + s * T::STAGE + A_BYTES), &bmap, fb, tap * g.C + c0, n0);
             };
             const bool early = a.weights_stable != 0;
             if (early)
@@ -998,17 +1005,18 @@ conv_tc_cluster_kernel(const __grid_constant__ CUtensorMap amap, const __grid_co
     constexpr int U = 2;                                  // items (8 channels of a row) in flight per thread
     uint4 rs[U];
     float4 b0[U], b1[U];
+    const int ch = GEN ? min(BN, g.K - n0) / 8 : BN / 8;  // items of a row
     auto load_items = [&](int e0) {
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const int e = min(e0 + u * CL_THREADS, r_n * (BN / 8) - 1);
-            const int m = m0 + r_lo + e / (BN / 8), k0 = n0 + (e % (BN / 8)) * 8;
+            const int e = min(e0 + u * CL_THREADS, r_n * ch - 1);
+            const int m = m0 + r_lo + e / ch, k0 = n0 + (e % ch) * 8;
             b0[u] = __ldg(reinterpret_cast<const float4 *>(a.bias + k0));
             b1[u] = __ldg(reinterpret_cast<const float4 *>(a.bias + k0 + 4));
             rs[u] = res ? __ldg(reinterpret_cast<const uint4 *>(res + (size_t)m * g.K + k0)) : make_uint4(0u, 0u, 0u, 0u);
         }
     };
-    if ((int)threadIdx.x < r_n * (BN / 8)) load_items(threadIdx.x);
+    if ((int)threadIdx.x < r_n * ch) load_items(threadIdx.x);
     cluster_wait();                                       // the partials of this CTA's rows are here
     if (warp == CL_MMA_WARP) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -1026,13 +1034,13 @@ conv_tc_cluster_kernel(const __grid_constant__ CUtensorMap amap, const __grid_co
             if (fd.cin < g.C) return ldh(x, pix * g.C + fd.cin);
             return a.cs_in ? ldh(static_cast<const __half *>(a.cs_in), pix) : 0.f;
         };
-        for (int e0 = threadIdx.x; e0 < r_n * (BN / 8); e0 += U * CL_THREADS) {
+        for (int e0 = threadIdx.x; e0 < r_n * ch; e0 += U * CL_THREADS) {
             if (e0 != (int)threadIdx.x) load_items(e0);
 #pragma unroll
             for (int u = 0; u < U; ++u) {
                 const int e = e0 + u * CL_THREADS;
-                if (e >= r_n * (BN / 8)) break;
-                const int r = e / (BN / 8), c = (e % (BN / 8)) * 8, m = m0 + r_lo + r, k0 = n0 + c;
+                if (e >= r_n * ch) break;
+                const int r = e / ch, c = (e % ch) * 8, m = m0 + r_lo + r, k0 = n0 + c;
                 float v[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
 #pragma unroll
                 for (int z = 0; z < CL_MAX_Z; ++z)
@@ -2436,6 +2444,15 @@ struct ClResident {
 const ClResident &cluster_resident() {
     static const ClResident r = [] {
         ClResident t;
+        // the query reports 0 for more shared memory than a kernel has opted in to
+        bool opt = true;
+        for (auto kern : {conv_tc_cluster_kernel<64>, conv_tc_cluster_kernel<64, true>})
+            opt = opt && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                              (int)ClTile<64>::max_smem()) == cudaSuccess;
+        for (auto kern : {conv_tc_cluster_kernel<128>, conv_tc_cluster_kernel<128, true>})
+            opt = opt && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                              (int)ClTile<128>::max_smem()) == cudaSuccess;
+        if (!opt) cudaGetLastError();
         for (int v = 0; v < 2; ++v)
             for (int Z = 0; Z <= CL_MAX_Z; ++Z) {
                 t.n[v][Z] = 0;
@@ -2464,11 +2481,11 @@ const ClResident &cluster_resident() {
 ClPick cluster_pick(int m_tiles, int K, int n_kb) {
     const ClResident &res = cluster_resident();
     ClPick best{0, 0, 1e30};
-    for (int BN = 64; BN <= 128 && BN <= K; BN *= 2)
+    for (int BN = 64; BN == 64 || (BN == 128 && K > 64); BN *= 2)
         for (int Z = 1; Z <= CL_MAX_Z && Z <= n_kb; ++Z) {
             const int kps = (n_kb + Z - 1) / Z;
             if (Z > 1 && (Z - 1) * kps >= n_kb) continue;        // an empty share
-            const long long cls = (long long)m_tiles * (K / BN), fit = res.n[BN == 128][Z];
+            const long long cls = (long long)m_tiles * ((K + BN - 1) / BN), fit = res.n[BN == 128][Z];
             if (fit < 1) continue;
             const double rounds = (double)((cls + fit - 1) / fit);
             const double us = 3.0 + 0.15 * Z + rounds * (2.5 + kps * (BN == 64 ? KB_US_64 : KB_US_128));
@@ -2541,6 +2558,8 @@ cudaError_t launch_conv_tc(const ConvArgs &a, const void *plan, cudaStream_t st,
                                pl->bmap128, a, g, nst);
         return cudaGetLastError();
     }
+    // N = 256 tiles have no persistent kernel on single CTAs
+    if (!pairs && pl->BN == 256) return cudaErrorNotSupported;
     const int tiles = g.m_tiles * g.n_tiles;
     // a 1x1 shortcut of the same input (a2, plan2) joins this launch when the
     // tiles allow; the caller launches it on its own otherwise
@@ -2621,6 +2640,79 @@ cudaError_t launch_conv_tc(const ConvArgs &a, const void *plan, cudaStream_t st,
     const cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess && merged) *merged = sc;
     return e;
+}
+
+// Layers outside tc_supported whose channels are multiples of 8 (16-byte rows
+// for the copies): one tile per cluster of conv_tc_cluster_kernel<.., true>.
+// conv_simt.cu ran these before; here a block that is mostly padding costs one
+// stage.  MobileNet-V2 in FP16, 32 x 32: one image 789 -> 274 us, 128 images
+// 2,202 -> 1,001 us (32 x 32 x 144 to 24 channels 48 us, 24 to 144 60 us, of
+// 44 MB each), the error against 64 bits unchanged.  Bound by a tile's latency:
+// copy, MMA, exchange and stores of a CTA are in series, two or three CTAs on
+// an SM overlap them.
+bool tc_general_supported(int C, int K, int R, int S, int stride, int pad) {
+    return C % 8 == 0 && K % 8 == 0 && R == S && R <= 7 && stride >= 1 && stride <= 2 && pad <= 3 && pad <= R / 2 + 1;
+}
+
+TcPlan *tc_general_plan_create(const ConvArgs &a, int max_batch, const void *w_dev, const void *x_dev) {
+    if (!load_encoders()) return nullptr;
+    TcPlan *pl = new TcPlan();
+    memset(pl, 0, sizeof(*pl));
+    pl->sms = sm_count();
+    TcGeom &g = pl->g;
+    g.PQ = a.P * a.Q; g.Q = a.Q; g.stride = a.stride; g.pad = a.pad; g.C = a.C; g.K = a.K;
+    g.RSC = a.R * a.S * a.C; g.S = a.S;
+    g.cpb = (a.C + BK - 1) / BK;
+    g.n_kb = a.R * a.S * g.cpb;
+    g.ctr_tap = ((a.R - 1) / 2) * a.S + (a.S - 1) / 2;
+    g.ct_mode = a.role == CT_ROLE_CT ? CT_COLUMN : CT_NONE_;
+    g.coef_h = coef_half_bits(a.coef);
+    cuuint64_t gdim[4] = {(cuuint64_t)a.C, (cuuint64_t)a.W, (cuuint64_t)a.H, (cuuint64_t)max_batch};
+    cuuint64_t gstr[3] = {(cuuint64_t)a.C * 2, (cuuint64_t)a.W * a.C * 2, (cuuint64_t)a.H * a.W * a.C * 2};
+    int lower[2] = {-a.pad, -a.pad};
+    int upper[2] = {a.pad - (a.S - 1), a.pad - (a.R - 1)};
+    cuuint32_t estr[4] = {1, (cuuint32_t)a.stride, (cuuint32_t)a.stride, 1};
+    bool ok = g_encode_im2col(&pl->amap, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 4, const_cast<void *>(x_dev), gdim, gstr, lower,
+                              upper, BK, BM, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                              CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    cuuint64_t bdim[3] = {(cuuint64_t)a.C, (cuuint64_t)(a.R * a.S), (cuuint64_t)a.K};
+    cuuint64_t bstr[2] = {(cuuint64_t)a.C * 2, (cuuint64_t)g.RSC * 2};
+    for (int rows : {64, 128}) {
+        cuuint32_t box[3] = {BK, 1, (cuuint32_t)rows}, bes[3] = {1, 1, 1};
+        ok = ok && g_encode_tiled(rows == 64 ? &pl->bmap64 : &pl->bmap128, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3,
+                                  const_cast<void *>(w_dev), bdim, bstr, box, bes, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                                  CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    }
+    ok = ok && cudaFuncSetAttribute(conv_tc_cluster_kernel<64, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)ClTile<64>::max_smem()) == cudaSuccess &&
+         cudaFuncSetAttribute(conv_tc_cluster_kernel<128, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)ClTile<128>::max_smem()) == cudaSuccess;
+    if (!ok || cluster_pick(1, g.K, g.n_kb).Z == 0) {
+        cudaGetLastError();
+        delete pl;
+        return nullptr;
+    }
+    return pl;
+}
+
+cudaError_t launch_conv_tc_general(const ConvArgs &a, const TcPlan *pl, cudaStream_t st) {
+    TcGeom g = pl->g;
+    g.M = a.N * a.P * a.Q;
+    g.m_tiles = (g.M + BM - 1) / BM;
+    const ClPick cl = cluster_pick(g.m_tiles, g.K, g.n_kb);
+    g.splits = cl.Z;
+    g.kps = (g.n_kb + cl.Z - 1) / cl.Z;
+    g.n_tiles = (g.K + cl.BN - 1) / cl.BN;
+    const dim3 grid(g.m_tiles * g.n_tiles * cl.Z);
+    const int nst = std::min(g.kps, cl.BN == 64 ? ClTile<64>::MAX_STAGES : ClTile<128>::MAX_STAGES);
+    if (cl.BN == 64)
+        pdl_launch_cluster(conv_tc_cluster_kernel<64, true>, grid, CL_THREADS, ClTile<64>::smem(nst), st, cl.Z, pl->amap,
+                           pl->bmap64, a, g, nst);
+    else
+        pdl_launch_cluster(conv_tc_cluster_kernel<128, true>, grid, CL_THREADS, ClTile<128>::smem(nst), st, cl.Z, pl->amap,
+                           pl->bmap128, a, g, nst);
+    return cudaGetLastError();
 }
 
 bool tc_small_supported(int C, int K, int R, int S, int stride, int pad) {

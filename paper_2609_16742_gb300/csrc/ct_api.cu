@@ -93,6 +93,7 @@ struct LayerRT {
     float *bias = nullptr;
     bool tc = false;
     TcPlan *plan = nullptr;
+    TcPlan *gplan = nullptr;     // FP16, channels multiples of 8 that the plan above does not take
     FfmaPlan *fplan = nullptr;   // FP32, input channels a multiple of 4: packed FFMA
     HaloPlan *hplan = nullptr;   // stride-1 3x3 layers: halo tiles when the batch fills the GPU
     bool tc_small = false;       // first layer with <= 4 input channels on the tensor cores
@@ -214,6 +215,7 @@ ct_status dalloc(ct_model *m, void **p, size_t bytes) {
 void free_all(ct_model *m) {
     for (auto &l : m->L) {
         if (l.plan) tc_plan_destroy(l.plan);
+        if (l.gplan) tc_plan_destroy(l.gplan);
         if (l.splan) tc_small_plan_destroy(l.splan);
         if (l.stplan) stem_plan_destroy(l.stplan);
         if (l.hplan) halo_plan_destroy(l.hplan);
@@ -696,6 +698,14 @@ ct_status build_impl(ct_model *m, const ct_model_desc *desc, const float *const 
             l.fplan = ffma_plan_create(a, B, l.w, m->slots[l.d.src].data);   // null: conv_simt runs the layer
             continue;
         }
+        if (l.d.op == CT_OP_CONV && prec == CT_FP16 && !l.tc && !l.dw && !(m->flags & CT_FLAG_SIMT_ONLY) &&
+            tc_general_supported(l.C, l.K, l.R, l.S, l.d.stride, l.d.pad) && m->slots[l.d.src].cp == l.C) {
+            ConvArgs a{};
+            a.N = B; a.H = l.H; a.W = l.W; a.C = l.C; a.K = l.K; a.R = l.R; a.S = l.S;
+            a.stride = l.d.stride; a.pad = l.d.pad; a.P = l.P; a.Q = l.Q; a.role = l.role; a.coef = l.coef;
+            l.gplan = tc_general_plan_create(a, B, l.w, m->slots[l.d.src].data);
+            continue;
+        }
         if (!l.tc) continue;
         ConvArgs a{};
         a.N = B; a.H = l.H; a.W = l.W; a.C = l.C; a.K = l.K; a.R = l.R; a.S = l.S;
@@ -1036,6 +1046,8 @@ ct_status infer_impl(ct_model *m, const float *input, int batch, float *logits, 
                     sc_done = i + 1;
                 } else if (l.tc) {
                     CUDA_TRY(launch(m, FAM_TC, flops, st, [&] { return launch_conv_tc(a, l.plan, st, &nk); }, &nk));
+                } else if (l.gplan) {
+                    CUDA_TRY(launch(m, FAM_TC, flops, st, [&] { return launch_conv_tc_general(a, l.gplan, st); }));
                 } else if (l.fplan) {
                     CUDA_TRY(launch(m, FAM_SIMT, flops, st, [&] { return launch_conv_ffma(a, l.fplan, st); }));
                 } else {

@@ -251,6 +251,10 @@ struct TcPlan;
 TcPlan *tc_plan_create(const ConvArgs &shape_args, int max_batch, const void *w_dev, const void *x_dev,
                        std::string *why);
 void tc_plan_destroy(TcPlan *p);
+// FP16 layers outside tc_supported with channels that are multiples of 8; null: conv_simt runs the layer
+bool tc_general_supported(int C, int K, int R, int S, int stride, int pad);
+TcPlan *tc_general_plan_create(const ConvArgs &shape_args, int max_batch, const void *w_dev, const void *x_dev);
+cudaError_t launch_conv_tc_general(const ConvArgs &a, const TcPlan *p, cudaStream_t st);
 bool tc_supported(int C, int K, int R, int S, int stride, int pad, std::string *why);
 
 // tensor-core conv for first layers with at most 4 input channels (input

@@ -95,3 +95,30 @@ def test_repeated_inferences_give_the_same_bits(batch):
         assert torch.equal(lg, ref[0]) and torch.equal(S, ref[1])
     assert ct().ct_device_error(m) == 0
     m.close()
+
+
+@pytest.mark.parametrize("C,K,k,stride,H,batch", [
+    (16, 96, 1, 1, 32, 2),      # a quarter of a K block
+    (24, 144, 1, 1, 9, 3),      # second filter tile of 16, 243 pixels
+    (96, 24, 1, 1, 16, 5),      # second K block half empty, 24 of 64 filters
+    (40, 72, 3, 2, 13, 2),      # nine taps of 40 channels
+    (200, 328, 3, 1, 7, 1),     # 36 K blocks, the last of each tap 8 channels wide
+    (960, 320, 1, 1, 4, 40),
+    (8, 8, 1, 1, 5, 1),         # the smallest
+    (128, 192, 1, 2, 10, 7),    # whole K blocks, filters not a power of two
+])
+def test_channels_that_do_not_fill_blocks_match_oracle(C, K, k, stride, H, batch):
+    wl, p, _ = net_of(C, K, k, stride, H, prec="fp16")
+    check(wl, p, batch, sorted({0, batch - 1}))
+
+
+def test_faults_in_partial_blocks_match_oracle():
+    C, K, batch = 24, 40, 2
+    wl, p, _ = net_of(C, K, 3, 1, 10, residual=True, prec="fp16")
+    Ct = C + 1
+    last = len(wl.layers) - 3
+    # bit 14 of a weight near 1/16 is large; of one in [1, 2) infinite
+    for f in [(0, last, (5 * Ct + 3) * 9 + 4, 13), (0, last, (39 * Ct + 23) * 9 + 8, 14), (0, last, (9 * Ct + C) * 9 + 4, 13),
+              (0, last, (K * Ct + 2) * 9 + 4, 13), (0, last, (K * Ct + C) * 9 + 0, 12), (1, last, 3 * 100 + 5, 13),
+              (1, last, C * 100 + 7, 13)]:
+        check(wl, p, batch, [0, batch - 1], f)
