@@ -454,7 +454,7 @@ def main():
     else:
         clock = pk.get("sm_max_mhz", 2070.0) * 1e6
         peak = props.multi_processor_count * 128 * 2 * clock / 1e12
-        roof = {"kernel": "conv_simt_kernel (FFMA)", "bound": "alu",
+        roof = {"kernel": "FP32 convolution family: conv_ffma2, conv_image3, conv_simt (FFMA)", "bound": "alu",
                 "achieved": si_fl / (si_ms / 1e3) / 1e12 if si_ms else 0.0,
                 "peak": peak, "unit": "TFLOP/s",
                 "peak_source": "%d SMs x 128 FFMA/clk x 2 flop x %.0f MHz (%s max SM clock)"

@@ -26,10 +26,9 @@
 // the verdict is NOT(|S - r| <= tau).
 //
 // What bounds it: latency at small batches, issue slots in the campaign.
-// LeNet-5: one to 64 images 36.5 -> 9.3 us (the host needs 8.6 us for a
-// call), 1,024 images 199 -> 48 us, 2,048 faults on 8 images 1.9 -> 0.30 ms,
-// against one conv output per thread with the unpooled tensors in shared
-// memory and a warp per FC neuron.
+// LeNet-5: one to 64 images 36.4 -> 9.6-9.8 us (the host needs 8.6 us for a
+// call), 2,048 faults on 8 images 1.88 -> 0.32 ms, against one conv output per
+// thread with the unpooled tensors in shared memory and a warp per FC neuron.
 // A convolution and its pool are one step: a task is one pooled output, whose
 // thread computes the window's four convolution outputs from two rolling
 // input rows in registers (four FFMAs per weight read), so the unpooled

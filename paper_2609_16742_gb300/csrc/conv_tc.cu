@@ -36,15 +36,16 @@
 // bytes every SM copies and reads per step.  Its epilogue sums the
 // carry-through column from the centre-tap input pixel.
 //
-// Layers with few tiles split K over a cluster (conv_tc_cluster_kernel).
+// Layers with few tiles split K over a cluster (conv_tc_cluster_kernel), which
+// also takes the channel counts that the other kernels do not.
 //
 // Warp roles.  conv_tc_kernel: producer warps (each owning whole ring slots),
 // one MMA warp (one elected lane issues tcgen05.mma), eight epilogue warps;
 // conv_tc_pair_kernel: three producer warps, each owning two ring slots (with
 // two, the copy issue held the 7 x 7 layers back by 8%, measured), the MMA
 // warp (issuing in the even CTA only), eight epilogue warps.
-// conv_tc_halo_kernel (320 threads): warp 0 issues TMA, warp 1 the MMAs,
-// warps 2-9 the epilogue.  Each TMEM lane quadrant (32 output pixels) is
+// conv_tc_halo_kernel (352 threads): warp 0 issues TMA, warps 1 and 10 the
+// MMAs of alternate tiles, warps 2-9 the epilogue.  Each TMEM lane quadrant (32 output pixels) is
 // read by two epilogue warps, each taking half of the tile's channels.
 // Every mbarrier wait is bounded; on expiry the kernel records an error code
 // in a device word, stops issuing work and exits after releasing TMEM.

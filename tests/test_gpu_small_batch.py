@@ -122,3 +122,15 @@ def test_faults_in_partial_blocks_match_oracle():
               (0, last, (K * Ct + 2) * 9 + 4, 13), (0, last, (K * Ct + C) * 9 + 0, 12), (1, last, 3 * 100 + 5, 13),
               (1, last, C * 100 + 7, 13)]:
         check(wl, p, batch, [0, batch - 1], f)
+
+
+@pytest.mark.parametrize("cin,K,H,batch", [(1, 4, 9, 3), (2, 36, 16, 1), (3, 32, 32, 9), (4, 128, 7, 5)])
+def test_image_layers_match_oracle(cin, K, H, batch):
+    Ly = synth.Layer
+    L = [Ly("conv", 0, 1, cin=cin, cout=K, k=3, stride=1, pad=1, relu=True),
+         Ly("gap", 1, 2),
+         Ly("fc", 2, 3, cin=K, cout=10, final=True)]
+    wl = synth.Workload("image", L, (cin, H, H), 10, 1, "fp16", 7, "normal")
+    p = synth.make_params(L, 7)
+    for f in [None, (0, 0, (K - 1) * cin * 9 + 8, 14), (0, 0, K * cin * 9 + 3, 14), (1, 0, H + 1, 13)]:
+        check(wl, p, batch, sorted({0, batch - 1}), f)
